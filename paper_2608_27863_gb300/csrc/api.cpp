@@ -244,6 +244,13 @@ int create_device(hdg_ctx* h) {
     size_t budget = (size_t)8 << 30;
     if (const char* s = std::getenv("HDG_SCRATCH_BYTES")) budget = std::strtoull(s, nullptr, 10);
     h->chunk = std::max<int64_t>(1, std::min<int64_t>(h->E, (int64_t)(budget / per)));
+    // FP64 elimination before any tuning call: panels of 8 columns (the pivot chain works on half the
+    // rows' words of a 16-wide one; 1-15 % faster on every element type), and the Schur product on the
+    // tensor cores from n_u = 40 on.  Elimination + Schur product, in ms, FP64 pipe / tensor cores:
+    // 2867 quads p = 1 0.33 / 0.53, p = 2 1.56 / 1.76, p = 3 (n_u = 64) 4.3 / 3.7; 693 hexes p = 1
+    // (n_u = 40) 1.29 / 0.85; 512 hexes p = 2 17.0 / 10.3; 210 hexes p = 3 69.4 / 37.0
+    h->elim_nb = 8;
+    h->schur64_mode = h->NU >= 40 ? 1 : 0;
     if (const char* s = std::getenv("HDG_ELIM_MINB")) h->elim_minb = std::atoi(s) == 1 ? 1 : 2;
     if ((rc = dev_alloc(h, &h->d_vcoef, (size_t)h->chunk * h->m * h->m * d * h->NCOEF * h->Nq))) return rc;
     if ((rc = dev_alloc(h, &h->d_fcoef, (size_t)h->chunk * h->nf * h->m * h->m * h->NCOEF * h->Nfq))) return rc;

@@ -200,7 +200,8 @@ struct hdg_ctx {
                                            // 2 FP32 sum factorisation
     int blocks64_mode = 1;                 // FP64 volume contraction: 0 dense GEMM, 1 sum factorisation
     int schur64_mode = 0;                  // FP64 Schur product: 0 inside the FP64 elimination, 1 on the BF16
-                                           // tensor cores by exact digit splitting (k_schur_ozaki)
+                                           // tensor cores by exact digit splitting (k_schur_ozaki); the
+                                           // default is set with the device storage
     double* d_m11 = nullptr;               // [E][NU][NU] interior block / its LU factors (FP64)
     float* d_m12 = nullptr;                // [E][NU][NT] Bt, then Z = L^{-1} P Bt
     double* d_mrt = nullptr;               // [E][NU] Rt, then z
@@ -213,7 +214,7 @@ struct hdg_ctx {
     int64_t chunk = 0;
     bool have_system = false;
     int elim_minb = 2;                     // k_elim variant: resident CTAs per SM the kernel is built for
-    int elim_nb = 16;                      // k_elim variant: panel width (16 or 8)
+    int elim_nb = 16;                      // k_elim variant: panel width (16 or 8; default set with the device storage)
     int elim_mixed_minb = 2;               // k_elim_mixed variant: resident CTAs per SM (2 or 3)
     int elim_mixed_split = 0;              // mixed elimination: 0 fused kernel, 1 FP64 LU + FP32 triangular solves
 

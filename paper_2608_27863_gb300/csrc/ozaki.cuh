@@ -10,18 +10,20 @@
 // by integer operations on its FP64 bits, into s digits of b bits:
 //     W_rk ~ 2^{e_r} sum_i 2^{-b i} a_i,   Z_kc ~ 2^{f_c} sum_j 2^{-b j} z_j,
 // with integer digits |a_i|, |z_j| < 2^b carrying the value's sign (truncation
-// error below 2^{-b s} of the row / column scale; b s >= 54).  A digit times
+// error below 2^{-b s} of the row / column scale; b s >= 60).  A digit times
 // a power of two is exact in BF16 (8 significant bits, b <= 8).  The integer
 // products A_i Z_j (K = n_u terms) are exact in the FP32 accumulator as long
 // as every partial sum stays below 2^24: with b chosen so that
-// 5 n_u (2^b - 1)^2 < 2^24, the pairs of each digit-sum group k = i + j <= 6
-// accumulate exactly into their own accumulator.  Pairs with k >= 7, whose
-// weight is 2^{-5b} or less relative to the leading group, share one
-// accumulator; pairs with k > s + 1 are dropped (below the truncation error).
+// (N - 1) n_u (2^b - 1)^2 < 2^24, the pairs of each digit-sum group k = i + j <= N
+// accumulate exactly into their own accumulator (N = 6 for b = 8, else 8: all 512
+// tensor-memory columns).  Pairs with k > N share the last accumulator, whose FP32
+// truncation is 2^{-24} of a sum that weighs 2^{-b (N - 1)} of the leading group;
+// pairs with k > s + 1 are dropped (below the truncation error).
 // Slices are staged pre-scaled by 2^{-b (i - 3)} and 2^{-b (j - 4)}, so every
 // accumulator holds 2^{-b (k - 7)} G_k (G_k = sum over i + j = k of A_i Z_j)
-// and the six accumulators sum to 2^{7b} 2^{-e_r - f_c} (W Z)_rc; the epilogue
-// adds them in FP64, scales and subtracts from Dt in FP64.
+// and the accumulators sum to 2^{7b} 2^{-e_r - f_c} (W Z)_rc; the epilogue
+// adds them in 128-bit integer arithmetic, converts once, scales and subtracts from
+// Dt in FP64.
 //
 // k_oz_scales first computes every row's and column's exponent once per element.
 // Then one CTA (16 warps) per (element, 128-row tile, 64-column tile) walks K in
@@ -32,8 +34,8 @@
 // the canonical K-major layout without swizzle (8-row x 16-byte core matrices,
 // K-adjacent cores 128 B apart, 8-row groups 512 B apart), and one thread
 // issues tcgen05.mma kind::f16 (BF16 inputs, FP32 accumulation in tensor
-// memory) for every kept digit pair.  The epilogue combines the six
-// accumulators exactly as 64-bit integers and converts once to FP64.  Waits on the MMA completion barrier are
+// memory) for every kept digit pair.  The epilogue combines the
+// accumulators as integers and converts once to FP64.  Waits on the MMA completion barrier are
 // bounded; on timeout the CTA latches status bit 4, waits once more (bounded)
 // and frees its tensor memory.
 #pragma once
@@ -53,13 +55,15 @@ constexpr int OZ_THREADS = 512;
 template <class C>
 struct OzakiCfg {
     static constexpr int K = C::NU, NT = C::NT;
-    // digit width: 5 K (2^b - 1)^2 < 2^24 keeps the groups k <= 6 exact
-    static constexpr int B = (5LL * K * 255 * 255 < (1LL << 24)) ? 8 : (5LL * K * 127 * 127 < (1LL << 24)) ? 7 : 6;
-    static constexpr int S = (54 + B - 1) / B;            // digits: b s >= 54
-    static constexpr int NACC = 6;                        // groups 2 .. 6 and the rest
+    // digit width: (NACC - 1) K (2^b - 1)^2 < 2^24 keeps the groups k <= NACC exact; at b = 8 the shared
+    // accumulator starts 2^{-40} below the leading group, so its FP32 truncation is far below FP64's and
+    // five exact groups are enough
+    static constexpr int B = (5LL * K * 255 * 255 < (1LL << 24)) ? 8 : (7LL * K * 127 * 127 < (1LL << 24)) ? 7 : 6;
+    static constexpr int S = (60 + B - 1) / B;            // digits: b s >= 60
+    static constexpr int NACC = B == 8 ? 6 : 8;           // groups 2 .. NACC and the rest
     static constexpr int MT = 128, NTN = 64, KC = 32;
     static constexpr int NMT = (NT + MT - 1) / MT, NNT = (NT + NTN - 1) / NTN;
-    static constexpr int TCOLS = 512;                     // NACC * NTN = 384 columns allocated as 512
+    static constexpr int TCOLS = 512;                     // NACC * NTN = 384 or 512 columns
     static constexpr int A_SLICE = MT * KC * 2, B_SLICE = NTN * KC * 2;   // bytes of one digit slice
     static constexpr int WRS = KC + 2;                    // raw W tile row (doubles): the TMA box is 2 wider than
                                                           // the chunk, which also makes the rows conflict-free
@@ -68,19 +72,20 @@ struct OzakiCfg {
     static constexpr int LOAD_BYTES = RAW;                // bytes one chunk's two TMA loads deliver
     static constexpr int SMEM = S * (A_SLICE + B_SLICE) + RAW + (MT + NTN) * 4 + 64 + 16;
     static_assert((S * (A_SLICE + B_SLICE)) % 128 == 0 && (MT * WRS * 8) % 128 == 0, "TMA destinations 128-B aligned");
-    static_assert(S <= 9 && B * S >= 54 && B * S <= 56, "digit layout");
+    static_assert(S <= 10 && B * S >= 60 && B * S <= 64, "digit layout");
     static_assert(NACC * NTN <= TCOLS, "tensor-memory columns");
-    static_assert((5LL * K * ((1 << B) - 1) * ((1 << B) - 1)) < (1LL << 24), "exact FP32 group accumulation");
+    static_assert(((NACC - 1LL) * K * ((1 << B) - 1) * ((1 << B) - 1)) < (1LL << 24), "exact FP32 group accumulation");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// exponent e with |v| < 2^e for a normal FP64 value with bits u; zero / subnormal -> INT_MIN
+// exponent e with |v| < 2^e for a normal FP64 value with bits u; zero / subnormal -> INT_MIN, infinity and
+// NaN -> 1025 (one above the largest finite value's)
 __device__ __forceinline__ int oz_exponent(unsigned long long u) {
     const int E = (int)((u >> 52) & 0x7FF);
     return E == 0 ? INT_MIN : E - 1022;
 }
 
-// trunc(|v| 2^{BS - e}) as an integer (< 2^BS <= 2^56) from the FP64 bits u of v
+// trunc(|v| 2^{BS - e}) as an integer (< 2^BS <= 2^64) from the FP64 bits u of v
 // (|v| < 2^e); zero or subnormal -> 0
 __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long u, int e, int BS) {
     const int E = (int)((u >> 52) & 0x7FF);
@@ -300,7 +305,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_schur_ozaki(double* top, doub
                 for (int j = 0; j < S; ++j) {
                     const int k = i + j + 2;                    // digit-sum group (digits counted from 1)
                     if (k > S + 1) continue;
-                    const int g = k <= 6 ? k - 2 : 5;
+                    const int g = k <= O::NACC ? k - 2 : O::NACC - 1;
                     for (int st = 0; st < nsteps; ++st) {
                         const uint32_t off = st * 256;          // 16 K values = two K-adjacent core matrices
                         const uint64_t da = umma_desc(smem_u32(As + i * O::A_SLICE) + off, 128, (KC / 8) * 128);
@@ -329,14 +334,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_schur_ozaki(double* top, doub
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
         // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (tile rows) and the 16-column
-        // quarter w / 4 of the tile; the six accumulators are combined exactly as integers in
-        // units of 2^{5b - 38} (the leading group needs at most 62 bits), converted once to FP64,
-        // scaled by 2^{e_r + f_c - 2b - 38} and subtracted from Dt
+        // quarter w / 4 of the tile; the accumulators are combined as two integers per output, hi
+        // (groups k <= 6, exact, units of 2^{5b - 38}: the leading group needs at most 62 bits) and
+        // lo (the groups below, units of 2^{-38})
         const int lg = warp & 3, c0 = (warp >> 2) * 16;
         const int r = lg * 32 + lane, row = m0 + r;
-        long long tot[16];
+        long long hi[16], lo[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) tot[j] = 0ll;
+        for (int j = 0; j < 16; ++j) { hi[j] = 0ll; lo[j] = 0ll; }
 #pragma unroll 1
         for (int g = 0; g < O::NACC; ++g) {
             uint32_t v[16];
@@ -348,9 +353,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_schur_ozaki(double* top, doub
                          : "r"(addr));
             asm volatile("tcgen05.wait::ld.sync.aligned;");
             // accumulator g holds a group only if some kept digit pair falls in it
-            if (g < 5 ? (g + 2 <= S + 1) : (S + 1 >= 7)) {
+            if (g + 2 > S + 1) continue;
+            if (g < 5) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) tot[j] += oz_acc_fixed(v[j], 38 - 5 * B);
+                for (int j = 0; j < 16; ++j) hi[j] += oz_acc_fixed(v[j], 38 - 5 * B);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) lo[j] += oz_acc_fixed(v[j], 38);
             }
         }
         if (row < NT) {
@@ -358,9 +367,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_schur_ozaki(double* top, doub
             for (int j = 0; j < 16; ++j) {
                 const int c = n0 + c0 + j;
                 if (c < NT) {
-                    const int sc = er[r] + fc[c0 + j] - 2 * B - 38;
-                    const double x = __ll2double_rn(tot[j]);
                     double* sp = Bm + (size_t)row * LD + NU + c;
+                    if (er[r] > 1024 || fc[c0 + j] > 1024) {   // an infinity or NaN in the row or column
+                        *sp = __longlong_as_double(0x7FF8000000000000ll);
+                        continue;
+                    }
+                    // hi 2^{5b} + lo, shifted left as far as 64 bits hold it, converted once to FP64
+                    const long long th = hi[j] + (lo[j] >> (5 * B));
+                    const unsigned long long tl = (unsigned long long)lo[j] & ((1ull << (5 * B)) - 1);
+                    const int up = min(__clzll(th ^ (th >> 63)) - 1, 5 * B);
+                    const double x = __ll2double_rn((long long)(((unsigned long long)th << up) | (tl >> (5 * B - up))));
+                    const int sc = er[r] + fc[c0 + j] - 2 * B - 38 - up;
                     if (sc > -1023 && sc < 1024)               // 2^sc as a normal double, from its bits
                         *sp -= x * __longlong_as_double((long long)(1023 + sc) << 52);
                     else

@@ -56,3 +56,41 @@ def test_tensor_core_schur_against_fp64_pipe(nb, record_property):
 def test_config2_full_size_sampled_tensor_core_schur():
     P = synth.config2()
     compare(P, rows=sampled_rows(P, 23, 12), tuning=OZ)
+
+
+@pytest.mark.parametrize("make,oz", [(lambda: synth.tiny(2, 1), False), (synth.config1, False),
+                                     (lambda: synth.tiny(2, 3), True), (lambda: synth.tiny(3, 1), True),
+                                     (lambda: synth.config2(n=3), True), (lambda: synth.config3(n=3), True)],
+                         ids=["quad-p1", "quad-p2", "quad-p3", "hex-p1", "hex-p2", "hex-p3"])
+def test_default_variant_and_its_agreement_with_the_fp64_pipe(make, oz):
+    """A fresh handle is bitwise the variant its sizes select; both Schur products agree to 64-bit rounding."""
+    from paper_2608_27863_gb300 import hdg as H
+    P = make()
+    fresh = GpuRun(P).linearize()
+    run = GpuRun(P)
+    got = {}
+    for mode in (0, 3):
+        H.hdg_set_tuning(run.h, elim_nb=8, schur_mode=mode)
+        got[mode] = run.linearize().blocks()
+    assert np.array_equal(fresh.blocks(), got[3 if oz else 0])
+    # both products differ from the exact one by rounding in K <= 320 terms of |W| |Z|, which is below the block
+    # scale here: 320 2^-53 = 3.6e-14
+    assert np.linalg.norm(got[3] - got[0]) <= 4e-14 * np.linalg.norm(got[0])
+    fresh.close()
+    run.close()
+
+
+def test_non_finite_input_stays_visible_in_the_blocks():
+    """A NaN on one face reaches every block that the FP64 pipe makes non-finite."""
+    from paper_2608_27863_gb300 import hdg as H
+    P = synth.config2(n=3)
+    run = GpuRun(P)
+    run.UH[5, 0, 0] = float("nan")
+    bad = {}
+    for mode in (0, 3):
+        H.hdg_set_tuning(run.h, elim_nb=8, schur_mode=mode)
+        v = run.linearize().blocks()
+        assert H.hdg_status(run.h) != 0
+        bad[mode] = ~np.isfinite(v).all(axis=(1, 2))
+    assert bad[0].any() and not (bad[0] & ~bad[3]).any()
+    run.close()
