@@ -24,9 +24,6 @@ static_assert(sizeof(TetElem) % 8 == 0, "descriptor copied as 64-bit words");
 
 constexpr int NPT = NQMAX + 4 * NFQMAX;   // volume + face points
 constexpr int NCM = NPMAX + 4 * NFPMAX;   // columns of one component: U nodes + trace nodes
-constexpr int KC = 40;                    // contraction: points staged per step
-constexpr int SRP = 36;                   // staged row-basis stride (NPMAX rounded up to 4)
-constexpr int STP = 96;                   // staged column stride (NCM rounded up to 4)
 constexpr int NB = 16;                    // largest elimination panel width (shared-memory sizing)
 constexpr int NRMAX = M * NPMAX + 4 * M * NFPMAX;
 
@@ -44,8 +41,10 @@ constexpr int64_t W_RV = W_CB + 4 * NFQMAX * 125;        // [NQMAX][a][r]
 constexpr int64_t W_RF = W_RV + NQMAX * 15;              // [4 NFQMAX][a]
 constexpr int64_t W_RB = W_RF + 4 * NFQMAX * M;          // [4 NFQMAX][a]
 constexpr int64_t W_MM = W_RB + 4 * NFQMAX * M;          // [NPMAX][NPMAX] mass matrix, then its Cholesky factor
-constexpr int64_t W_DP = W_MM + NPMAX * NPMAX;           // [NQMAX][3][NPMAX] physical gradients
-constexpr int64_t W_VQ = W_DP + NQMAX * 3 * NPMAX;       // [3][NPT][NCM] psi | chi
+constexpr int64_t W_DP = W_MM + NPMAX * NPMAX;           // [NQMAX][3][NPMAX] physical gradients, then (FP64 form)
+                                                         // the modal lifting operators [3][Np][Nc]
+constexpr int64_t W_VQ = W_DP + NQMAX * 3 * NPMAX;       // mixed form: [3][NPT][NCM] psi | chi; FP64 form: the face,
+                                                         // then the volume coupling matrices of the contraction
 constexpr int64_t W_GHF = W_VQ + 3LL * NPT * NCM;       // mixed form: FP32 copies of G | H
 constexpr int64_t W_END = W_GHF + (3LL * NPMAX * NCM + 1) / 2;
 
@@ -56,13 +55,12 @@ constexpr int S_Q = S_US + M * NPMAX;                    // [3][m][Np]
 constexpr int S_QL = S_Q + 3 * M * NPMAX;                // [3][m][Np] lifted gradient
 constexpr int S_UH = S_QL + 3 * M * NPMAX;               // [t] element trace
 constexpr int S_DYN = S_UH + 4 * M * NFPMAX;             // phase scratch
-constexpr int S_GEMM = KC * (SRP + STP);
 constexpr int S_ELIM = NRMAX * NB + NB * TCW;
-constexpr int S_TOTAL = S_DYN + (S_GEMM > S_ELIM ? S_GEMM : S_ELIM);
+constexpr int S_TOTAL = S_DYN + S_ELIM;
 
 struct KArgs {
     const TetElem* el; const int32_t* order; int64_t E; int32_t* next;
-    const double* tab; const float* tabf; const double* gvol; const double* gface;
+    const double* tab; const float* tabf; const double* gvol; const double* gface; const int32_t* fnod;
     const double* U; const double* Q; const double* UH; const double* Ustar;
     double* mat; double* rec; double* work; int64_t wstride;
     PhysT<double> ph; PhysT<float> phf;                  // phf: Jacobian terms of the mixed form
@@ -108,21 +106,6 @@ __device__ __forceinline__ int bcol(const TetElem& d, int b, int c) {
     return d.NU + d.toff[f] + b * d.nfp[f] + r;
 }
 
-// one out[i][c] += sum_k R[k][i] T[k][c] pass over a staged chunk; 4 x 4 register tiles
-template <class T>
-__device__ __forceinline__ void gemm_chunk(const T* sR, const T* sT, int kc, int ti, int tc, T acc[4][4]) {
-    for (int k = 0; k < kc; ++k) {
-        T rv[4], tv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { rv[u] = sR[k * SRP + 4 * ti + u]; tv[u] = sT[k * STP + 4 * tc + u]; }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = fma(rv[u], tv[v], acc[u][v]);
-    }
-}
-
-
 // A0: gather the element's nodal state and trace into shared memory
 __device__ void gather_element(const KArgs& A, const TetElem& d, double* sm) {
     const int tid = threadIdx.x, NU = d.NU, t = d.t;
@@ -165,6 +148,343 @@ __device__ void load_geometry(const KArgs& A, const TetElem& d, double* gv, doub
 }
 
 // ---------------------------------------------------------------------------
+// FP64 form: the contraction A2.
+//
+// The q variation of a unit column c is -sum_j phi_j GH_k[j][c] (GH = [G | H]), a
+// polynomial of the element space, so the viscous part of a block factors into
+// matrices that do not know the columns, times the lifting operators:
+//   C_ab[i][c] = K0_ab[i][c] - sum_k sum_j Kk_ab[i][j] GH_k[j][c],
+//   Kk_ab[i][j] = sum_g (sum_r dphi_r[g][i] o_abrk[g]) phi_j[g]       (k = 0: the basis column itself)
+// and the sum over the collapsed volume points factors once more, one axis at a
+// time, with phi_j = sum_m psi_m Vinv[m][j], psi_ijk = A_i(a) B_ij(b) C_ijk(c):
+// per row 36 x 30 + 36 x 15 + 6 x 35 multiply-adds at p = 4 instead of 216 x 35.
+// The face terms are the same with the trace basis as rows,
+//   F_ab[l][c] = sum_s mu_l (...) ,
+// of which only the n_tri(p) element nodes on the face couple to the state, and the
+// element rows of a face are dt times its flux rows seen from the nodes (the
+// restriction of phi_i to the face lies in the trace space).  Row a = 0 has no
+// viscous part, nor does dF_momentum / dE: 8 of the 25 pairs stop at K0.
+// One p = 4 element with degree-4 faces: 21e6 multiply-adds for 78e6 of the product
+// of every row basis with every column at every point, which this replaced; the
+// 3,600-element launch (tet p = 1..4, curved) fell from 288 to 124 ms.  Every phase
+// runs over a flat list of (pair, tile) items, so that low degrees fill the CTA too.
+constexpr int NVIS = 17;                       // component pairs with a viscous part
+constexpr int NKM = M * M + 3 * NVIS;          // volume matrices: K0 of every pair, K1..3 of the viscous ones
+constexpr int NKF = M * M + M + 3 * NVIS;      // face matrices: uhat of every pair, tau u on the diagonal, q 1..3
+static_assert((int64_t)NKM * NPMAX * NPMAX <= 3LL * NPT * NCM && 4LL * NKF * NFPMAX * NFPMAX <= 3LL * NPT * NCM,
+              "coupling matrices fit the workspace");
+static_assert(3 * NPMAX * NCM <= NQMAX * 3 * NPMAX, "modal lifting operators fit the workspace");
+
+// component pair of position q in the list of pairs, the viscous ones first
+__device__ __forceinline__ void pair_of(int q, int& a, int& b) {
+    if (q < 12) { a = 1 + (q >> 2); b = q & 3; }
+    else if (q < NVIS) { a = M - 1; b = q - 12; }
+    else if (q < NVIS + M) { a = 0; b = q - NVIS; }
+    else { a = q - NVIS - M + 1; b = M - 1; }
+}
+
+// volume matrices in the modal basis, KM[matrix][m][i]: matrix q < 25 is K0 of pair q,
+// 25 + 3 q + k - 1 is Kk; one (matrix, i) per thread and step, st = the 1-D factors
+template <int P>
+__device__ __noinline__ void contract_volume(const double* __restrict__ dphi, const double* __restrict__ cv,
+                                             const double* st, double* __restrict__ KM) {
+    constexpr int N1 = P + 1, Q = P + 2, NT2 = (P + 1) * (P + 2) / 2, NP = (P + 1) * (P + 2) * (P + 3) / 6;
+    constexpr int NQ = Q * Q * Q;
+    const double* TA = st;
+    const double* TB = TA + Q * N1;
+    const double* TC = TB + Q * NT2;
+    for (int item = threadIdx.x; item < NKM * NP; item += NTH) {
+        const int mat = item / NP, i = item - mat * NP;
+        const int q = mat < M * M ? mat : (mat - M * M) / 3, kind = mat < M * M ? 0 : (mat - M * M) % 3 + 1;
+        int a, b;
+        pair_of(q, a, b);
+        const double* o = cv + (a * 3 * M + b) * 4 + kind;
+        const double* dp = dphi + i;
+        double v[NP];
+#pragma unroll
+        for (int m = 0; m < NP; ++m) v[m] = 0.0;
+#pragma unroll 1
+        for (int gc = 0; gc < Q; ++gc) {
+            double u[NT2];
+#pragma unroll
+            for (int m = 0; m < NT2; ++m) u[m] = 0.0;
+#pragma unroll 1
+            for (int gb = 0; gb < Q; ++gb) {
+                const int g0 = (gc * Q + gb) * Q;
+                double t[N1];
+#pragma unroll
+                for (int m = 0; m < N1; ++m) t[m] = 0.0;
+#pragma unroll
+                for (int ga = 0; ga < Q; ++ga) {
+                    const int g = g0 + ga;
+                    const double* og = o + (size_t)g * 300;
+                    const double x = dp[g * NP] * og[0] + dp[(NQ + g) * NP] * og[M * 4] +
+                                     dp[(2 * NQ + g) * NP] * og[2 * M * 4];
+#pragma unroll
+                    for (int m = 0; m < N1; ++m) t[m] = fma(TA[ga * N1 + m], x, t[m]);
+                }
+                int ij = 0;
+#pragma unroll
+                for (int m = 0; m < N1; ++m)
+#pragma unroll
+                    for (int j = 0; j < N1 - m; ++j, ++ij) u[ij] = fma(TB[gb * NT2 + ij], t[m], u[ij]);
+            }
+            int ij = 0, ijk = 0;
+#pragma unroll
+            for (int m = 0; m < N1; ++m)
+#pragma unroll
+                for (int j = 0; j < N1 - m; ++j, ++ij)
+#pragma unroll
+                    for (int k = 0; k < N1 - m - j; ++k, ++ijk) v[ijk] = fma(TC[gc * NP + ijk], u[ij], v[ijk]);
+        }
+        double* out = KM + (size_t)mat * NP * NP + i;
+#pragma unroll
+        for (int m = 0; m < NP; ++m) out[m * NP] = v[m];
+    }
+}
+
+// face matrices KF[face][matrix][j][l] (strides NFPMAX): matrix q < 25 couples uhat node j of the
+// face in pair q, 25 + a the element's node j on the face through tau (a = b), 30 + 3 q + k - 1 that
+// node's q_k
+__device__ __noinline__ void contract_faces(const TetElem& d, const double* __restrict__ tab,
+                                            const double* __restrict__ cf, double* __restrict__ KF) {
+    const int nP = (d.p + 1) * (d.p + 2) / 2;
+    for (int f = 0; f < 4; ++f) {
+        const int nfp = d.nfp[f], nfq = d.nfq[f];
+        const double* mu = tab + d.ttab[f];
+        const double* ph = tab + d.ctab[f];
+        const double* co = cf + (size_t)d.soff[f] * 125;
+        for (int item = threadIdx.x; item < NKF * nfp; item += NTH) {
+            const int mat = item / nfp, l = item - mat * nfp;
+            int a, b, kind;
+            if (mat < M * M) { pair_of(mat, a, b); kind = 1; }
+            else if (mat < M * M + M) { a = b = mat - M * M; kind = 0; }
+            else { pair_of((mat - M * M - M) / 3, a, b); kind = 2 + (mat - M * M - M) % 3; }
+            const double* ch = kind == 1 ? mu : ph;
+            const int n = kind == 1 ? nfp : nP;
+            const double* o = co + (a * M + b) * 5 + kind;
+            double acc[NFPMAX];
+#pragma unroll
+            for (int j = 0; j < NFPMAX; ++j) acc[j] = 0.0;
+            for (int s = 0; s < nfq; ++s) {
+                const double w = mu[s * nfp + l] * o[(size_t)s * 125];
+#pragma unroll
+                for (int j = 0; j < NFPMAX; ++j)
+                    if (j < n) acc[j] = fma(w, ch[s * n + j], acc[j]);
+            }
+            double* out = KF + ((size_t)(f * NKF + mat) * NFPMAX) * NFPMAX + l;
+#pragma unroll
+            for (int j = 0; j < NFPMAX; ++j)
+                if (j < n) out[j * NFPMAX] = acc[j];
+        }
+    }
+}
+
+// the flux rows of every face into the trace rows of the bordered matrix, tiles of 5 rows x 4 columns
+__device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& d, const int* fpo,
+                                                 const double* __restrict__ Gk, const double* __restrict__ Hk,
+                                                 const double* __restrict__ KF, double* __restrict__ Mx) {
+    const int Np = d.Np, sfp = d.t / M, Nc = Np + sfp, nct = (Nc + 3) / 4, nP = (d.p + 1) * (d.p + 2) / 2;
+    int tiles[5];
+    tiles[0] = 0;
+    for (int f = 0; f < 4; ++f) tiles[f + 1] = tiles[f] + M * M * ((d.nfp[f] + 4) / 5) * nct;
+    for (int item = threadIdx.x; item < tiles[4]; item += NTH) {
+        int f = 0;
+        while (item >= tiles[f + 1]) ++f;
+        const int nfp = d.nfp[f], ntl = (nfp + 4) / 5, per = ntl * nct;
+        const int loc = item - tiles[f], q = loc / per, rem = loc - q * per, l0 = 5 * (rem / nct), c0 = 4 * (rem % nct);
+        int a, b;
+        pair_of(q, a, b);
+        const int32_t* fn = A.fnod + ((size_t)d.p * NCODE + d.code[f]) * FNOD;
+        const double* Kf = KF + (size_t)f * NKF * NFPMAX * NFPMAX + l0;
+        double acc[5][4];
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+        if (q < NVIS) {
+            const double* gp[4];
+            int gs[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int c = min(c0 + v, Nc - 1);
+                gp[v] = c < Np ? Gk + c : Hk + (c - Np);
+                gs[v] = c < Np ? Np : sfp;
+            }
+            for (int k = 0; k < 3; ++k) {
+                const double* Kk = Kf + (size_t)(M * M + M + 3 * q + k) * NFPMAX * NFPMAX;
+#pragma unroll 2
+                for (int j = 0; j < nP; ++j) {
+                    const int row = k * Np + fn[j];
+                    double kv[5], gv[4];
+#pragma unroll
+                    for (int u = 0; u < 5; ++u) kv[u] = Kk[j * NFPMAX + u];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) gv[v] = gp[v][(size_t)row * gs[v]];
+#pragma unroll
+                    for (int u = 0; u < 5; ++u)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) acc[u][v] = fma(-kv[u], gv[v], acc[u][v]);
+                }
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int c = c0 + v;
+            if (c >= Nc) continue;
+            const int lf = c - Np - fpo[f], jp = c < Np && a == b ? fn[NFPMAX + c] : -1;
+            const int64_t col = bcol(d, b, c);
+#pragma unroll
+            for (int u = 0; u < 5; ++u) {
+                if (l0 + u >= nfp) continue;
+                double x = acc[u][v];
+                if (c >= Np && lf >= 0 && lf < nfp) x += Kf[((size_t)q * NFPMAX + lf) * NFPMAX + u];
+                if (jp >= 0) x += Kf[((size_t)(M * M + a) * NFPMAX + jp) * NFPMAX + u];
+                Mx[(int64_t)(d.NU + d.toff[f] + a * nfp + l0 + u) * d.LD + col] = x;
+            }
+        }
+    }
+}
+
+// the element rows: volume matrices times Vinv and the modal lifting operators GM[k][m][c], plus dt times
+// the flux rows of the faces a node lies on; tiles of 5 rows x 4 columns
+template <int P>
+__device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem& d,
+                                                   const double* __restrict__ Vinv, const double* __restrict__ KM,
+                                                   const double* __restrict__ GM, double* Mx) {
+    constexpr int NP = (P + 1) * (P + 2) * (P + 3) / 6, NTI = (NP + 4) / 5;
+    const int sfp = d.t / M, Nc = NP + sfp, nct = (Nc + 3) / 4;
+    for (int item = threadIdx.x; item < M * M * NTI * nct; item += NTH) {
+        const int q = item / (NTI * nct), rem = item - q * NTI * nct, i0 = 5 * (rem / nct), c0 = 4 * (rem % nct);
+        int a, b;
+        pair_of(q, a, b);
+        int iu[5], cc[4];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) iu[u] = min(i0 + u, NP - 1);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) cc[v] = min(c0 + v, Nc - 1);
+        double acc[5][4];
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+        if (c0 < NP) {
+            const double* K0 = KM + (size_t)q * NP * NP;
+#pragma unroll 2
+            for (int m = 0; m < NP; ++m) {
+                double kv[5], gv[4];
+#pragma unroll
+                for (int u = 0; u < 5; ++u) kv[u] = K0[m * NP + iu[u]];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) gv[v] = cc[v] < NP ? Vinv[m * NP + cc[v]] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 5; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v] = fma(kv[u], gv[v], acc[u][v]);
+            }
+        }
+        if (q < NVIS) {
+            const double* Kk = KM + (size_t)(M * M + 3 * q) * NP * NP;
+#pragma unroll 2
+            for (int m = 0; m < 3 * NP; ++m) {          // K1, K2, K3 follow each other, and so do GM_1..3
+                double kv[5], gv[4];
+#pragma unroll
+                for (int u = 0; u < 5; ++u) kv[u] = Kk[m * NP + iu[u]];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) gv[v] = GM[m * Nc + cc[v]];
+#pragma unroll
+                for (int u = 0; u < 5; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v] = fma(-kv[u], gv[v], acc[u][v]);
+            }
+        }
+        int64_t col[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) col[v] = bcol(d, b, cc[v]);
+        for (int f = 0; f < 4; ++f) {
+            const int32_t* fi = A.fnod + ((size_t)P * NCODE + d.code[f]) * FNOD + NFPMAX;
+            const double* row0 = Mx + (int64_t)(d.NU + d.toff[f] + a * d.nfp[f]) * d.LD;
+            const double* Pr = A.tab + d.ctab[f] + (size_t)d.nfq[f] * ((P + 1) * (P + 2) / 2);
+#pragma unroll
+            for (int u = 0; u < 5; ++u) {
+                const int jp = fi[iu[u]];
+                if (jp < 0) continue;
+                if (d.pf[f] == P) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v] = fma(A.dt, row0[(int64_t)jp * d.LD + col[v]], acc[u][v]);
+                } else {
+                    for (int l = 0; l < d.nfp[f]; ++l) {
+                        const double w = A.dt * Pr[l * ((P + 1) * (P + 2) / 2) + jp];
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) acc[u][v] = fma(w, row0[(int64_t)l * d.LD + col[v]], acc[u][v]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (i0 + u < NP && c0 + v < Nc) Mx[(int64_t)(a * NP + i0 + u) * d.LD + col[v]] = acc[u][v];
+    }
+}
+
+// trace rows of boundary faces that are not flux rows: the algebraic forms' face mass couplings
+// (kind 0: the interior state, kind 1: uhat of the same face)
+__device__ __noinline__ void contract_boundary_rows(const KArgs& A, const TetElem& d, const int* fpo,
+                                                    const double* __restrict__ cb, double* __restrict__ Mx) {
+    const int Np = d.Np, Nc = Np + d.t / M;
+    for (int f = 0; f < 4; ++f) {
+        if (d.tag[f] == 0) continue;
+        const int nfp = d.nfp[f], nfq = d.nfq[f];
+        const double* mu = A.tab + d.ttab[f];
+        const double* phf = A.tab + d.ftab[f];
+        for (int item = threadIdx.x; item < M * M * nfp * Nc; item += NTH) {
+            const int ab = item / (nfp * Nc), rem = item - ab * nfp * Nc, l = rem / Nc, c = rem - l * Nc;
+            const int a = ab / M, b = ab - a * M;
+            if (boundary_row_is_flux<M>(d.tag[f], a)) continue;
+            const int lf = c - Np - fpo[f];
+            const double* ch = c < Np ? phf + c : mu + lf;
+            const int cs = c < Np ? Np : nfp;
+            const double* o = cb + (size_t)d.soff[f] * 125 + ab * 5 + (c < Np ? 0 : 1);
+            double s = 0.0;
+            if (c < Np || (lf >= 0 && lf < nfp))
+                for (int g = 0; g < nfq; ++g) s = fma(mu[g * nfp + l] * o[(size_t)g * 125], ch[(size_t)g * cs], s);
+            Mx[(int64_t)(d.NU + d.toff[f] + a * nfp + l) * d.LD + bcol(d, b, c)] = s;
+        }
+    }
+}
+
+template <int P>
+__device__ void contract_fp64(const KArgs& A, const TetElem& d, const int* fpo, const double* cv, const double* cf,
+                              const double* cb, const double* Gk, const double* Hk, double* KM, double* GM,
+                              double* st, double* Mx) {
+    constexpr int NP = (P + 1) * (P + 2) * (P + 3) / 6, Q = P + 2;
+    constexpr int NFAC = Q * (P + 1) + Q * ((P + 1) * (P + 2) / 2) + Q * NP;
+    const int tid = threadIdx.x, sfp = d.t / M, Nc = NP + sfp;
+    const double* Vinv = A.tab + d.stab + NFAC;
+    for (int i = tid; i < NFAC; i += NTH) st[i] = A.tab[d.stab + i];
+    for (int idx = tid; idx < 3 * NP * Nc; idx += NTH) {         // GM_k = Vinv [G_k | H_k]
+        const int k = idx / (NP * Nc), rem = idx - k * NP * Nc, m = rem / Nc, c = rem - m * Nc;
+        const double* g = c < NP ? Gk + (size_t)k * NP * NP + c : Hk + (size_t)k * NP * sfp + (c - NP);
+        const int gs = c < NP ? NP : sfp;
+        double s = 0.0;
+#pragma unroll 5
+        for (int j = 0; j < NP; ++j) s = fma(Vinv[m * NP + j], g[(size_t)j * gs], s);
+        GM[idx] = s;
+    }
+    contract_faces(d, A.tab, cf, KM);
+    __syncthreads();
+    contract_trace_rows(A, d, fpo, Gk, Hk, KM, Mx);
+    __syncthreads();
+    contract_volume<P>(A.tab + d.vtab + (size_t)Q * Q * Q * NP, cv, st, KM);
+    __syncthreads();
+    contract_element_rows<P>(A, d, Vinv, KM, GM, Mx);
+    __syncthreads();
+    contract_boundary_rows(A, d, fpo, cb, Mx);
+}
+
+// ---------------------------------------------------------------------------
 // Mixed form: the contraction A2 on the tensor cores.
 //
 // The column operand of a component pair, T_ab[k][c] = sum_j s_j o_ab[k][j]
@@ -185,7 +505,7 @@ constexpr int TMT = 128;                      // rows per tile (tensor-memory la
 constexpr int TNP = 96;                       // columns: Nc <= 95, padded to a multiple of 16
 constexpr int TSTAGE = 2 * (TMT + TNP) * TKC; // floats per stage: A hi | B hi | A lo | B lo
 constexpr int TTCOLS = 128;                   // tensor-memory columns per CTA
-static_assert(2 * TSTAGE * (int)sizeof(float) <= (S_GEMM > S_ELIM ? S_GEMM : S_ELIM) * (int)sizeof(double),
+static_assert(2 * TSTAGE * (int)sizeof(float) <= S_ELIM * (int)sizeof(double),
               "two operand stages fit the phase scratch");
 static_assert((S_DYN * sizeof(double)) % 16 == 0, "operand stages 16-byte aligned");
 
@@ -907,42 +1227,37 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
         }
     }
     const TJ* tabJ = jtab<TJ>(A);
-    const TJ* GJ;
-    const TJ* HJ;
-    if constexpr (sizeof(TJ) == sizeof(double)) {
-        GJ = reinterpret_cast<const TJ*>(Gk);
-        HJ = reinterpret_cast<const TJ*>(Hk);
-    } else {
+    TJ* vq = reinterpret_cast<TJ*>(W + W_VQ);
+    if constexpr (sizeof(TJ) == sizeof(float)) {
         TJ* gh = reinterpret_cast<TJ*>(W + W_GHF);
         for (int i = tid; i < 3 * Np * (Np + sfp); i += NTH) gh[i] = (TJ)Gk[i];   // G and H are contiguous
-        GJ = gh;
-        HJ = gh + 3 * Np * Np;
+        const TJ* GJ = gh;
+        const TJ* HJ = gh + 3 * Np * Np;
+        __syncthreads();
+        const int nc4 = (Nc + 3) / 4;                   // four columns per thread: one basis load per 4 FMAs
+        for (int idx = tid; idx < 3 * npt * nc4; idx += NTH) {
+            const int k = idx / (npt * nc4), rem = idx - k * npt * nc4, x = rem / nc4, c0 = 4 * (rem - x * nc4);
+            const TJ* br = basis_row_t(tabJ, d, x);
+            const TJ* gp[4];
+            int st[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int c = min(c0 + u, Nc - 1);
+                if (c < Np) { gp[u] = GJ + (size_t)k * Np * Np + c; st[u] = Np; }
+                else { gp[u] = HJ + (size_t)k * Np * sfp + (c - Np); st[u] = sfp; }
+            }
+            TJ s[4] = {0, 0, 0, 0};
+            for (int j = 0; j < Np; ++j) {
+                const TJ b = br[j];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s[u] += b * gp[u][j * st[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c0 + u < Nc) vq[((size_t)k * NPT + x) * NCM + c0 + u] = s[u];
+        }
         __syncthreads();
     }
-    TJ* vq = reinterpret_cast<TJ*>(W + W_VQ);
-    const int nc4 = (Nc + 3) / 4;                       // four columns per thread: one basis load per 4 FMAs
-    for (int idx = tid; idx < 3 * npt * nc4; idx += NTH) {
-        const int k = idx / (npt * nc4), rem = idx - k * npt * nc4, x = rem / nc4, c0 = 4 * (rem - x * nc4);
-        const TJ* br = basis_row_t(tabJ, d, x);
-        const TJ* gp[4];
-        int st[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int c = min(c0 + u, Nc - 1);
-            if (c < Np) { gp[u] = GJ + (size_t)k * Np * Np + c; st[u] = Np; }
-            else { gp[u] = HJ + (size_t)k * Np * sfp + (c - Np); st[u] = sfp; }
-        }
-        TJ s[4] = {0, 0, 0, 0};
-        for (int j = 0; j < Np; ++j) {
-            const TJ b = br[j];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) s[u] += b * gp[u][j * st[u]];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (c0 + u < Nc) vq[((size_t)k * NPT + x) * NCM + c0 + u] = s[u];
-    }
-    __syncthreads();
     // A1: fluxes and their Jacobians at the points
     const PhysT<double>& P = A.ph;
     using SJ = std::conditional_t<sizeof(TJ) == sizeof(float), float, double>;   // Jacobian terms' type
@@ -1053,11 +1368,16 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
             }
             TJ* of = cf + (size_t)r * 125;
             TJ* ob = cb + (size_t)r * 125;
-            // element rows take dt * dfhat; trace rows dfhat on flux rows, the algebraic forms
+            // element rows take dt * dfhat (the FP64 form stores dfhat); trace rows dfhat on flux rows, the algebraic forms
             // otherwise (tag 1 uhat - u_b, tag 2 uhat - u, tags 3 / 4 uhat_v, and on isothermal
             // walls uhat_rhoE - uhat_rho e_w)
             auto put = [&](int a, int b, int kind, double v) {
-                of[(a * M + b) * 5 + kind] = (TJ)(A.dt * v);
+                if (sizeof(TJ) == sizeof(double)) {       // FP64 contraction: one copy, dt applied to its rows
+                    of[(a * M + b) * 5 + kind] = (TJ)v;
+                    if (tag == 0) return;
+                } else {
+                    of[(a * M + b) * 5 + kind] = (TJ)(A.dt * v);
+                }
                 double w = v;
                 if (!boundary_row_is_flux<M>(tag, a)) {
                     w = 0.0;
@@ -1133,127 +1453,14 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
         contract_tc(d, tabJ, cv, cf, cb, vq, fpo, Mx, reinterpret_cast<float*>(sD), *ts, sflag);
         __syncthreads();
     } else {
-        // A2: contraction into the bordered matrix, one (a, b) component pair at a time
-        TJ* sR = reinterpret_cast<TJ*>(sD);  // [KC][SRP] row basis
-        TJ* sT = sR + KC * SRP;              // [KC][STP] column variations times coefficients
-        const TJ* dphiJ = tabJ + d.vtab + (size_t)Nq * Np;
-        const TJ* phiJ = tabJ + d.vtab;
-        const int nrt = (Np + 3) / 4, nct = (Nc + 3) / 4;
-        const int ti = tid / nct, tc = tid - ti * nct;
-        const bool act = tid < nrt * nct;
-        const int K1 = 3 * Nq + sfq;         // element rows: volume (g, r) then face points
-        for (int ab = 0; ab < M * M; ++ab) {
-            const int a = ab / M, b = ab - a * M;
-            TJ acc[4][4] = {};
-            for (int k0 = 0; k0 < K1; k0 += KC) {
-                const int kc = min(KC, K1 - k0);
-                // operands of the chunk; four entries per thread per pass, their loads
-                // issued before any store so that they are in flight together
-                for (int base = tid; base < kc * SRP; base += 4 * NTH) {
-                    TJ vv[4];
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int idx = base + u * NTH;
-                        const int kk = idx / SRP, i = idx - kk * SRP, K = k0 + kk;
-                        TJ v = 0;
-                        if (idx < kc * SRP && i < Np) {
-                            if (K < 3 * Nq) v = dphiJ[((size_t)(K % 3) * Nq + K / 3) * Np + i];
-                            else v = basis_row_t(tabJ, d, Nq + K - 3 * Nq)[i];
-                        }
-                        vv[u] = v;
-                    }
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (base + u * NTH < kc * SRP) sR[base + u * NTH] = vv[u];
-                }
-                for (int base = tid; base < kc * STP; base += 4 * NTH) {
-                    TJ vv[4];
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int idx = base + u * NTH;
-                        const int kk = idx / STP, c = idx - kk * STP, K = k0 + kk;
-                        TJ v = 0;
-                        if (idx < kc * STP && c < Nc) {
-                            if (K < 3 * Nq) {
-                                const int g = K / 3, r = K - 3 * g;
-                                const TJ* o = cv + (size_t)g * 300 + ((a * 3 + r) * M + b) * 4;
-                                if (c < Np) v = o[0] * phiJ[(size_t)g * Np + c];
-                                for (int l = 0; l < 3; ++l) v -= o[1 + l] * vq[((size_t)l * NPT + g) * NCM + c];
-                            } else {
-                                const int rr = K - 3 * Nq, x = Nq + rr;
-                                const TJ* o = cf + (size_t)rr * 125 + (a * M + b) * 5;
-                                if (c < Np) {
-                                    v = o[0] * basis_row_t(tabJ, d, x)[c];
-                                } else {
-                                    const int f = face_of_point(d, rr);
-                                    const int l = c - Np - fpo[f];
-                                    if (l >= 0 && l < d.nfp[f])
-                                        v = o[1] * tabJ[d.ttab[f] + (size_t)(rr - d.soff[f]) * d.nfp[f] + l];
-                                }
-                                for (int l = 0; l < 3; ++l) v -= o[2 + l] * vq[((size_t)l * NPT + x) * NCM + c];
-                            }
-                        }
-                        vv[u] = v;
-                    }
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (base + u * NTH < kc * STP) sT[base + u * NTH] = vv[u];
-                }
-                __syncthreads();
-                if (act) gemm_chunk(sR, sT, kc, ti, tc, acc);
-                __syncthreads();
-            }
-            if (act)
-                for (int u = 0; u < 4; ++u) {
-                    const int i = 4 * ti + u;
-                    if (i >= Np) continue;
-                    for (int v = 0; v < 4; ++v) {
-                        const int c = 4 * tc + v;
-                        if (c >= Nc) continue;
-                        Mx[(size_t)(a * Np + i) * LD + bcol(d, b, c)] = (double)acc[u][v];   // mass term added below
-                    }
-                }
-            // trace rows (f', a, l'): K = the points of face f'
-            for (int f2 = 0; f2 < 4; ++f2) {
-                const int nfq = d.nfq[f2], nfp = d.nfp[f2];
-                const TJ* mu = tabJ + d.ttab[f2];
-                for (int idx = tid; idx < nfq * SRP; idx += NTH) {
-                    const int kk = idx / SRP, l = idx - kk * SRP;
-                    sR[idx] = l < nfp ? mu[(size_t)kk * nfp + l] : TJ(0);
-                }
-                for (int idx = tid; idx < nfq * STP; idx += NTH) {
-                    const int kk = idx / STP, c = idx - kk * STP, rr = d.soff[f2] + kk, x = Nq + rr;
-                    TJ v = 0;
-                    if (c < Nc) {
-                        const TJ* o = cb + (size_t)rr * 125 + (a * M + b) * 5;
-                        if (c < Np) {
-                            v = o[0] * basis_row_t(tabJ, d, x)[c];
-                        } else {
-                            const int l = c - Np - fpo[f2];
-                            if (l >= 0 && l < nfp) v = o[1] * mu[(size_t)kk * nfp + l];
-                        }
-                        for (int l = 0; l < 3; ++l) v -= o[2 + l] * vq[((size_t)l * NPT + x) * NCM + c];
-                    }
-                    sT[idx] = v;
-                }
-                __syncthreads();
-                const int nrt2 = (nfp + 3) / 4;
-                const int ti2 = tid / nct, tc2 = tid - ti2 * nct;
-                if (tid < nrt2 * nct) {
-                    TJ acc2[4][4] = {};
-                    gemm_chunk(sR, sT, nfq, ti2, tc2, acc2);
-                    for (int u = 0; u < 4; ++u) {
-                        const int l = 4 * ti2 + u;
-                        if (l >= nfp) continue;
-                        for (int v = 0; v < 4; ++v) {
-                            const int c = 4 * tc2 + v;
-                            if (c >= Nc) continue;
-                            Mx[(size_t)(NU + d.toff[f2] + a * nfp + l) * LD + bcol(d, b, c)] = (double)acc2[u][v];
-                        }
-                    }
-                }
-                __syncthreads();
-            }
+        // A2 on the FP64 pipe
+        double* KM = W + W_VQ;
+        double* GM = W + W_DP;
+        switch (d.p) {
+            case 1: contract_fp64<1>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
+            case 2: contract_fp64<2>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
+            case 3: contract_fp64<3>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
+            default: contract_fp64<4>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
         }
         __syncthreads();
     }
@@ -1864,6 +2071,7 @@ int create_device(hdg_ctx* h, std::string& err) {
     UP(c->d_gvol, c->gvol); UP(c->d_gface, c->gface); UP(c->d_hoff, c->hoff); UP(c->d_boff, c->boff);
     UP(c->d_rowptr, c->rowptr); UP(c->d_col, c->col); UP(c->d_cptr, c->cptr); UP(c->d_centry, c->centry);
     UP(c->d_f2e, c->f2e); UP(c->d_f2lf, c->f2lf); UP(c->d_diagb, c->diagb); UP(c->d_bjoff, c->bjoff);
+    UP(c->d_fnod, c->fnod);
 #undef UP
     if ((rc = tet_alloc(h, &c->d_mat, (size_t)c->n_mat, err))) return rc;
     if ((rc = tet_alloc(h, &c->d_rec, (size_t)c->n_rec, err))) return rc;
@@ -1935,7 +2143,7 @@ int linearize(hdg_ctx* h, const double* U, const double* Q, const double* UH, co
     Ctx* c = h->tet;
     KArgs A;
     A.el = c->d_el; A.order = c->d_order; A.E = c->E; A.next = c->d_next;
-    A.tab = c->d_tab; A.tabf = c->d_tabf; A.gvol = c->d_gvol; A.gface = c->d_gface;
+    A.tab = c->d_tab; A.tabf = c->d_tabf; A.gvol = c->d_gvol; A.gface = c->d_gface; A.fnod = c->d_fnod;
     A.U = U; A.Q = Q; A.UH = UH; A.Ustar = Ustar;
     A.mat = c->d_mat; A.rec = c->d_rec; A.work = c->d_work; A.wstride = c->work_stride;
     A.ph = phys_t<double>(h->phys); A.phf = phys_t<float>(h->phys); A.dt = dt; A.a_ii = a_ii; A.tau = h->phys.tau;
@@ -2032,7 +2240,7 @@ KArgs base_args(hdg_ctx* h, const double* U, const double* Q, const double* UH, 
     KArgs A;
     std::memset(&A, 0, sizeof(A));
     A.el = c->d_el; A.order = c->d_order; A.E = c->E; A.next = c->d_next;
-    A.tab = c->d_tab; A.tabf = c->d_tabf; A.gvol = c->d_gvol; A.gface = c->d_gface;
+    A.tab = c->d_tab; A.tabf = c->d_tabf; A.gvol = c->d_gvol; A.gface = c->d_gface; A.fnod = c->d_fnod;
     A.U = U; A.Q = Q; A.UH = UH; A.Ustar = Ustar;
     A.mat = c->d_mat; A.rec = c->d_rec; A.work = c->d_work; A.wstride = c->work_stride;
     A.ph = phys_t<double>(h->phys); A.phf = phys_t<float>(h->phys); A.dt = dt; A.a_ii = a_ii; A.tau = h->phys.tau;

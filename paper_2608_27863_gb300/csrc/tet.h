@@ -25,6 +25,7 @@ constexpr int NQMAX = 216;      // (PMAX+2)^3
 constexpr int NFPMAX = 15;      // (PMAX+1)(PMAX+2)/2
 constexpr int NFQMAX = 36;      // (PMAX+2)^2
 constexpr int NCODE = 24;       // 4 local faces x 6 orderings of their vertices
+constexpr int FNOD = NFPMAX + NPMAX;   // entries of one face's node maps
 
 inline int n_tet(int p) { return (p + 1) * (p + 2) * (p + 3) / 6; }
 inline int n_tri(int p) { return (p + 1) * (p + 2) / 2; }
@@ -38,6 +39,15 @@ void build_tri(int p, TriTab& t);
 // with face code c (= 4-face index * 6 + ordering): phif [Nfq][Np]; the
 // outward reference area normal nu [3]
 void build_face(int p, int pF, int code, std::vector<double>& phif, double nu[3]);
+// 1-D factors of the collapsed modal basis psi_ijk = A_i(a) B_ij(b) C_ijk(c) of degree p at the volume rule's
+// points, i slowest and k fastest: A [p+2][p+1], B [p+2][n_tri], C [p+2][Np], then Vinv [Np][Np] with
+// phi_j = sum_m psi_m Vinv[m][j]
+void build_sumfac(int p, std::vector<double>& t);
+// the element basis of degree p on a face of degree pF: at the face's rule points [Nfq][n_tri(p)] and at its
+// trace nodes [Nfp][n_tri(p)], the columns the nodes that lie on the face in the face's canonical order
+void build_coupling(int p, int pF, std::vector<double>& t);
+// node maps of one face code (FNOD entries)
+void build_face_nodes(int p, int code, int32_t* map);
 // local vertices (L0, L1, L2) of face code c
 void code_vertices(int code, int L[3]);
 
@@ -53,7 +63,8 @@ struct TetElem {
     int64_t goff;      // curved: volume records [Nq][10] (w |J|, J^{-1} row-major [r][k])
     int64_t gfoff;     // curved: face records [sfq][3] (w_s |J| J^{-T} nu)
     int64_t koff;      // element trace residual R_uhat^K [t] (residual evaluation)
-    int32_t vtab, ftab[4], ttab[4], pad;   // table offsets: volume, face (p, pF, code), trace (pF)
+    int32_t vtab, ftab[4], ttab[4];        // table offsets: volume, face (p, pF, code), trace (pF)
+    int32_t stab, ctab[4];                 // table offsets: sum factorisation (p), face coupling (p, pF)
     double detJ, Jinv[9];                  // affine elements
     double hinv;                           // |K|^{-1/3} (state-dependent stabilization)
 };
@@ -72,6 +83,9 @@ struct Ctx {
     std::vector<int32_t> order;            // elements by decreasing cost
     std::vector<double> tab;               // all tables
     std::vector<int32_t> vtab, ttab, ftab; // offsets: [p], [pF], [(p * 5 + pF) * 24 + code]
+    std::vector<int32_t> stab, ctab;       // offsets: [p], [p * 5 + pF]
+    std::vector<int32_t> fnod;             // [(p * 24 + code)][FNOD]: element node of each face node of degree p
+                                           // (canonical order, 15), then the face node of each element node or -1
     std::vector<double> gvol, gface;       // curved geometry records
     bool has_tag[5] = {};
     // device
@@ -79,6 +93,7 @@ struct Ctx {
     int32_t* d_order = nullptr;
     double* d_tab = nullptr;
     float* d_tabf = nullptr;               // FP32 copy of the tables (mixed-form contraction)
+    int32_t* d_fnod = nullptr;             // face node maps
     double* d_gvol = nullptr;
     double* d_gface = nullptr;
     int64_t* d_hoff = nullptr;

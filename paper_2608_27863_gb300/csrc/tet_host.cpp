@@ -226,6 +226,84 @@ void code_vertices(int code, int L[3]) {
     for (int k = 0; k < 3; ++k) L[k] = kFace[f][kPerm[s][k]];
 }
 
+// The collapsed modal basis P_i(a) ((1-b)/2)^i P_j^{2i+1}(b) ((1-c)/2)^{i+j} P_k^{2i+2j+2}(c) (orthogonal on the
+// tetrahedron): its factors over one collapsed coordinate each.
+void build_sumfac(int p, std::vector<double>& t) {
+    const int n = p + 2, Np = n_tet(p);
+    std::vector<double> a, b, c, w;
+    gauss_jacobi(n, 0, a, w);
+    gauss_jacobi(n, 1, b, w);
+    gauss_jacobi(n, 2, c, w);
+    auto fa = [](int i, double x) { return jacobi(i, 0.0, 0.0, x); };
+    auto fb = [](int i, int j, double x) { return std::pow(0.5 * (1.0 - x), i) * jacobi(j, 2.0 * i + 1.0, 0.0, x); };
+    auto fc = [](int ij, int k, double x) { return std::pow(0.5 * (1.0 - x), ij) * jacobi(k, 2.0 * ij + 2.0, 0.0, x); };
+    t.clear();
+    for (int q = 0; q < n; ++q)
+        for (int i = 0; i <= p; ++i) t.push_back(fa(i, a[q]));
+    for (int q = 0; q < n; ++q)
+        for (int i = 0; i <= p; ++i)
+            for (int j = 0; j <= p - i; ++j) t.push_back(fb(i, j, b[q]));
+    for (int q = 0; q < n; ++q)
+        for (int i = 0; i <= p; ++i)
+            for (int j = 0; j <= p - i; ++j)
+                for (int k = 0; k <= p - i - j; ++k) t.push_back(fc(i + j, k, c[q]));
+    // values at the element nodes; where a collapsed coordinate is undefined (b = 1 or c = 1) every function
+    // that depends on it carries a zero factor, so any value serves
+    const auto lat = tet_lattice(p);
+    std::vector<double> V, inv;
+    for (const auto& l : lat) {
+        const double x = -1.0 + 2.0 * l[0] / p, y = -1.0 + 2.0 * l[1] / p, z = -1.0 + 2.0 * l[2] / p;
+        const double ca = l[1] + l[2] < p ? 2.0 * (1.0 + x) / (-y - z) - 1.0 : -1.0;
+        const double cb = l[2] < p ? 2.0 * (1.0 + y) / (1.0 - z) - 1.0 : -1.0;
+        for (int i = 0; i <= p; ++i)
+            for (int j = 0; j <= p - i; ++j)
+                for (int k = 0; k <= p - i - j; ++k) V.push_back(fa(i, ca) * fb(i, j, cb) * fc(i + j, k, z));
+    }
+    invert(Np, V, inv);
+    t.insert(t.end(), inv.begin(), inv.end());
+}
+
+void build_face_nodes(int p, int code, int32_t* map) {
+    int L[3];
+    code_vertices(code, L);
+    const auto lat = tet_lattice(p);
+    const auto tri = tri_lattice(p);
+    for (int i = 0; i < FNOD; ++i) map[i] = -1;
+    for (size_t j = 0; j < tri.size(); ++j) {
+        int cnt[4] = {0, 0, 0, 0};
+        cnt[L[0]] = p - tri[j][0] - tri[j][1];
+        cnt[L[1]] = tri[j][0];
+        cnt[L[2]] = tri[j][1];
+        for (size_t n = 0; n < lat.size(); ++n)
+            if (lat[n][0] == cnt[1] && lat[n][1] == cnt[2] && lat[n][2] == cnt[3]) {
+                map[j] = (int32_t)n;
+                map[NFPMAX + n] = (int32_t)j;
+            }
+    }
+}
+
+void build_coupling(int p, int pF, std::vector<double>& t) {
+    // the restriction depends on the degrees only, so face code 0 serves: its points at the rule and at the nodes
+    int L[3];
+    int32_t map[FNOD];
+    code_vertices(0, L);
+    build_face_nodes(p, 0, map);
+    const auto Vinv = tet_vinv(p);
+    const int nP = n_tri(p);
+    TriTab tr;
+    build_tri(pF, tr);
+    t.clear();
+    auto put = [&](double m1, double m2) {
+        double x[3], phi[NPMAX];
+        for (int k = 0; k < 3; ++k)
+            x[k] = (1.0 - m1 - m2) * kV[L[0]][k] + m1 * kV[L[1]][k] + m2 * kV[L[2]][k];
+        tet_lagrange(p, Vinv, x, phi, nullptr);
+        for (int j = 0; j < nP; ++j) t.push_back(phi[map[j]]);
+    };
+    for (int q = 0; q < tr.Nfq; ++q) put(0.5 * (1.0 + tr.xs[2 * q]), 0.5 * (1.0 + tr.xs[2 * q + 1]));
+    for (const auto& l : tri_lattice(pF)) put((double)l[0] / pF, (double)l[1] / pF);
+}
+
 void build_vol(int p, VolTab& t) {
     t.p = p;
     t.Np = n_tet(p);
@@ -464,6 +542,21 @@ int create_host(hdg_ctx* h, const hdg_tet_mesh* mesh, std::string& err) {
         c->tab.insert(c->tab.end(), tt[p].mu.begin(), tt[p].mu.end());
         c->tab.insert(c->tab.end(), tt[p].ws.begin(), tt[p].ws.end());
     }
+    c->stab.assign(PMAX + 1, -1);
+    c->ctab.assign((PMAX + 1) * (PMAX + 1), -1);
+    c->fnod.assign((size_t)(PMAX + 1) * NCODE * FNOD, -1);
+    for (int p = 1; p <= PMAX; ++p) {
+        std::vector<double> t;
+        build_sumfac(p, t);
+        c->stab[p] = (int32_t)c->tab.size();
+        c->tab.insert(c->tab.end(), t.begin(), t.end());
+        for (int q = p; q <= PMAX; ++q) {
+            build_coupling(p, q, t);
+            c->ctab[p * (PMAX + 1) + q] = (int32_t)c->tab.size();
+            c->tab.insert(c->tab.end(), t.begin(), t.end());
+        }
+        for (int code = 0; code < NCODE; ++code) build_face_nodes(p, code, &c->fnod[((size_t)p * NCODE + code) * FNOD]);
+    }
     std::vector<double> fnu((size_t)(PMAX + 1) * (PMAX + 1) * NCODE * 3, 0.0);
     for (int p = 1; p <= pmax; ++p)
         for (int q = p; q <= pmax; ++q)
@@ -506,11 +599,13 @@ int create_host(hdg_ctx* h, const hdg_tet_mesh* mesh, std::string& err) {
             sfp += d.nfp[f];
             d.ftab[f] = c->ftab[((size_t)p * (PMAX + 1) + d.pf[f]) * NCODE + d.code[f]];
             d.ttab[f] = c->ttab[d.pf[f]];
+            d.ctab[f] = c->ctab[p * (PMAX + 1) + d.pf[f]];
         }
         d.t = t;
         d.sfq = sfq;
         d.LD = (d.NU + t + 1 + 1) & ~1;
         d.vtab = c->vtab[p];
+        d.stab = c->stab[p];
         d.uoff = c->uoff[e];
         d.moff = moff;
         moff += (int64_t)(d.NU + t) * d.LD;

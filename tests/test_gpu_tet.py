@@ -360,3 +360,22 @@ def test_config4_full_size_sampled():
             assert np.linalg.norm(got - ref) < TOL * np.linalg.norm(ref), e
     finally:
         H.hdg_destroy(h)
+
+
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_tet_contraction_one_degree_all_boundary_kinds(H, p):
+    """Every tile remainder of the FP64 contraction: one degree at a time, the four boundary kinds, curved elements."""
+    mesh = tm.kuhn_box((2, 1, 1), [np.linspace(0, 1, 3), np.linspace(0, .5, 2), np.linspace(0, .5, 2)],
+                       (False, False, False), tags={(0, 0): 1, (0, 1): 2, (1, 0): 3, (1, 1): 4}, degrees=p,
+                       bump=tm.wall_bump(0.05), curved_layers=1)
+    prob, pb, h, dev = setup(H, mesh, twall=0.8)
+    try:
+        H.hdg_linearize_condense(h, dev["U"], dev["Q"], dev["UH"], dev["Ustar"], None, prob.dt, prob.a_ii)
+        assert H.hdg_status(h) == H.HDG_OK
+        vals = torch.zeros(H.hdg_tet_query(h)["n_vals"], dtype=torch.float64, device="cuda")
+        H.hdg_get_blocks(h, vals)
+        torch.cuda.synchronize()
+        errs, _, _ = block_errors(H, h, pb, vals.cpu().numpy())
+        assert errs.max() < TOL, errs.max()
+    finally:
+        H.hdg_destroy(h)
