@@ -153,34 +153,28 @@ int matvec(hdg_ctx* h, const double* x, double* y) {
     return rc;
 }
 
-// Classical Gram-Schmidt with one reorthogonalisation (CGS2) of vn against
-// V_0 .. V_j: hcol[0..j] = the projection coefficients (FP64, fixed-order
-// reductions), vn orthogonalised in place.  All k dot products of a pass in one
-// launch (eight basis vectors per block row of the grid) instead of one kernel
-// pair per basis vector as modified Gram-Schmidt needs.
-void cgs2(hdg_ctx* h, const double* V, int64_t N, int j, double* vn, double* hcol, double* htmp) {
-    const int k = j + 1;
-    for (int pass = 0; pass < 2; ++pass) {
-        double* hp = pass == 0 ? hcol : htmp;
-        k_mdot_part<<<dim3(kRedBlocks, (k + 7) / 8), 256, 0, h->stream>>>(V, N, k, vn, N, h->d_mred);
-        k_mdot_final<<<(k + 3) / 4, 128, 0, h->stream>>>(h->d_mred, kRedBlocks, k, hp);
-        k_msub<<<grid_for(N), 256, 0, h->stream>>>(V, N, hp, k, vn, N);
+// Krylov basis, reduction partials and coefficients for restart length m; grows to the largest asked for
+int ensure_krylov_workspace(hdg_ctx* h, int m) {
+    if (h->gm_cap >= m) return HDG_OK;
+    const int64_t N = len_t(h);
+    int rc;
+    if ((rc = alloc(h, (void**)&h->d_V, sizeof(double) * (size_t)(m + 1) * N))) return rc;
+    if ((rc = alloc(h, (void**)&h->d_w, sizeof(double) * N))) return rc;
+    if (!h->d_red) {
+        if ((rc = alloc(h, (void**)&h->d_red, sizeof(double) * kRedBlocks))) return rc;
+        if ((rc = alloc(h, (void**)&h->d_ticket, sizeof(unsigned)))) return rc;
+        CKS(cudaMemsetAsync(h->d_ticket, 0, sizeof(unsigned), h->stream));
     }
-    k_vadd<<<1, 64, 0, h->stream>>>(hcol, htmp, k);
+    if ((rc = alloc(h, (void**)&h->d_mred, sizeof(double) * kOrthBlocks * (m + 1)))) return rc;
+    if ((rc = alloc(h, (void**)&h->d_h, sizeof(double) * 2 * (m + 2)))) return rc;
+    h->gm_cap = m;
+    return HDG_OK;
 }
 
 // workspace of the synchronisation-free solver: Krylov basis, Newton work, device scalars
 int ensure_fixed_workspace(hdg_ctx* h, int m) {
-    const int64_t N = len_t(h);
     int rc;
-    if (h->gm_cap < m) {
-        if ((rc = alloc(h, (void**)&h->d_V, sizeof(double) * (size_t)(m + 1) * N))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_w, sizeof(double) * N))) return rc;
-        if (!h->d_red && (rc = alloc(h, (void**)&h->d_red, sizeof(double) * kRedBlocks * 8))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_mred, sizeof(double) * kRedBlocks * 8 * ((m + 8) / 8)))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_h, sizeof(double) * 2 * (m + 2)))) return rc;
-        h->gm_cap = m;
-    }
+    if ((rc = ensure_krylov_workspace(h, m))) return rc;
     if (h->fx_cap < m) {
         const size_t n = 1 + (size_t)m * m + 3 * (size_t)m + 1 + (m + 1);
         if ((rc = alloc(h, (void**)&h->d_fx, sizeof(double) * n))) return rc;
@@ -226,12 +220,10 @@ int gmres_fixed_async(hdg_ctx* h, const double* b, double* x, int m, bool use_x0
         double* vn = V + (size_t)(j + 1) * N;
         if ((rc = matvec(h, vj, w))) return rc;
         if ((rc = precond_apply(h, w, vn))) return rc;
-        cgs2(h, V, N, j, vn, hc, hc + m + 2);
-        dev_dot(h, vn, vn, N, hc + j + 1, true);
+        orthogonalise(h->stream, V, N, j + 1, vn, hc, hc + m + 2, h->d_mred, h->d_ticket, Givens{hc, R, cs, sn, gv, m});
         k_scale_safe<<<grid_for(N), 256, 0, h->stream>>>(vn, hc + j + 1, vn, N);
-        k_givens_step<<<1, 1, 0, h->stream>>>(hc, j, m, R, cs, sn, gv);
     }
-    k_backsolve<<<1, 1, 0, h->stream>>>(R, gv, m, m, y);
+    k_backsolve<<<1, 32, 0, h->stream>>>(R, gv, m, m, y);
     if (!use_x0) CKS(cudaMemsetAsync(x, 0, sizeof(double) * N, h->stream));
     k_combine<<<grid_for(N), 256, 0, h->stream>>>(V, N, y, m, x, N);
     CKS(cudaGetLastError());
@@ -436,15 +428,7 @@ int hdg_gmres(hdg_handle h, const double* b, double* x, int restart, int max_ite
         return fail(h, HDG_EINVAL, "precond = 1 needs the selected preconditioner set up (hdg_blockjacobi_setup / hdg_schwarz_setup)");
     const int64_t N = len_t(h);
     int rc;
-    if (h->gm_cap < restart) {
-        // workspace grows to the largest restart length requested; kept until destroy
-        if ((rc = alloc(h, (void**)&h->d_V, sizeof(double) * (size_t)(restart + 1) * N))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_w, sizeof(double) * N))) return rc;
-        if (!h->d_red && (rc = alloc(h, (void**)&h->d_red, sizeof(double) * kRedBlocks * 8))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_mred, sizeof(double) * kRedBlocks * 8 * ((restart + 8) / 8)))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_h, sizeof(double) * 2 * (restart + 2)))) return rc;
-        h->gm_cap = restart;
-    }
+    if ((rc = ensure_krylov_workspace(h, restart))) return rc;
     double* V = h->d_V;
     double* w = h->d_w;
     double* dh = h->d_h;
@@ -487,8 +471,7 @@ int hdg_gmres(hdg_handle h, const double* b, double* x, int restart, int max_ite
             } else if ((rc = matvec(h, vj, vn))) {
                 return rc;
             }
-            cgs2(h, V, N, j, vn, dh, dh + m + 2);   // Gram-Schmidt with reorthogonalisation
-            dev_dot(h, vn, vn, N, dh + j + 1, true);
+            orthogonalise(h->stream, V, N, j + 1, vn, dh, dh + m + 2, h->d_mred, h->d_ticket, Givens{});
             k_scale_dev<<<grid_for(N), 256, 0, h->stream>>>(vn, dh + j + 1, vn, N);
             CKS(cudaMemcpyAsync(hc.data(), dh, sizeof(double) * (j + 2), cudaMemcpyDeviceToHost, h->stream));
             CKS(cudaStreamSynchronize(h->stream));

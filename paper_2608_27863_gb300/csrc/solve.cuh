@@ -379,16 +379,20 @@ constexpr int kMaxBasis = 512;   // Krylov basis vectors (restart + 1 <= 501)
 __global__ void k_dot_part(const double* x, const double* y, int64_t n, double* part);
 __global__ void k_dot_final(const double* part, int nparts, double* out, int take_sqrt);
 __global__ void k_axpy_dev(const double* coef, double sign, const double* x, double* y, int64_t n);
-__global__ void k_mdot_part(const double* V, int64_t ldv, int k, const double* w, int64_t n, double* part);
-__global__ void k_mdot_final(const double* part, int nparts, int k, double* out);
-__global__ void k_msub(const double* V, int64_t ldv, const double* coef, int k, double* w, int64_t n);
-__global__ void k_vadd(double* a, const double* b, int k);
+// Givens QR on the device: column col[0..k] of the Hessenberg matrix, R [m][m], rotations cs / sn and the
+// rotated right-hand side gv (R == NULL: no step)
+struct Givens { const double* col; double* R; double* cs; double* sn; double* gv; int m; };
+constexpr int kOrthBlocks = 152;  // one per SM
+// Classical Gram-Schmidt with one reorthogonalisation (CGS2) of w against V_0 .. V_{k-1} (length n each):
+// hcol[0..k-1] the projection coefficients, hcol[k] = ||w|| afterwards, w orthogonalised in place (not scaled).
+// htmp [k], part [k][kOrthBlocks], ticket one zeroed word.
+void orthogonalise(cudaStream_t st, const double* V, int64_t n, int k, double* w, double* hcol, double* htmp,
+                   double* part, unsigned* ticket, const Givens& G);
 __global__ void k_scale_dev(const double* x, const double* div, double* y, int64_t n);
 __global__ void k_axpby(double a, const double* x, double b, double* y, int64_t n);
 __global__ void k_combine(const double* V, int64_t ldv, const double* coef, int k, double* x, int64_t n);
 __global__ void k_sum_parts(const double* p1, int64_t n1, const double* p2, int64_t n2, double* out);
 __global__ void k_scale_safe(const double* x, const double* div, double* y, int64_t n);
-__global__ void k_givens_step(const double* hcol, int j, int m, double* R, double* cs, double* sn, double* gv);
 __global__ void k_backsolve(const double* R, const double* gv, int k, int m, double* y);
 __global__ void k_set_first(const double* beta, double* gv, int m);
 __global__ void k_hist_push(const double* norms, double* hist, int* counter, int cap);

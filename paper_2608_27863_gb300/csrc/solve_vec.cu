@@ -1,6 +1,8 @@
 // FP64 vector kernels for the trace-space Krylov solver.  Reductions use a
 // fixed grid and a fixed combination order, so results are bitwise
 // reproducible from run to run.
+#include <algorithm>
+
 #include "solve.cuh"
 
 namespace hdg {
@@ -21,85 +23,222 @@ __global__ void k_dot_part(const double* x, const double* y, int64_t n, double* 
 }
 
 // sum of part[0 .. nparts) by one warp: lane l adds parts l, l + 32, ... in
-// order, then a fixed shuffle tree (stride-8 parts for the Gram-Schmidt partials)
-__device__ __forceinline__ double warp_sum_parts(const double* part, int nparts, int stride) {
+// order, then a fixed shuffle tree
+__device__ __forceinline__ double warp_sum_parts(const double* part, int nparts) {
     const int lane = threadIdx.x & 31;
     double t = 0.0;
-    for (int b = lane; b < nparts; b += 32) t += part[(size_t)b * stride];
+    for (int b = lane; b < nparts; b += 32) t += part[b];
     for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
     return t;
 }
 
 __global__ void k_dot_final(const double* part, int nparts, double* out, int take_sqrt) {
     if (blockIdx.x == 0 && threadIdx.x < 32) {
-        const double t = warp_sum_parts(part, nparts, 1);
+        const double t = warp_sum_parts(part, nparts);
         if (threadIdx.x == 0) *out = take_sqrt ? sqrt(t) : t;
     }
 }
 
-// Partial sums of the dot products of w with vectors 8 y .. 8 y + 7 of V
-// (y = blockIdx.y; fewer in the last group), one set per block x:
-// part[y][block x][8].  All groups run in one launch.
-__global__ void k_mdot_part(const double* V, int64_t ldv, int k, const double* w, int64_t n, double* part) {
-    __shared__ double red[8][8];
-    const int j0 = 8 * blockIdx.y;
-    const int nv = min(8, k - j0);
-    double acc[8];
+// The eight sums over a warp of acc[0..7]: lane l returns the sum of acc[l >> 2].  Lanes
+// exchange halves of the set, so 9 additions replace the 40 of eight separate trees (an FP64
+// addition of a warp takes 16 cycles of an SM here, and they were most of the dot kernel's time).
+__device__ __forceinline__ double warp_sum8(const double (&acc)[8]) {
+    const int lane = threadIdx.x & 31;
+    double v4[4], v2[2], v;
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double wi = w[i];
+    for (int q = 0; q < 4; ++q)
+        v4[q] = (h16 ? acc[q + 4] : acc[q]) + __shfl_xor_sync(0xffffffffu, h16 ? acc[q] : acc[q + 4], 16);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q < nv) acc[q] = fma(V[(size_t)(j0 + q) * ldv + i], wi, acc[q]);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        double s = acc[q];
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (lane == 0) red[q][warp] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        double t = 0.0;
-        for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) t += red[threadIdx.x][w2];
-        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 8 + threadIdx.x] = t;
-    }
+    for (int q = 0; q < 2; ++q)
+        v2[q] = (h8 ? v4[q + 2] : v4[q]) + __shfl_xor_sync(0xffffffffu, h8 ? v4[q] : v4[q + 2], 8);
+    v = (h4 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, h4 ? v2[0] : v2[1], 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
 }
 
-// out[j] = sum over blocks of the partials of vector j, one warp per j < k
-__global__ void k_mdot_final(const double* part, int nparts, int k, double* out) {
-    const int j = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (j < k) {
-        const double t = warp_sum_parts(part + (size_t)(j >> 3) * nparts * 8 + (j & 7), nparts, 8);
-        if ((threadIdx.x & 31) == 0) out[j] = t;
-    }
-}
-
-// w -= sum_j coef[j] V_j (j ascending; eight basis vectors loaded ahead)
-__global__ void k_msub(const double* V, int64_t ldv, const double* coef, int k, double* w, int64_t n) {
-    __shared__ double cf[kMaxBasis];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) cf[j] = coef[j];
+// Apply the previous rotations to column j of the Hessenberg matrix, form rotation j and rotate
+// the right-hand side; R [m][m] upper triangle, cs / sn rotations, gv the rotated rhs.  Called by
+// the whole block with col[0..j+1], c[0..j) and s[0..j) staged in shared memory.
+__device__ void givens_column(double* col, const double* c, const double* s, int j, const Givens& G) {
     __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        double s = w[i];
-        int j = 0;
-        for (; j + 8 <= k; j += 8) {
-            double v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = V[(size_t)(j + q) * ldv + i];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) s = fma(-cf[j + q], v[q], s);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < j; ++i) {
+            const double t = c[i] * col[i] + s[i] * col[i + 1];
+            col[i + 1] = -s[i] * col[i] + c[i] * col[i + 1];
+            col[i] = t;
         }
-        for (; j < k; ++j) s = fma(-cf[j], V[(size_t)j * ldv + i], s);
-        w[i] = s;
+        const double h0 = col[j], h1 = col[j + 1], den = hypot(h0, h1);
+        const double cj = den > 0.0 ? h0 / den : 1.0, sj = den > 0.0 ? h1 / den : 0.0;
+        G.cs[j] = cj;
+        G.sn[j] = sj;
+        col[j] = den;
+        const double g = G.gv[j];
+        G.gv[j + 1] = -sj * g;
+        G.gv[j] = cj * g;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) G.R[(size_t)i * G.m + j] = col[i];
+}
+
+// One pass of the classical Gram-Schmidt process of w against V_0 .. V_{k-1}:
+//   MODE 0  out[j] = V_j . w
+//   MODE 1  w -= sum_j coef[j] V_j, out[j] = V_j . w (the new w), add[j] += out[j]
+//   MODE 2  w -= sum_j coef[j] V_j, *out = ||w||_2 (the new w), then the Givens step of column
+//           k - 1 when G.R is given (hcol = G.col, *out its last entry)
+// The last block to finish sums the blocks' partials in block order, so that no launch
+// follows for the sums: an orthogonalisation with its norm and Givens step is three launches
+// instead of nine, which is what sets the time of small systems (one SDIRK3 step on 64 quads,
+// 1,536 unknowns, 480 GMRES iterations in a graph: 42.3 -> 26.1 ms, with the back substitution by a
+// warp instead of a thread).  Large systems are bound by the FP64 pipe, 2 k n multiply-adds of
+// 629e9 per second (2.7e5 unknowns, k ~ 78: 34 us a pass; MODE 0 62, MODE 1 90, MODE 2 38 us).
+// Tried for MODE 0: 256 threads with four rows in flight 69 us (MODE 1 116: too few loads in
+// flight for its first part), no barrier between the groups 102 us (the warps drift over all k
+// streams).  part: [k][gridDim.x]; ticket: zero between launches.
+template <int MODE, int NTHR>
+__global__ void __launch_bounds__(NTHR) k_orth(const double* __restrict__ V, int64_t ldv, int k, double* w, int64_t n,
+                                               const double* coef, double* part, unsigned* ticket, double* out,
+                                               double* add, Givens G) {
+    constexpr int NW = NTHR / 32;
+    extern __shared__ double wsum[];                    // [k][NW] the warps' sums (MODE 0, 1)
+    __shared__ double cf[kMaxBasis];
+    __shared__ double red[NW];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nb = gridDim.x;
+    const int64_t i0 = (int64_t)blockIdx.x * NTHR + tid, step = (int64_t)nb * NTHR;
+    double nrm = 0.0;
+    if (MODE > 0) {
+        for (int j = tid; j < k; j += NTHR) cf[j] = coef[j];
+        __syncthreads();
+        for (int64_t i = i0; i < n; i += step) {
+            double s = w[i];
+            int j = 0;
+            for (; j + 8 <= k; j += 8) {
+                double v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[q] = V[(size_t)(j + q) * ldv + i];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) s = fma(-cf[j + q], v[q], s);
+            }
+            for (; j < k; ++j) s = fma(-cf[j], V[(size_t)j * ldv + i], s);
+            w[i] = s;
+            if (MODE == 2) nrm = fma(s, s, nrm);
+        }
+    }
+    if (MODE == 2) {
+        for (int off = 16; off > 0; off >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, off);
+        if (lane == 0) red[warp] = nrm;
+        __syncthreads();
+        if (tid == 0) {
+            double t = 0.0;
+            for (int q = 0; q < NW; ++q) t += red[q];
+            part[blockIdx.x] = t;
+        }
+    } else {
+        // steps of (eight vectors, RU rows per thread), the next step's values loaded before the current
+        // ones are used; a barrier per group keeps the block's warps on the same eight streams
+        constexpr int RU = NTHR > 128 ? 2 : 1;
+        const int nst = (int)((n + step * RU - 1) / (step * RU)), total = ((k + 7) / 8) * nst;
+        double cur[RU][8], cw[RU], acc[8];
+        auto load = [&](int it, double (&v)[RU][8], double (&wv)[RU]) {
+            const int j0 = 8 * (it / nst), st = it % nst;
+#pragma unroll
+            for (int r = 0; r < RU; ++r) {
+                const int64_t i = i0 + (int64_t)(st * RU + r) * step;
+                const bool in = i < n;
+                wv[r] = in ? w[i] : 0.0;                // written above by this thread
+#pragma unroll
+                for (int q = 0; q < 8; ++q) v[r][q] = in && j0 + q < k ? V[(size_t)(j0 + q) * ldv + i] : 0.0;
+            }
+        };
+        load(0, cur, cw);
+        for (int it = 0; it < total; ++it) {
+            const int j0 = 8 * (it / nst), st = it % nst;
+            double nxt[RU][8], nw[RU];
+            if (it + 1 < total) load(it + 1, nxt, nw);
+            if (st == 0) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+            }
+#pragma unroll
+            for (int r = 0; r < RU; ++r)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[q] = fma(cur[r][q], cw[r], acc[q]);
+            if (st == nst - 1) {
+                const double v = warp_sum8(acc);
+                if ((lane & 3) == 0 && j0 + (lane >> 2) < k) wsum[(j0 + (lane >> 2)) * NW + warp] = v;
+                if (NTHR > 128) __syncthreads();
+            }
+#pragma unroll
+            for (int r = 0; r < RU; ++r) {
+                cw[r] = nw[r];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) cur[r][q] = nxt[r][q];
+            }
+        }
+        __syncthreads();
+        for (int j = tid; j < k; j += NTHR) {
+            double t = 0.0;
+#pragma unroll
+            for (int q = 0; q < NW; ++q) t += wsum[j * NW + q];
+            part[(size_t)j * nb + blockIdx.x] = t;
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(ticket, 1u) == (unsigned)nb - 1u;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid == 0) *ticket = 0u;
+    if (MODE == 2) {
+        if (warp == 0) {
+            const double t = warp_sum_parts(part, nb);
+            if (lane == 0) red[0] = sqrt(t);
+        }
+        __syncthreads();
+        const double h = red[0];
+        if (tid == 0) *out = h;
+        if (G.R) {
+            __shared__ double gc[kMaxBasis], gs[kMaxBasis];
+            for (int i = tid; i < k; i += NTHR) cf[i] = G.col[i];
+            for (int i = tid; i < k - 1; i += NTHR) { gc[i] = G.cs[i]; gs[i] = G.sn[i]; }
+            if (tid == 0) cf[k] = h;
+            givens_column(cf, gc, gs, k - 1, G);
+        }
+    } else {
+        for (int j = warp; j < k; j += NW) {
+            const double t = warp_sum_parts(part + (size_t)j * nb, nb);
+            if (lane == 0) {
+                out[j] = t;
+                if (MODE == 1) add[j] += t;
+            }
+        }
     }
 }
 
-// a[i] += b[i], i < k (small vectors)
-__global__ void k_vadd(double* a, const double* b, int k) {
-    for (int i = threadIdx.x; i < k; i += blockDim.x) a[i] += b[i];
+void orthogonalise(cudaStream_t st, const double* V, int64_t n, int k, double* w, double* hcol, double* htmp,
+                   double* part, unsigned* ticket, const Givens& G) {
+    // one block per SM; narrow blocks while they alone do not reach every SM
+    const Givens none{};
+    if (n <= (int64_t)kOrthBlocks * 128) {
+        const unsigned nb = (unsigned)((n + 127) / 128);
+        const size_t sm = sizeof(double) * k * 4;
+        k_orth<0, 128><<<nb, 128, sm, st>>>(V, n, k, w, n, nullptr, part, ticket, hcol, nullptr, none);
+        k_orth<1, 128><<<nb, 128, sm, st>>>(V, n, k, w, n, hcol, part, ticket, htmp, hcol, none);
+        k_orth<2, 128><<<nb, 128, 0, st>>>(V, n, k, w, n, htmp, part, ticket, hcol + k, nullptr, G);
+    } else {
+        const unsigned nb = (unsigned)std::min<int64_t>(kOrthBlocks, (n + 511) / 512);
+        const size_t sm = sizeof(double) * k * 16;
+        if (sm > 40 * 1024) {                           // k > 320 of at most 501
+            cudaFuncSetAttribute(k_orth<0, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            cudaFuncSetAttribute(k_orth<1, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        }
+        k_orth<0, 512><<<nb, 512, sm, st>>>(V, n, k, w, n, nullptr, part, ticket, hcol, nullptr, none);
+        k_orth<1, 512><<<nb, 512, sm, st>>>(V, n, k, w, n, hcol, part, ticket, htmp, hcol, none);
+        k_orth<2, 512><<<nb, 512, 0, st>>>(V, n, k, w, n, htmp, part, ticket, hcol + k, nullptr, G);
+    }
 }
 
 __global__ void k_axpy_dev(const double* coef, double sign, const double* x, double* y, int64_t n) {
@@ -155,37 +294,19 @@ __global__ void k_scale_safe(const double* x, const double* div, double* y, int6
         y[i] = x[i] * s;
 }
 
-// Device-side Givens QR of the Hessenberg matrix, one column per call (single thread):
-// hcol[0..j+1] is column j of H; R [m][m] upper triangle, cs/sn rotations, gv the rotated rhs.
-__global__ void k_givens_step(const double* hcol, int j, int m, double* R, double* cs, double* sn, double* gv) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double h[2];
-    double col[512];
-    for (int i = 0; i <= j + 1 && i < 512; ++i) col[i] = hcol[i];
-    for (int i = 0; i < j; ++i) {
-        double t = cs[i] * col[i] + sn[i] * col[i + 1];
-        col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-        col[i] = t;
-    }
-    h[0] = col[j];
-    h[1] = col[j + 1];
-    const double den = hypot(h[0], h[1]);
-    cs[j] = den > 0.0 ? h[0] / den : 1.0;
-    sn[j] = den > 0.0 ? h[1] / den : 0.0;
-    col[j] = den;
-    for (int i = 0; i <= j; ++i) R[(size_t)i * m + j] = col[i];
-    gv[j + 1] = -sn[j] * gv[j];
-    gv[j] = cs[j] * gv[j];
-}
-
-// y = R^{-1} gv (k x k upper triangle, zero diagonals skipped)
+// y = R^{-1} gv (k x k upper triangle, zero diagonals skipped), one warp: the solved entry
+// updates the entries above it, lanes over the rows
 __global__ void k_backsolve(const double* R, const double* gv, int k, int m, double* y) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double g[kMaxBasis];
+    const int lane = threadIdx.x;
+    for (int i = lane; i < k; i += 32) g[i] = gv[i];
+    __syncwarp();
     for (int i = k - 1; i >= 0; --i) {
-        double s = gv[i];
-        for (int l = i + 1; l < k; ++l) s -= R[(size_t)i * m + l] * y[l];
         const double d = R[(size_t)i * m + i];
-        y[i] = d != 0.0 ? s / d : 0.0;
+        const double yi = d != 0.0 ? g[i] / d : 0.0;
+        for (int l = lane; l < i; l += 32) g[l] -= R[(size_t)l * m + i] * yi;
+        if (lane == 0) y[i] = yi;
+        __syncwarp();
     }
 }
 

@@ -37,6 +37,56 @@ __device__ __forceinline__ int patch_face(const TetElem& d, int i) {
     return f;
 }
 
+// The 32 x 32 diagonal blocks of the factors P S_r = L U replaced in place by their triangles' inverses
+// (unit lower L^{-1} below the diagonal, U^{-1} on and above it), one warp per triangle, a column of
+// the inverse per lane: a substitution then multiplies by them instead of running 32 dependent
+// steps per block.  A zero or non-finite pivot counts as one (it is flagged by the elimination).
+// buf: 4 x 32 x 33 words of shared memory; the CTA's NTH threads.
+template <class T>
+__device__ void asm_invert_diagonal(T* A, int t, int lda, T* buf) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T* S = buf + (warp >> 1) * 32 * 33;
+    static_assert(NTH / 64 * 32 * 33 <= TMAX * ASM_NB, "staged blocks fit the panel");
+    const int nblk = (t + 31) / 32;
+    __syncthreads();
+    for (int g0 = 0; g0 < nblk; g0 += NTH / 64) {                  // a pair of warps per block
+        const int blk = g0 + (warp >> 1), b0 = 32 * blk, nb = max(0, min(32, t - b0));
+        const bool lower = (warp & 1) == 0;
+        T x[32];
+        for (int r = warp & 1; r < nb; r += 2) S[r * 33 + lane] = lane < nb ? A[(size_t)(b0 + r) * lda + b0 + lane] : T(0);
+        __syncthreads();
+        if (blk < nblk) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) x[r] = r == lane ? T(1) : T(0);
+            if (lower) {
+#pragma unroll
+                for (int r = 1; r < 32; ++r)
+#pragma unroll
+                    for (int c = 0; c < r; ++c)
+                        if (r < nb) x[r] = fma(-S[r * 33 + c], x[c], x[r]);
+            } else {
+#pragma unroll
+                for (int r = 31; r >= 0; --r) {
+                    if (r >= nb) continue;
+#pragma unroll
+                    for (int c = r + 1; c < 32; ++c)
+                        if (c < nb) x[r] = fma(-S[r * 33 + c], x[c], x[r]);
+                    T dk = S[r * 33 + r];
+                    if (dk == T(0) || !isfinite(dk)) dk = T(1);
+                    x[r] /= dk;
+                }
+            }
+        }
+        if (lane < nb) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                if (r < nb && (lower ? lane < r : lane >= r)) A[(size_t)(b0 + r) * lda + b0 + lane] = x[r];
+        }
+        __syncthreads();                                           // the staged blocks are free
+    }
+}
+
+
 template <class T>
 __global__ void __launch_bounds__(NTH, 2) k_tet_asm_factor(const TetElem* __restrict__ el, const int32_t* order,
                                                            int64_t E, int32_t* next, const T* __restrict__ vals,
@@ -116,29 +166,60 @@ __global__ void __launch_bounds__(NTH, 2) k_tet_asm_factor(const TetElem* __rest
         }
         __syncthreads();
         for (int i = tid; i < t; i += NTH) gp[i] = sperm[i];
+        asm_invert_diagonal(A, t, lda, pan);
         __syncthreads();
     }
 }
 
+// VW consecutive values of a factor row, 16 bytes
+template <class T> struct Vec16;
+template <> struct Vec16<float> { using V = float4; };
+template <> struct Vec16<double> { using V = double2; };
+
+// sum over k in [k0, k1) of row[k] y[k] by the four threads of a row (q = 0..3), k0 a multiple of 32;
+// the loads of up to eight groups of 16 bytes per thread go out together
 template <class T>
-__device__ __forceinline__ T warp_sum(T s) {
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+__device__ __forceinline__ T asm_row_dot(const T* row, const T* y, int k0, int k1, int q) {
+    using V = typename Vec16<T>::V;
+    constexpr int VW = 16 / sizeof(T), U = 8;
+    T s = T(0);
+    for (int k = k0 + q * VW; k < k1; k += 4 * VW * U) {
+        V v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k + 4 * VW * u < k1) v[u] = __ldcs(reinterpret_cast<const V*>(row + k + 4 * VW * u));
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const T* x = reinterpret_cast<const T*>(&v[u]);
+#pragma unroll
+            for (int w = 0; w < VW; ++w) {
+                const int kk = k + 4 * VW * u + w;
+                if (kk < k1) s = fma(x[w], y[kk], s);
+            }
+        }
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
     return s;
 }
 
-// z_r = S_r^{-1} R_r x = U^{-1} L^{-1} P R_r x for every patch, in the factors' precision
+// z_r = S_r^{-1} R_r x = U^{-1} L^{-1} P R_r x for every patch, in the factors' precision, one CTA per
+// patch: 32-row blocks, the rows first reduced by the solved part (four threads per row, every 16-byte
+// load of a row in flight at once, the block's diagonal part loaded ahead of them), then the inverse of
+// the 32 x 32 diagonal triangle (stored by the set-up) times the result.  Bound by the stream of the
+// factors (FP32, 2520 patches of t = 219 on average, 0.52 GB): 123 us; 296 with one warp per row, whose
+// eight rows of a block waited for each other's loads, and 191 with a 32-step substitution per block.
 template <class T>
-__global__ void __launch_bounds__(ASM_SOLVE_THREADS) k_tet_asm_solve(const TetElem* __restrict__ el,
-                                                                     const T* __restrict__ lu,
-                                                                     const int64_t* __restrict__ aoff,
-                                                                     const int32_t* __restrict__ perm,
-                                                                     const int64_t* __restrict__ poff,
-                                                                     const double* __restrict__ x, double* z) {
+__global__ void __launch_bounds__(ASM_SOLVE_THREADS, 8) k_tet_asm_solve(const TetElem* __restrict__ el,
+                                                                        const T* __restrict__ lu,
+                                                                        const int64_t* __restrict__ aoff,
+                                                                        const int32_t* __restrict__ perm,
+                                                                        const int64_t* __restrict__ poff,
+                                                                        const double* __restrict__ x, double* z) {
+    static_assert(ASM_SOLVE_THREADS == 128, "four threads per row of a 32-row block");
     __shared__ T y[TMAX];
-    __shared__ T D[32][33];
-    __shared__ T part[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = ASM_SOLVE_THREADS / 32;
+    __shared__ T rhs[32];
+    const int tid = threadIdx.x, r = tid >> 2, q = tid & 3;
     const int64_t e = blockIdx.x;
     const TetElem& d = el[e];
     const int t = d.t, lda = (t + 3) & ~3;
@@ -149,60 +230,39 @@ __global__ void __launch_bounds__(ASM_SOLVE_THREADS) k_tet_asm_solve(const TetEl
         y[i] = (T)x[d.hoff[f] + (s - d.toff[f])];
     }
     __syncthreads();
-    // forward substitution with the unit lower factor
-    for (int b0 = 0; b0 < t; b0 += 32) {
+    // row r of the block at b0: its diagonal part (columns c with c % 4 == q) and its right-hand side
+    // less the sum over the solved columns [k0, k1)
+    T dg[8];
+    auto reduce_rows = [&](int b0, int nb, int k0, int k1) {
+        const T* row = A + (size_t)(b0 + min(r, nb - 1)) * lda;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) dg[u] = q + 4 * u < nb ? row[b0 + q + 4 * u] : T(0);
+        const T s = asm_row_dot(row, y, k0, k1, q);
+        if (q == 0) rhs[r] = r < nb ? y[b0 + r] - s : T(0);
+    };
+    // the block's rows: rhs = y - part, then the inverse triangle of the diagonal block times it
+    auto solve_block = [&](int b0, int nb, bool lower) {
+        __syncthreads();
+        T s = lower && q == 0 ? rhs[r] : T(0);                    // the lower factor's unit diagonal
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int c = q + 4 * u;
+            if (c < nb && (lower ? c < r : c >= r)) s = fma(dg[u], rhs[c], s);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (q == 0 && r < nb) y[b0 + r] = s;
+        __syncthreads();
+    };
+    for (int b0 = 0; b0 < t; b0 += 32) {                          // forward substitution
         const int nb = min(32, t - b0);
-        for (int rr = warp; rr < nb; rr += NW) {
-            const T* row = A + (size_t)(b0 + rr) * lda;
-            T s = T(0);
-            for (int k = lane; k < b0; k += 32) s = fma(row[k], y[k], s);
-            s = warp_sum(s);
-            if (lane == 0) part[rr] = s;
-        }
-        for (int idx = tid; idx < nb * 32; idx += ASM_SOLVE_THREADS) {
-            const int r = idx >> 5, c = idx & 31;
-            if (c < nb) D[r][c] = A[(size_t)(b0 + r) * lda + b0 + c];
-        }
-        __syncthreads();
-        if (warp == 0) {
-            T v = lane < nb ? y[b0 + lane] - part[lane] : T(0);
-            for (int k = 0; k < nb; ++k) {
-                const T yk = __shfl_sync(0xffffffffu, v, k);
-                if (lane > k && lane < nb) v = fma(-D[lane][k], yk, v);
-            }
-            if (lane < nb) y[b0 + lane] = v;
-        }
-        __syncthreads();
+        reduce_rows(b0, nb, 0, b0);
+        solve_block(b0, nb, true);
     }
-    // back substitution with the upper factor
-    for (int b1 = t; b1 > 0; b1 -= 32) {
-        const int b0 = max(0, b1 - 32), nb = b1 - b0;
-        for (int rr = warp; rr < nb; rr += NW) {
-            const T* row = A + (size_t)(b0 + rr) * lda;
-            T s = T(0);
-            for (int k = b1 + lane; k < t; k += 32) s = fma(row[k], y[k], s);
-            s = warp_sum(s);
-            if (lane == 0) part[rr] = s;
-        }
-        for (int idx = tid; idx < nb * 32; idx += ASM_SOLVE_THREADS) {
-            const int r = idx >> 5, c = idx & 31;
-            if (c < nb) D[r][c] = A[(size_t)(b0 + r) * lda + b0 + c];
-        }
-        __syncthreads();
-        if (warp == 0) {
-            T v = lane < nb ? y[b0 + lane] - part[lane] : T(0);
-            for (int k = nb - 1; k >= 0; --k) {
-                if (lane == k) {
-                    T dk = D[k][k];
-                    if (dk == T(0) || !isfinite(dk)) dk = T(1);   // flagged at set-up
-                    v = v / dk;
-                }
-                const T xk = __shfl_sync(0xffffffffu, v, k);
-                if (lane < k) v = fma(-D[lane][k], xk, v);
-            }
-            if (lane < nb) y[b0 + lane] = v;
-        }
-        __syncthreads();
+    for (int b0 = (t - 1) & ~31; b0 >= 0; b0 -= 32) {             // back substitution
+        const int nb = min(32, t - b0);
+        reduce_rows(b0, nb, b0 + 32, t);
+        solve_block(b0, nb, false);
     }
     double* zr = z + poff[e];
     for (int i = tid; i < t; i += ASM_SOLVE_THREADS) zr[i] = (double)y[i];
