@@ -205,3 +205,26 @@ def test_linearize_returns_the_fp64_residual_norm(prec):
     assert abs(r - full) < TOL * full
     assert np.array_equal(run.blocks(), v0) and np.array_equal(run.rhs(), g0)
     run.close()
+
+
+@pytest.mark.parametrize("n,restart", [(8, 12), (41, 350)], ids=["one-wave-of-narrow-blocks", "wide-blocks-long-basis"])
+def test_gmres_reports_the_residual_it_reaches(n, restart):
+    """Both block widths of the Gram-Schmidt kernels and a basis past the default shared memory: the Krylov
+    recurrence's residual is the true one (64-bit CGS2 keeps the basis orthogonal to rounding)."""
+    import torch
+    from paper_2608_27863_gb300 import hdg as H
+    P = synth.config1(n=n)
+    run = GpuRun(P)
+    dt = P.dt if n == 8 else 300 * P.dt          # a long step: hundreds of iterations
+    H.hdg_linearize_condense(run.h, run.U, run.Q, run.UH, run.Ustar, run.nu, dt, P.a_ii)
+    N = run.UH.numel()
+    assert (N <= 152 * 128) == (n == 8)
+    b = torch.randn(N, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    x, r = torch.zeros_like(b), torch.empty_like(b)
+    it, rel = H.hdg_gmres(run.h, b, x, restart=restart, max_iter=restart, rtol=1e-14, precond=False,
+                          raise_on_noconv=False)
+    assert it == restart or it > 320
+    H.hdg_trace_matvec(run.h, x, r)
+    true = float((b - r).norm() / b.norm())
+    assert abs(true - rel) <= 1e-9 * max(true, rel) + 1e-13, (true, rel)
+    run.close()
