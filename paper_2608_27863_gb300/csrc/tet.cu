@@ -35,16 +35,15 @@ constexpr int64_t W_PQ = W_PU + NPT * M;                 // [NPT][m][3] q
 constexpr int64_t W_PL = W_PQ + NPT * M * 3;             // [NPT][m][3] lifted q
 constexpr int64_t W_PH = W_PL + NPT * M * 3;             // [4 NFQMAX][m] uhat
 constexpr int64_t W_CV = W_PH + 4 * NFQMAX * M;          // [NQMAX][a][r][b][kind 4]
-constexpr int64_t W_CF = W_CV + (int64_t)NQMAX * 300;    // [4 NFQMAX][a][b][kind 5]  element rows (dt folded)
-constexpr int64_t W_CB = W_CF + 4 * NFQMAX * 125;        // [4 NFQMAX][a][b][kind 5]  trace rows
+constexpr int64_t W_CF = W_CV + (int64_t)NQMAX * 300;    // [4 NFQMAX][a][b][kind 5]  flux rows
+constexpr int64_t W_CB = W_CF + 4 * NFQMAX * 125;        // [4 NFQMAX][a][b][kind 5]  boundary faces' trace rows
 constexpr int64_t W_RV = W_CB + 4 * NFQMAX * 125;        // [NQMAX][a][r]
 constexpr int64_t W_RF = W_RV + NQMAX * 15;              // [4 NFQMAX][a]
 constexpr int64_t W_RB = W_RF + 4 * NFQMAX * M;          // [4 NFQMAX][a]
 constexpr int64_t W_MM = W_RB + 4 * NFQMAX * M;          // [NPMAX][NPMAX] mass matrix, then its Cholesky factor
-constexpr int64_t W_DP = W_MM + NPMAX * NPMAX;           // [NQMAX][3][NPMAX] physical gradients, then (FP64 form)
-                                                         // the modal lifting operators [3][Np][Nc]
-constexpr int64_t W_VQ = W_DP + NQMAX * 3 * NPMAX;       // mixed form: [3][NPT][NCM] psi | chi; FP64 form: the face,
-                                                         // then the volume coupling matrices of the contraction
+constexpr int64_t W_DP = W_MM + NPMAX * NPMAX;           // [NQMAX][3][NPMAX] physical gradients, then the modal
+                                                         // lifting operators [3][Np][Nc]
+constexpr int64_t W_VQ = W_DP + NQMAX * 3 * NPMAX;       // the face, then the volume matrices of the contraction
 constexpr int64_t W_GHF = W_VQ + 3LL * NPT * NCM;       // mixed form: FP32 copies of G | H
 constexpr int64_t W_END = W_GHF + (3LL * NPMAX * NCM + 1) / 2;
 
@@ -148,7 +147,7 @@ __device__ void load_geometry(const KArgs& A, const TetElem& d, double* gv, doub
 }
 
 // ---------------------------------------------------------------------------
-// FP64 form: the contraction A2.
+// The contraction A2, on the FP64 pipe (FP64 form) or the FP32 one (mixed form).
 //
 // The q variation of a unit column c is -sum_j phi_j GH_k[j][c] (GH = [G | H]), a
 // polynomial of the element space, so the viscous part of a block factors into
@@ -166,7 +165,10 @@ __device__ void load_geometry(const KArgs& A, const TetElem& d, double* gv, doub
 // viscous part, nor does dF_momentum / dE: 8 of the 25 pairs stop at K0.
 // One p = 4 element with degree-4 faces: 21e6 multiply-adds for 78e6 of the product
 // of every row basis with every column at every point, which this replaced; the
-// 3,600-element launch (tet p = 1..4, curved) fell from 288 to 124 ms.  Every phase
+// 3,600-element launch (tet p = 1..4, curved) fell from 288 to 124 ms in FP64.  The mixed
+// form's products ran as 3xTF32 tensor-core tiles whose operand forming bound them (25 Np rows x
+// (4 Nq + 5 sum Nfq) coefficients per element); the factored form has so few multiply-adds that the
+// FP32 pipe is faster: 7,200 elements 74.3 -> 62.3 ms, and closer to 64 bits (9.1e-6 -> 7.6e-6).  Every phase
 // runs over a flat list of (pair, tile) items, so that low degrees fill the CTA too.
 constexpr int NVIS = 17;                       // component pairs with a viscous part
 constexpr int NKM = M * M + 3 * NVIS;          // volume matrices: K0 of every pair, K1..3 of the viscous ones
@@ -185,40 +187,40 @@ __device__ __forceinline__ void pair_of(int q, int& a, int& b) {
 
 // volume matrices in the modal basis, KM[matrix][m][i]: matrix q < 25 is K0 of pair q,
 // 25 + 3 q + k - 1 is Kk; one (matrix, i) per thread and step, st = the 1-D factors
-template <int P>
-__device__ __noinline__ void contract_volume(const double* __restrict__ dphi, const double* __restrict__ cv,
-                                             const double* st, double* __restrict__ KM) {
+template <int P, class T>
+__device__ __noinline__ void contract_volume(const T* __restrict__ dphi, const T* __restrict__ cv, const T* st,
+                                             T* __restrict__ KM) {
     constexpr int N1 = P + 1, Q = P + 2, NT2 = (P + 1) * (P + 2) / 2, NP = (P + 1) * (P + 2) * (P + 3) / 6;
     constexpr int NQ = Q * Q * Q;
-    const double* TA = st;
-    const double* TB = TA + Q * N1;
-    const double* TC = TB + Q * NT2;
+    const T* TA = st;
+    const T* TB = TA + Q * N1;
+    const T* TC = TB + Q * NT2;
     for (int item = threadIdx.x; item < NKM * NP; item += NTH) {
         const int mat = item / NP, i = item - mat * NP;
         const int q = mat < M * M ? mat : (mat - M * M) / 3, kind = mat < M * M ? 0 : (mat - M * M) % 3 + 1;
         int a, b;
         pair_of(q, a, b);
-        const double* o = cv + (a * 3 * M + b) * 4 + kind;
-        const double* dp = dphi + i;
-        double v[NP];
+        const T* o = cv + (a * 3 * M + b) * 4 + kind;
+        const T* dp = dphi + i;
+        T v[NP];
 #pragma unroll
-        for (int m = 0; m < NP; ++m) v[m] = 0.0;
+        for (int m = 0; m < NP; ++m) v[m] = T(0);
 #pragma unroll 1
         for (int gc = 0; gc < Q; ++gc) {
-            double u[NT2];
+            T u[NT2];
 #pragma unroll
-            for (int m = 0; m < NT2; ++m) u[m] = 0.0;
+            for (int m = 0; m < NT2; ++m) u[m] = T(0);
 #pragma unroll 1
             for (int gb = 0; gb < Q; ++gb) {
                 const int g0 = (gc * Q + gb) * Q;
-                double t[N1];
+                T t[N1];
 #pragma unroll
-                for (int m = 0; m < N1; ++m) t[m] = 0.0;
+                for (int m = 0; m < N1; ++m) t[m] = T(0);
 #pragma unroll
                 for (int ga = 0; ga < Q; ++ga) {
                     const int g = g0 + ga;
-                    const double* og = o + (size_t)g * 300;
-                    const double x = dp[g * NP] * og[0] + dp[(NQ + g) * NP] * og[M * 4] +
+                    const T* og = o + (size_t)g * 300;
+                    const T x = dp[g * NP] * og[0] + dp[(NQ + g) * NP] * og[M * 4] +
                                      dp[(2 * NQ + g) * NP] * og[2 * M * 4];
 #pragma unroll
                     for (int m = 0; m < N1; ++m) t[m] = fma(TA[ga * N1 + m], x, t[m]);
@@ -237,7 +239,7 @@ __device__ __noinline__ void contract_volume(const double* __restrict__ dphi, co
 #pragma unroll
                     for (int k = 0; k < N1 - m - j; ++k, ++ijk) v[ijk] = fma(TC[gc * NP + ijk], u[ij], v[ijk]);
         }
-        double* out = KM + (size_t)mat * NP * NP + i;
+        T* out = KM + (size_t)mat * NP * NP + i;
 #pragma unroll
         for (int m = 0; m < NP; ++m) out[m * NP] = v[m];
     }
@@ -246,33 +248,34 @@ __device__ __noinline__ void contract_volume(const double* __restrict__ dphi, co
 // face matrices KF[face][matrix][j][l] (strides NFPMAX): matrix q < 25 couples uhat node j of the
 // face in pair q, 25 + a the element's node j on the face through tau (a = b), 30 + 3 q + k - 1 that
 // node's q_k
-__device__ __noinline__ void contract_faces(const TetElem& d, const double* __restrict__ tab,
-                                            const double* __restrict__ cf, double* __restrict__ KF) {
+template <class T>
+__device__ __noinline__ void contract_faces(const TetElem& d, const T* __restrict__ tab, const T* __restrict__ cf,
+                                            T* __restrict__ KF) {
     const int nP = (d.p + 1) * (d.p + 2) / 2;
     for (int f = 0; f < 4; ++f) {
         const int nfp = d.nfp[f], nfq = d.nfq[f];
-        const double* mu = tab + d.ttab[f];
-        const double* ph = tab + d.ctab[f];
-        const double* co = cf + (size_t)d.soff[f] * 125;
+        const T* mu = tab + d.ttab[f];
+        const T* ph = tab + d.ctab[f];
+        const T* co = cf + (size_t)d.soff[f] * 125;
         for (int item = threadIdx.x; item < NKF * nfp; item += NTH) {
             const int mat = item / nfp, l = item - mat * nfp;
             int a, b, kind;
             if (mat < M * M) { pair_of(mat, a, b); kind = 1; }
             else if (mat < M * M + M) { a = b = mat - M * M; kind = 0; }
             else { pair_of((mat - M * M - M) / 3, a, b); kind = 2 + (mat - M * M - M) % 3; }
-            const double* ch = kind == 1 ? mu : ph;
+            const T* ch = kind == 1 ? mu : ph;
             const int n = kind == 1 ? nfp : nP;
-            const double* o = co + (a * M + b) * 5 + kind;
-            double acc[NFPMAX];
+            const T* o = co + (a * M + b) * 5 + kind;
+            T acc[NFPMAX];
 #pragma unroll
-            for (int j = 0; j < NFPMAX; ++j) acc[j] = 0.0;
+            for (int j = 0; j < NFPMAX; ++j) acc[j] = T(0);
             for (int s = 0; s < nfq; ++s) {
-                const double w = mu[s * nfp + l] * o[(size_t)s * 125];
+                const T w = mu[s * nfp + l] * o[(size_t)s * 125];
 #pragma unroll
                 for (int j = 0; j < NFPMAX; ++j)
                     if (j < n) acc[j] = fma(w, ch[s * n + j], acc[j]);
             }
-            double* out = KF + ((size_t)(f * NKF + mat) * NFPMAX) * NFPMAX + l;
+            T* out = KF + ((size_t)(f * NKF + mat) * NFPMAX) * NFPMAX + l;
 #pragma unroll
             for (int j = 0; j < NFPMAX; ++j)
                 if (j < n) out[j * NFPMAX] = acc[j];
@@ -281,9 +284,10 @@ __device__ __noinline__ void contract_faces(const TetElem& d, const double* __re
 }
 
 // the flux rows of every face into the trace rows of the bordered matrix, tiles of 5 rows x 4 columns
+template <class T>
 __device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& d, const int* fpo,
-                                                 const double* __restrict__ Gk, const double* __restrict__ Hk,
-                                                 const double* __restrict__ KF, double* __restrict__ Mx) {
+                                                 const T* __restrict__ Gk, const T* __restrict__ Hk,
+                                                 const T* __restrict__ KF, double* __restrict__ Mx) {
     const int Np = d.Np, sfp = d.t / M, Nc = Np + sfp, nct = (Nc + 3) / 4, nP = (d.p + 1) * (d.p + 2) / 2;
     int tiles[5];
     tiles[0] = 0;
@@ -296,14 +300,14 @@ __device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& 
         int a, b;
         pair_of(q, a, b);
         const int32_t* fn = A.fnod + ((size_t)d.p * NCODE + d.code[f]) * FNOD;
-        const double* Kf = KF + (size_t)f * NKF * NFPMAX * NFPMAX + l0;
-        double acc[5][4];
+        const T* Kf = KF + (size_t)f * NKF * NFPMAX * NFPMAX + l0;
+        T acc[5][4];
 #pragma unroll
         for (int u = 0; u < 5; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+            for (int v = 0; v < 4; ++v) acc[u][v] = T(0);
         if (q < NVIS) {
-            const double* gp[4];
+            const T* gp[4];
             int gs[4];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -312,11 +316,11 @@ __device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& 
                 gs[v] = c < Np ? Np : sfp;
             }
             for (int k = 0; k < 3; ++k) {
-                const double* Kk = Kf + (size_t)(M * M + M + 3 * q + k) * NFPMAX * NFPMAX;
+                const T* Kk = Kf + (size_t)(M * M + M + 3 * q + k) * NFPMAX * NFPMAX;
 #pragma unroll 2
                 for (int j = 0; j < nP; ++j) {
                     const int row = k * Np + fn[j];
-                    double kv[5], gv[4];
+                    T kv[5], gv[4];
 #pragma unroll
                     for (int u = 0; u < 5; ++u) kv[u] = Kk[j * NFPMAX + u];
 #pragma unroll
@@ -337,7 +341,7 @@ __device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& 
 #pragma unroll
             for (int u = 0; u < 5; ++u) {
                 if (l0 + u >= nfp) continue;
-                double x = acc[u][v];
+                T x = acc[u][v];
                 if (c >= Np && lf >= 0 && lf < nfp) x += Kf[((size_t)q * NFPMAX + lf) * NFPMAX + u];
                 if (jp >= 0) x += Kf[((size_t)(M * M + a) * NFPMAX + jp) * NFPMAX + u];
                 Mx[(int64_t)(d.NU + d.toff[f] + a * nfp + l0 + u) * d.LD + col] = x;
@@ -348,10 +352,10 @@ __device__ __noinline__ void contract_trace_rows(const KArgs& A, const TetElem& 
 
 // the element rows: volume matrices times Vinv and the modal lifting operators GM[k][m][c], plus dt times
 // the flux rows of the faces a node lies on; tiles of 5 rows x 4 columns
-template <int P>
-__device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem& d,
-                                                   const double* __restrict__ Vinv, const double* __restrict__ KM,
-                                                   const double* __restrict__ GM, double* Mx) {
+template <int P, class T>
+__device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem& d, const T* __restrict__ tab,
+                                                   const T* __restrict__ Vinv, const T* __restrict__ KM,
+                                                   const T* __restrict__ GM, double* Mx) {
     constexpr int NP = (P + 1) * (P + 2) * (P + 3) / 6, NTI = (NP + 4) / 5;
     const int sfp = d.t / M, Nc = NP + sfp, nct = (Nc + 3) / 4;
     for (int item = threadIdx.x; item < M * M * NTI * nct; item += NTH) {
@@ -363,20 +367,20 @@ __device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem
         for (int u = 0; u < 5; ++u) iu[u] = min(i0 + u, NP - 1);
 #pragma unroll
         for (int v = 0; v < 4; ++v) cc[v] = min(c0 + v, Nc - 1);
-        double acc[5][4];
+        T acc[5][4];
 #pragma unroll
         for (int u = 0; u < 5; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+            for (int v = 0; v < 4; ++v) acc[u][v] = T(0);
         if (c0 < NP) {
-            const double* K0 = KM + (size_t)q * NP * NP;
+            const T* K0 = KM + (size_t)q * NP * NP;
 #pragma unroll 2
             for (int m = 0; m < NP; ++m) {
-                double kv[5], gv[4];
+                T kv[5], gv[4];
 #pragma unroll
                 for (int u = 0; u < 5; ++u) kv[u] = K0[m * NP + iu[u]];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) gv[v] = cc[v] < NP ? Vinv[m * NP + cc[v]] : 0.0;
+                for (int v = 0; v < 4; ++v) gv[v] = cc[v] < NP ? Vinv[m * NP + cc[v]] : T(0);
 #pragma unroll
                 for (int u = 0; u < 5; ++u)
 #pragma unroll
@@ -384,10 +388,10 @@ __device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem
             }
         }
         if (q < NVIS) {
-            const double* Kk = KM + (size_t)(M * M + 3 * q) * NP * NP;
+            const T* Kk = KM + (size_t)(M * M + 3 * q) * NP * NP;
 #pragma unroll 2
             for (int m = 0; m < 3 * NP; ++m) {          // K1, K2, K3 follow each other, and so do GM_1..3
-                double kv[5], gv[4];
+                T kv[5], gv[4];
 #pragma unroll
                 for (int u = 0; u < 5; ++u) kv[u] = Kk[m * NP + iu[u]];
 #pragma unroll
@@ -404,19 +408,19 @@ __device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem
         for (int f = 0; f < 4; ++f) {
             const int32_t* fi = A.fnod + ((size_t)P * NCODE + d.code[f]) * FNOD + NFPMAX;
             const double* row0 = Mx + (int64_t)(d.NU + d.toff[f] + a * d.nfp[f]) * d.LD;
-            const double* Pr = A.tab + d.ctab[f] + (size_t)d.nfq[f] * ((P + 1) * (P + 2) / 2);
+            const T* Pr = tab + d.ctab[f] + (size_t)d.nfq[f] * ((P + 1) * (P + 2) / 2);
 #pragma unroll
             for (int u = 0; u < 5; ++u) {
                 const int jp = fi[iu[u]];
                 if (jp < 0) continue;
                 if (d.pf[f] == P) {
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[u][v] = fma(A.dt, row0[(int64_t)jp * d.LD + col[v]], acc[u][v]);
+                    for (int v = 0; v < 4; ++v) acc[u][v] = fma((T)A.dt, (T)row0[(int64_t)jp * d.LD + col[v]], acc[u][v]);
                 } else {
                     for (int l = 0; l < d.nfp[f]; ++l) {
-                        const double w = A.dt * Pr[l * ((P + 1) * (P + 2) / 2) + jp];
+                        const T w = (T)A.dt * Pr[l * ((P + 1) * (P + 2) / 2) + jp];
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) acc[u][v] = fma(w, row0[(int64_t)l * d.LD + col[v]], acc[u][v]);
+                        for (int v = 0; v < 4; ++v) acc[u][v] = fma(w, (T)row0[(int64_t)l * d.LD + col[v]], acc[u][v]);
                     }
                 }
             }
@@ -431,23 +435,24 @@ __device__ __noinline__ void contract_element_rows(const KArgs& A, const TetElem
 
 // trace rows of boundary faces that are not flux rows: the algebraic forms' face mass couplings
 // (kind 0: the interior state, kind 1: uhat of the same face)
-__device__ __noinline__ void contract_boundary_rows(const KArgs& A, const TetElem& d, const int* fpo,
-                                                    const double* __restrict__ cb, double* __restrict__ Mx) {
+template <class T>
+__device__ __noinline__ void contract_boundary_rows(const TetElem& d, const int* fpo, const T* __restrict__ tab,
+                                                    const T* __restrict__ cb, double* __restrict__ Mx) {
     const int Np = d.Np, Nc = Np + d.t / M;
     for (int f = 0; f < 4; ++f) {
         if (d.tag[f] == 0) continue;
         const int nfp = d.nfp[f], nfq = d.nfq[f];
-        const double* mu = A.tab + d.ttab[f];
-        const double* phf = A.tab + d.ftab[f];
+        const T* mu = tab + d.ttab[f];
+        const T* phf = tab + d.ftab[f];
         for (int item = threadIdx.x; item < M * M * nfp * Nc; item += NTH) {
             const int ab = item / (nfp * Nc), rem = item - ab * nfp * Nc, l = rem / Nc, c = rem - l * Nc;
             const int a = ab / M, b = ab - a * M;
             if (boundary_row_is_flux<M>(d.tag[f], a)) continue;
             const int lf = c - Np - fpo[f];
-            const double* ch = c < Np ? phf + c : mu + lf;
+            const T* ch = c < Np ? phf + c : mu + lf;
             const int cs = c < Np ? Np : nfp;
-            const double* o = cb + (size_t)d.soff[f] * 125 + ab * 5 + (c < Np ? 0 : 1);
-            double s = 0.0;
+            const T* o = cb + (size_t)d.soff[f] * 125 + ab * 5 + (c < Np ? 0 : 1);
+            T s = T(0);
             if (c < Np || (lf >= 0 && lf < nfp))
                 for (int g = 0; g < nfq; ++g) s = fma(mu[g * nfp + l] * o[(size_t)g * 125], ch[(size_t)g * cs], s);
             Mx[(int64_t)(d.NU + d.toff[f] + a * nfp + l) * d.LD + bcol(d, b, c)] = s;
@@ -455,54 +460,40 @@ __device__ __noinline__ void contract_boundary_rows(const KArgs& A, const TetEle
     }
 }
 
-template <int P>
-__device__ void contract_fp64(const KArgs& A, const TetElem& d, const int* fpo, const double* cv, const double* cf,
-                              const double* cb, const double* Gk, const double* Hk, double* KM, double* GM,
-                              double* st, double* Mx) {
+template <int P, class T>
+__device__ void contract(const KArgs& A, const TetElem& d, const int* fpo, const T* tab, const T* cv, const T* cf,
+                         const T* cb, const T* Gk, const T* Hk, T* KM, T* GM, T* st, double* Mx) {
     constexpr int NP = (P + 1) * (P + 2) * (P + 3) / 6, Q = P + 2;
     constexpr int NFAC = Q * (P + 1) + Q * ((P + 1) * (P + 2) / 2) + Q * NP;
     const int tid = threadIdx.x, sfp = d.t / M, Nc = NP + sfp;
-    const double* Vinv = A.tab + d.stab + NFAC;
-    for (int i = tid; i < NFAC; i += NTH) st[i] = A.tab[d.stab + i];
+    const T* Vinv = tab + d.stab + NFAC;
+    for (int i = tid; i < NFAC; i += NTH) st[i] = tab[d.stab + i];
     for (int idx = tid; idx < 3 * NP * Nc; idx += NTH) {         // GM_k = Vinv [G_k | H_k]
         const int k = idx / (NP * Nc), rem = idx - k * NP * Nc, m = rem / Nc, c = rem - m * Nc;
-        const double* g = c < NP ? Gk + (size_t)k * NP * NP + c : Hk + (size_t)k * NP * sfp + (c - NP);
+        const T* g = c < NP ? Gk + (size_t)k * NP * NP + c : Hk + (size_t)k * NP * sfp + (c - NP);
         const int gs = c < NP ? NP : sfp;
-        double s = 0.0;
+        T s = T(0);
 #pragma unroll 5
         for (int j = 0; j < NP; ++j) s = fma(Vinv[m * NP + j], g[(size_t)j * gs], s);
         GM[idx] = s;
     }
-    contract_faces(d, A.tab, cf, KM);
+    contract_faces<T>(d, tab, cf, KM);
     __syncthreads();
-    contract_trace_rows(A, d, fpo, Gk, Hk, KM, Mx);
+    contract_trace_rows<T>(A, d, fpo, Gk, Hk, KM, Mx);
     __syncthreads();
-    contract_volume<P>(A.tab + d.vtab + (size_t)Q * Q * Q * NP, cv, st, KM);
+    contract_volume<P, T>(tab + d.vtab + (size_t)Q * Q * Q * NP, cv, st, KM);
     __syncthreads();
-    contract_element_rows<P>(A, d, Vinv, KM, GM, Mx);
+    contract_element_rows<P, T>(A, d, tab, Vinv, KM, GM, Mx);
     __syncthreads();
-    contract_boundary_rows(A, d, fpo, cb, Mx);
+    contract_boundary_rows<T>(d, fpo, tab, cb, Mx);
 }
 
 // ---------------------------------------------------------------------------
-// Mixed form: the contraction A2 on the tensor cores.
-//
-// The column operand of a component pair, T_ab[k][c] = sum_j s_j o_ab[k][j]
-// B_j[k][c], is linear in the point coefficients o_ab, so the element rows
-// C_ab[i][c] = sum_k R[k][i] T_ab[k][c] are also the product
-//   C[(ab, i)][c] = sum_{(j, k)} (s_j R[k][i] o_ab[k][j]) B[(j, k)][c]
-// whose column operand B is the same for all 25 pairs: the pairs stack along M
-// (25 Np rows) and B is formed once per chunk for all of them.  At a volume
-// point g the three directions of R (dphi_r[g][i]) fold into the row operand
-// too, since B depends on g only: 4 Nq terms (j = basis, psi/chi 1..3), then
-// 5 terms per face point (basis, face trace basis, psi/chi 1..3).  The trace
-// rows of face f are the same product with R = mu_f and the trace-row
-// coefficients over the points of f.  The products are 3xTF32 (hi hi + hi lo +
-// lo hi) accumulated in FP32 in tensor memory; 8 warps form the operands of
-// chunk c + 1 while the tensor cores run chunk c.
+// 3xTF32 tiles on the tensor cores (hi hi + hi lo + lo hi, FP32 accumulation in
+// tensor memory) for the Schur product of the mixed form.
 constexpr int TKC = 16;                       // K per staged chunk
 constexpr int TMT = 128;                      // rows per tile (tensor-memory lanes)
-constexpr int TNP = 96;                       // columns: Nc <= 95, padded to a multiple of 16
+constexpr int TNP = 96;                       // columns per tile
 constexpr int TSTAGE = 2 * (TMT + TNP) * TKC; // floats per stage: A hi | B hi | A lo | B lo
 constexpr int TTCOLS = 128;                   // tensor-memory columns per CTA
 static_assert(2 * TSTAGE * (int)sizeof(float) <= S_ELIM * (int)sizeof(double),
@@ -523,151 +514,6 @@ __device__ __forceinline__ void tc_put4(float* hi, float* lo, int row, int kq, c
     *reinterpret_cast<float4*>(hi + off) = h;
     *reinterpret_cast<float4*>(lo + off) =
         make_float4(tf32_round(v[0] - h.x), tf32_round(v[1] - h.y), tf32_round(v[2] - h.z), tf32_round(v[3] - h.w));
-}
-
-// one segment of the stacked product: the element rows (f = -1) or the trace
-// rows of face f.  Its K runs over blocks of one j each (volume j = 0..3 over
-// the Nq points, then face j = 0..4 over the sum_f Nfq face points; trace rows:
-// j = 0..4 over the Nfq points of face f), every block padded to whole chunks
-// so that a chunk has one j and consecutive points.
-struct TcSeg {
-    int f, rows, rdiv;      // rdiv: rows per pair (Np, or Nfp of face f)
-    int cv, cf, nch;        // chunks per volume block, per face block; chunks in all
-};
-
-struct TcChunk {
-    bool vol;
-    int j, p0, np;          // the chunk's points p0 .. p0 + 15 below the block's end np (face points:
-                            // an index into the sum_f Nfq face points)
-};
-
-__device__ __forceinline__ TcChunk tc_chunk(const TetElem& d, const TcSeg& sg, int ci) {
-    TcChunk k;
-    if (sg.f < 0 && ci < 4 * sg.cv) {
-        k.vol = true; k.j = ci / sg.cv; k.p0 = (ci - k.j * sg.cv) * TKC; k.np = d.Nq;
-        return k;
-    }
-    const int c2 = sg.f < 0 ? ci - 4 * sg.cv : ci;
-    k.vol = false; k.j = c2 / sg.cf;
-    const int base = sg.f < 0 ? 0 : d.soff[sg.f];
-    k.p0 = base + (c2 - k.j * sg.cf) * TKC;
-    k.np = base + (sg.f < 0 ? d.sfq : d.nfq[sg.f]);
-    return k;
-}
-
-// the row of the tile this thread forms: (pair, i), fixed over the chunks of a tile
-struct TcRow {
-    bool live;
-    int i, cvo, cfo;        // basis index; coefficient offsets of the pair in cv and in cf / cb
-};
-
-// operands of chunk k of the row tile at m0 into stage sb (A hi | B hi | A lo | B lo);
-// thread tid forms row tid % 128 for the K quads tid / 128 and tid / 128 + 2, and
-// column operand entries tid and tid + 256.  Every load of a thread's entries
-// goes out before the first is used (indices clamped into range, padding masked
-// afterwards), so that they are in flight together.
-__device__ void tc_form(const TetElem& d, const TcSeg& sg, const TcRow& rw, const TcChunk& k, int ncp,
-                        const float* tabJ, const float* cv, const float* cfb, const float* vq, const int* fpo,
-                        float* sb) {
-    const int tid = threadIdx.x, Np = d.Np, Nq = d.Nq, Nc = Np + d.t / M;
-    float* Ah = sb;
-    float* Bh = Ah + TMT * TKC;
-    float* Al = Bh + TNP * TKC;
-    float* Bl = Al + TMT * TKC;
-    const int rl = tid & (TMT - 1);
-    const float sgn = k.vol ? (k.j > 0 ? -1.f : 1.f) : (k.j > 1 ? -1.f : 1.f);
-    float va[2][4], vb[2][4];
-    // row operand
-    if (k.vol) {
-        const float* dphi = tabJ + d.vtab + (size_t)Nq * Np + rw.i;
-        const float* o = cv + rw.cvo + k.j;
-        float g0[2][4], g1[2][4], g2[2][4], c0[2][4], c1[2][4], c2[2][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int p = min(k.p0 + 4 * ((tid >> 7) + 2 * h) + u, k.np - 1);
-                g0[h][u] = dphi[(size_t)p * Np];
-                g1[h][u] = dphi[((size_t)Nq + p) * Np];
-                g2[h][u] = dphi[((size_t)2 * Nq + p) * Np];
-                const float* op = o + (size_t)p * 300;
-                c0[h][u] = op[0];
-                c1[h][u] = op[M * 4];
-                c2[h][u] = op[2 * M * 4];
-            }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                va[h][u] = sgn * fmaf(g2[h][u], c2[h][u], fmaf(g1[h][u], c1[h][u], g0[h][u] * c0[h][u]));
-    } else {
-        float rb[2][4], cb4[2][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int p = min(k.p0 + 4 * ((tid >> 7) + 2 * h) + u, k.np - 1);
-                rb[h][u] = sg.f < 0 ? basis_row_t(tabJ, d, Nq + p)[rw.i]
-                                    : tabJ[d.ttab[sg.f] + (size_t)(p - d.soff[sg.f]) * sg.rdiv + rw.i];
-                cb4[h][u] = cfb[(size_t)p * 125 + rw.cfo + k.j];
-            }
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) va[h][u] = sgn * rb[h][u] * cb4[h][u];
-    }
-    // column operand
-    int nn[2], qq[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int it = min(tid + h * NTH, ncp * (TKC / 4) - 1);
-        nn[h] = it % ncp;
-        qq[h] = it / ncp;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int p = min(k.p0 + 4 * qq[h] + u, k.np - 1), c = min(nn[h], Nc - 1);
-            float x;
-            if (k.vol) {
-                x = k.j == 0 ? tabJ[d.vtab + (size_t)p * Np + min(c, Np - 1)]
-                             : vq[((size_t)(k.j - 1) * NPT + p) * NCM + c];
-            } else if (k.j == 0) {
-                x = basis_row_t(tabJ, d, Nq + p)[min(c, Np - 1)];
-            } else if (k.j == 1) {
-                const int f = face_of_point(d, p), nf = d.nfp[f];
-                const int l = min(max(c - Np - fpo[f], 0), nf - 1);
-                x = tabJ[d.ttab[f] + (size_t)(p - d.soff[f]) * nf + l];
-            } else {
-                x = vq[((size_t)(k.j - 2) * NPT + Nq + p) * NCM + c];
-            }
-            vb[h][u] = x;
-        }
-    }
-    // masks and stores
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int q = (tid >> 7) + 2 * h;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (!rw.live || k.p0 + 4 * q + u >= k.np) va[h][u] = 0.f;
-        tc_put4(Ah, Al, rl, q, va[h]);
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (tid + h * NTH >= ncp * (TKC / 4)) continue;
-        const int n = nn[h], q = qq[h];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            bool ok = n < Nc && k.p0 + 4 * q + u < k.np;
-            if (ok && k.j == 0) ok = n < Np;
-            if (ok && !k.vol && k.j == 1) {
-                const int p = k.p0 + 4 * q + u, f = face_of_point(d, p), l = n - Np - fpo[f];
-                ok = l >= 0 && l < d.nfp[f];
-            }
-            if (!ok) vb[h][u] = 0.f;
-        }
-        tc_put4(Bh, Bl, n, q, vb[h]);
-    }
-    asm volatile("fence.proxy.async.shared::cta;");
 }
 
 // wait for the batch committed to stage sb (if any); on a timeout the status
@@ -769,53 +615,6 @@ __device__ void tc_tile_store(const TcState& ts, int ncp, Store&& store) {
 __device__ __forceinline__ void tc_tile_done() {
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-}
-
-// the whole contraction of one element (element rows, then the trace rows of
-// each face) into the bordered matrix Mx, FP64 storage
-__device__ void contract_tc(const TetElem& d, const float* tabJ, const float* cv, const float* cf, const float* cb,
-                            const float* vq, const int* fpo, double* Mx, float* st0, TcState& ts, int* sflag) {
-    const int tid = threadIdx.x;
-    const int Np = d.Np, LD = d.LD, NU = d.NU, Nc = Np + d.t / M;
-    const int ncp = (Nc + 15) / 16 * 16;
-    for (int sgi = -1; sgi < 4; ++sgi) {
-        TcSeg sg;
-        sg.f = sgi;
-        sg.rdiv = sgi < 0 ? Np : d.nfp[sgi];
-        sg.rows = M * M * sg.rdiv;
-        sg.cv = (d.Nq + TKC - 1) / TKC;
-        sg.cf = ((sgi < 0 ? d.sfq : d.nfq[sgi]) + TKC - 1) / TKC;
-        sg.nch = (sgi < 0 ? 4 * sg.cv : 0) + 5 * sg.cf;
-        const float* cfb = sgi < 0 ? cf : cb;
-        for (int m0 = 0; m0 < sg.rows; m0 += TMT) {
-            TcRow rw;
-            {
-                const int r = m0 + (tid & (TMT - 1));
-                const int ab = r / sg.rdiv, a = ab / M, b = ab - a * M;
-                rw.live = r < sg.rows;
-                rw.i = rw.live ? r - ab * sg.rdiv : 0;
-                rw.cvo = rw.live ? (a * 3 * M + b) * 4 : 0;
-                rw.cfo = rw.live ? (a * M + b) * 5 : 0;
-            }
-            auto form = [&](int ci, float* sb) {
-                tc_form(d, sg, rw, tc_chunk(d, sg, ci), ncp, tabJ, cv, cfb, vq, fpo, sb);
-            };
-            if (tc_tile(ts, st0, sg.nch, ncp, form, sflag)) {
-                tc_tile_store(ts, ncp, [&](int rl, int c0, const uint32_t* v) {
-                    const int r = m0 + rl;
-                    if (r >= sg.rows) return;
-                    const int ab = r / sg.rdiv, i = r - ab * sg.rdiv, a = ab / M, b = ab - a * M;
-                    const int64_t row = sgi < 0 ? (int64_t)a * Np + i : (int64_t)NU + d.toff[sgi] + a * sg.rdiv + i;
-#pragma unroll
-                    for (int jj = 0; jj < 16; ++jj) {
-                        const int c = c0 + jj;
-                        if (c < Nc) Mx[row * LD + bcol(d, b, c)] = (double)__uint_as_float(v[jj]);
-                    }
-                });
-            }
-            tc_tile_done();
-        }
-    }
 }
 
 // The trace rows' Schur product of the mixed form on the tensor cores:
@@ -1105,7 +904,7 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
     // physical gradients at the volume points and the basis values, both times the
     // point weight w|J| (so that E and M take one multiply-add per point), mass matrix
     double* dp = W + W_DP;                               // [Nq][3][NPMAX] w|J| grad phi_i
-    double* wphi = W + W_VQ;                             // [Nq][NPMAX] w|J| phi_i (free until psi/chi)
+    double* wphi = W + W_VQ;                             // [Nq][NPMAX] w|J| phi_i (free until the contraction)
     for (int idx = tid; idx < Nq * Np; idx += NTH) {
         const int g = idx / Np, i = idx - g * Np;
         const double* Ji = gv + g * 10 + 1;
@@ -1193,7 +992,7 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
         dq0[idx] = -s - sQ[idx];
     }
     __syncthreads();
-    // values at the points; psi | chi (the q variation of unit U / Uhat columns)
+    // values at the points
     double* pu = W + W_PU;
     double* pq = W + W_PQ;
     double* pl = W + W_PL;
@@ -1227,37 +1026,16 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
         }
     }
     const TJ* tabJ = jtab<TJ>(A);
-    TJ* vq = reinterpret_cast<TJ*>(W + W_VQ);
+    const TJ* GJ;
     if constexpr (sizeof(TJ) == sizeof(float)) {
         TJ* gh = reinterpret_cast<TJ*>(W + W_GHF);
-        for (int i = tid; i < 3 * Np * (Np + sfp); i += NTH) gh[i] = (TJ)Gk[i];   // G and H are contiguous
-        const TJ* GJ = gh;
-        const TJ* HJ = gh + 3 * Np * Np;
-        __syncthreads();
-        const int nc4 = (Nc + 3) / 4;                   // four columns per thread: one basis load per 4 FMAs
-        for (int idx = tid; idx < 3 * npt * nc4; idx += NTH) {
-            const int k = idx / (npt * nc4), rem = idx - k * npt * nc4, x = rem / nc4, c0 = 4 * (rem - x * nc4);
-            const TJ* br = basis_row_t(tabJ, d, x);
-            const TJ* gp[4];
-            int st[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int c = min(c0 + u, Nc - 1);
-                if (c < Np) { gp[u] = GJ + (size_t)k * Np * Np + c; st[u] = Np; }
-                else { gp[u] = HJ + (size_t)k * Np * sfp + (c - Np); st[u] = sfp; }
-            }
-            TJ s[4] = {0, 0, 0, 0};
-            for (int j = 0; j < Np; ++j) {
-                const TJ b = br[j];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) s[u] += b * gp[u][j * st[u]];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c0 + u < Nc) vq[((size_t)k * NPT + x) * NCM + c0 + u] = s[u];
-        }
-        __syncthreads();
+        for (int i = tid; i < 3 * Np * Nc; i += NTH) gh[i] = (TJ)Gk[i];   // G and H are contiguous
+        GJ = gh;
+    } else {
+        GJ = Gk;
     }
+    const TJ* HJ = GJ + 3 * Np * Np;
+    __syncthreads();
     // A1: fluxes and their Jacobians at the points
     const PhysT<double>& P = A.ph;
     using SJ = std::conditional_t<sizeof(TJ) == sizeof(float), float, double>;   // Jacobian terms' type
@@ -1368,16 +1146,12 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
             }
             TJ* of = cf + (size_t)r * 125;
             TJ* ob = cb + (size_t)r * 125;
-            // element rows take dt * dfhat (the FP64 form stores dfhat); trace rows dfhat on flux rows, the algebraic forms
-            // otherwise (tag 1 uhat - u_b, tag 2 uhat - u, tags 3 / 4 uhat_v, and on isothermal
-            // walls uhat_rhoE - uhat_rho e_w)
+            // flux rows take dfhat; the trace rows of boundary faces that are not flux rows the algebraic
+            // forms (tag 1 uhat - u_b, tag 2 uhat - u, tags 3 / 4 uhat_v, and on isothermal walls
+            // uhat_rhoE - uhat_rho e_w)
             auto put = [&](int a, int b, int kind, double v) {
-                if (sizeof(TJ) == sizeof(double)) {       // FP64 contraction: one copy, dt applied to its rows
-                    of[(a * M + b) * 5 + kind] = (TJ)v;
-                    if (tag == 0) return;
-                } else {
-                    of[(a * M + b) * 5 + kind] = (TJ)(A.dt * v);
-                }
+                of[(a * M + b) * 5 + kind] = (TJ)v;
+                if (tag == 0) return;
                 double w = v;
                 if (!boundary_row_is_flux<M>(tag, a)) {
                     w = 0.0;
@@ -1448,19 +1222,16 @@ __device__ void process_element(const KArgs& A, const TetElem& d, double* W, dou
         }
     }
     __syncthreads();
-    if constexpr (sizeof(TJ) == sizeof(float)) {
-        // A2 on the tensor cores (pairs stacked, coefficients folded into the row operand)
-        contract_tc(d, tabJ, cv, cf, cb, vq, fpo, Mx, reinterpret_cast<float*>(sD), *ts, sflag);
-        __syncthreads();
-    } else {
-        // A2 on the FP64 pipe
-        double* KM = W + W_VQ;
-        double* GM = W + W_DP;
+    // A2: contraction into the bordered matrix
+    {
+        TJ* KM = reinterpret_cast<TJ*>(W + W_VQ);
+        TJ* GM = reinterpret_cast<TJ*>(W + W_DP);
+        TJ* st = reinterpret_cast<TJ*>(sD);
         switch (d.p) {
-            case 1: contract_fp64<1>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
-            case 2: contract_fp64<2>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
-            case 3: contract_fp64<3>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
-            default: contract_fp64<4>(A, d, fpo, cv, cf, cb, Gk, Hk, KM, GM, sD, Mx); break;
+            case 1: contract<1, TJ>(A, d, fpo, tabJ, cv, cf, cb, GJ, HJ, KM, GM, st, Mx); break;
+            case 2: contract<2, TJ>(A, d, fpo, tabJ, cv, cf, cb, GJ, HJ, KM, GM, st, Mx); break;
+            case 3: contract<3, TJ>(A, d, fpo, tabJ, cv, cf, cb, GJ, HJ, KM, GM, st, Mx); break;
+            default: contract<4, TJ>(A, d, fpo, tabJ, cv, cf, cb, GJ, HJ, KM, GM, st, Mx); break;
         }
         __syncthreads();
     }
