@@ -24,6 +24,7 @@
 
 #include "common.h"
 #include "physics.cuh"
+#include "pivot.cuh"
 #include "tc_util.cuh"
 #include "tma.h"
 
@@ -869,6 +870,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim(double* top, double* bot, in
     double* ust = pan + NR * NB;            // [NB][TCW]
     __shared__ int piv[NB];
     __shared__ int sflag;
+    __shared__ double s_inv;
     if (tid == 0) sflag = 0;
 
     for (int k0 = 0; k0 < NU; k0 += NB) {
@@ -883,19 +885,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim(double* top, double* bot, in
             // warp 0 alone: pivot search (largest magnitude, lowest row on ties) and the row
             // interchange inside the panel; one barrier per step
             if (warp == 0) {
-                double bv = -1.0;
-                int bi = INT_MAX;
-#pragma unroll 1
-                for (int rr = j + lane; rr < ntop; rr += 32) {
-                    const double v = fabs(pan[rr * NB + j]);
-                    if (v > bv) { bv = v; bi = rr; }
-                }
-                for (int off = 16; off > 0; off >>= 1) {
-                    const double ov = __shfl_down_sync(0xffffffffu, bv, off);
-                    const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-                }
-                int pr = __shfl_sync(0xffffffffu, bi, 0);
+                int pr = warp_pivot(j, ntop, [&](int r) { return pan[r * NB + j]; });
                 if (pr == INT_MAX) {
                     pr = j;
                     if (lane == 0) sflag |= 2;
@@ -905,15 +895,16 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim(double* top, double* bot, in
                     pan[j * NB + lane] = pan[pr * NB + lane];
                     pan[pr * NB + lane] = t;
                 }
-                if (lane == 0) piv[j] = pr;
+                __syncwarp();
+                if (lane == 0) {
+                    piv[j] = pr;
+                    int fl = 0;
+                    s_inv = pivot_reciprocal(pan[j * NB + j], fl);
+                    if (fl) sflag |= fl;
+                }
             }
             __syncthreads();
-            double pv = pan[j * NB + j];
-            if (pv == 0.0 || !isfinite(pv)) {
-                if (tid == 0) sflag |= (pv == 0.0) ? 1 : 2;
-                pv = 1.0;
-            }
-            const double inv = 1.0 / pv;
+            const double inv = s_inv;
 #pragma unroll 1
             for (int rr = j + 1 + tid; rr < nrows; rr += NTH) {
                 double l = pan[rr * NB + j] * inv;

@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim_mixed(Regions<float> R, int6
     float* prow = ust32 + NB * 64;                           // [NB]      pivot row (FP32)
     __shared__ int piv[NB];
     __shared__ int sflag;
+    __shared__ double s_inv;
     if (tid == 0) sflag = 0;
 
     for (int k0 = 0; k0 < NU; k0 += NB) {
@@ -133,19 +134,7 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim_mixed(Regions<float> R, int6
             // warp 0 alone: pivot search (largest magnitude, lowest row on ties), row
             // interchange inside the panel and the FP32 pivot row; one barrier per step
             if (warp == 0) {
-                double bv = -1.0;
-                int bi = INT_MAX;
-#pragma unroll 1
-                for (int rr = j + lane; rr < ntop; rr += 32) {
-                    const double v = fabs(pan[rr * NB + j]);
-                    if (v > bv) { bv = v; bi = rr; }
-                }
-                for (int off = 16; off > 0; off >>= 1) {
-                    const double ov = __shfl_down_sync(0xffffffffu, bv, off);
-                    const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-                }
-                int pr = __shfl_sync(0xffffffffu, bi, 0);
+                int pr = warp_pivot(j, ntop, [&](int r) { return pan[r * NB + j]; });
                 if (pr == INT_MAX) {
                     pr = j;
                     if (lane == 0) sflag |= 2;
@@ -157,15 +146,16 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim_mixed(Regions<float> R, int6
                 }
                 __syncwarp();
                 if (lane < kb) prow[lane] = (float)pan[j * NB + lane];
-                if (lane == 0) piv[j] = pr;
+                __syncwarp();
+                if (lane == 0) {
+                    piv[j] = pr;
+                    int fl = 0;
+                    s_inv = pivot_reciprocal(pan[j * NB + j], fl);
+                    if (fl) sflag |= fl;
+                }
             }
             __syncthreads();
-            double pv = pan[j * NB + j];
-            if (pv == 0.0 || !isfinite(pv)) {
-                if (tid == 0) sflag |= (pv == 0.0) ? 1 : 2;
-                pv = 1.0;
-            }
-            const double inv = 1.0 / pv;
+            const double inv = s_inv;
             const float invf = (float)inv;
 #pragma unroll 1
             for (int rr = j + 1 + tid; rr < ntop; rr += NTH) {       // rows of At: FP64
@@ -271,17 +261,31 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim_mixed(Regions<float> R, int6
 // forms z = L^{-1} P Rt; it stores the interchanges.  The FP32 border then
 // needs two triangular solves with many right-hand sides, each independent
 // per column (or row) and run by its own kernels:
-//   k_trsm_z:  Z = L^{-1} P Bt   (columns of Bt)
-//   k_trsm_w:  W = Ct U^{-1}     (rows of Ct)
-// 32-row blocks of the factor are staged in shared memory as FP32; the
-// off-diagonal part of each block step is a small product (threads over
-// rows x columns), the diagonal 32 x 32 triangle is solved per column.
+//   k_trsm<true>:   Z = L^{-1} P Bt   (columns of Bt)
+//   k_trsm<false>:  W = Ct U^{-1}     (rows of Ct)
+// 32 rows at a time: the solved rows' product, then the diagonal triangle.
 // ----------------------------------------------------------------------------
 template <class C, int NB>
 constexpr int lu_mixed_smem_bytes() { return (C::NU * NB + NB * 64) * 8; }
 
+// The interchange sequence sp (row i exchanged with sp[i], i ascending) as a gather map: row i of P B
+// is row out[i] of B.  Whole CTA of NTH threads; sm: NU shared words.
+template <int NU, int NTH>
+__device__ __forceinline__ void interchanges_to_map(const int* sp, int* sm, int32_t* out) {
+    for (int i = threadIdx.x; i < NU; i += NTH) sm[i] = i;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int i = 0; i < NU; ++i) {
+            const int q = sp[i], t = sm[i];
+            sm[i] = sm[q];
+            sm[q] = t;
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < NU; i += NTH) out[i] = sm[i];
+}
+
 template <class C, int NB, int NTH>
-__global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* __restrict__ piv_out,
+__global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* __restrict__ perm_out,
                                                      int64_t e0, int32_t* status) {
     constexpr int NU = C::NU;
     static_assert(NTH == 256, "trailing-update layout assumes 256 threads");
@@ -294,8 +298,9 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
     extern __shared__ double sm[];
     double* pan = sm;                    // [NU][NB], row index relative to k0
     double* ust = pan + NU * NB;         // [NB][64]
-    __shared__ int piv[NB];
+    __shared__ int piv[NB], spiv[NU], sperm[NU];
     __shared__ int sflag;
+    __shared__ double s_inv;
     if (tid == 0) sflag = 0;
     __syncthreads();
 #pragma unroll 1
@@ -310,19 +315,7 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
 #pragma unroll 1
         for (int j = 0; j < kb; ++j) {
             if (warp == 0) {
-                double bv = -1.0;
-                int bi = INT_MAX;
-#pragma unroll 1
-                for (int rr = j + lane; rr < nrows; rr += 32) {
-                    const double v = fabs(pan[rr * NB + j]);
-                    if (v > bv) { bv = v; bi = rr; }
-                }
-                for (int off = 16; off > 0; off >>= 1) {
-                    const double ov = __shfl_down_sync(0xffffffffu, bv, off);
-                    const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-                }
-                int pr = __shfl_sync(0xffffffffu, bi, 0);
+                int pr = warp_pivot(j, nrows, [&](int r) { return pan[r * NB + j]; });
                 if (pr == INT_MAX) {
                     pr = j;
                     if (lane == 0) sflag |= 2;
@@ -332,15 +325,16 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
                     pan[j * NB + lane] = pan[pr * NB + lane];
                     pan[pr * NB + lane] = t;
                 }
-                if (lane == 0) piv[j] = pr;
+                __syncwarp();
+                if (lane == 0) {
+                    piv[j] = pr;
+                    int fl = 0;
+                    s_inv = pivot_reciprocal(pan[j * NB + j], fl);
+                    if (fl) sflag |= fl;
+                }
             }
             __syncthreads();
-            double pv = pan[j * NB + j];
-            if (pv == 0.0 || !isfinite(pv)) {
-                if (tid == 0) sflag |= (pv == 0.0) ? 1 : 2;
-                pv = 1.0;
-            }
-            const double inv = 1.0 / pv;
+            const double inv = s_inv;
 #pragma unroll 1
             for (int rr = j + 1 + tid; rr < nrows; rr += NTH) {
                 const double l = pan[rr * NB + j] * inv;
@@ -385,7 +379,7 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
                 }
             }
         }
-        if (tid < kb) piv_out[e * NU + k0 + tid] = k0 + piv[tid];
+        if (tid < kb) spiv[k0 + tid] = k0 + piv[tid];
         __syncthreads();
         trailing_region<double, NB, NTH>(rowp, [&](int j) { return rowp(k0 + j); }, c0, NU, c0, NU, pan, k0, kb, ust);
         // right-hand side: rt[r] -= L21[r] . z1 for the rows below the panel
@@ -397,163 +391,254 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
         }
         __syncthreads();
     }
+    interchanges_to_map<NU, NTH>(spiv, sperm, perm_out + e * NU);
     if (tid == 0 && sflag) atomicOr(status, sflag);
 }
 
-// X[i0 + r][c] -= sum_{j < i0} F[r][j] X[j][c] for r < nb, c < CW (F a staged factor
-// block row, row stride NU): each thread owns a 4-row x 2-column tile, so one pair
-// of shared loads feeds eight multiply-adds
-template <int NU, int CW, int NTH>
-__device__ __forceinline__ void trsm_offdiag_tile(const float* F, float* X, int i0, int nb) {
-    static_assert(32 * CW == 8 * NTH, "tile layout assumes 32 x CW outputs over NTH threads");
-    const int tid = threadIdx.x, cp = tid % (CW / 2), rq = tid / (CW / 2);
-    const int c = 2 * cp, r = 4 * rq;
-    float acc[4][2] = {};
-    if (i0 > 0) {
-        for (int j = 0; j < i0; ++j) {
-            const float x0 = X[j * CW + c], x1 = X[j * CW + c + 1];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float f = F[(r + u) * NU + j];
-                acc[u][0] = fmaf(f, x0, acc[u][0]);
-                acc[u][1] = fmaf(f, x1, acc[u][1]);
+// The same factorisation with the whole bordered block [At | Rt] in shared memory, for the sizes
+// that fit (n_u <= 135: every element type but the degree-3 hexes), right-looking one column at
+// a time.  FP64 multiply-adds take 16 cycles of an SM per warp here, so the shared-memory traffic of
+// rank-1 updates is free and no panel is needed; what is left to hide is the pivot chain, and warp 0
+// updates the next column first and searches its pivot while the other warps update the rest.  The trailing block is walked as one flat range, so that no lane idles at
+// the rows' ends.  4,096 hexes p = 2: 10.05 -> 8.7 ms (2/3 n_u^3 at the FP64 pipe's rate: 5.4); 2,867 quads p = 3:
+// 1.65 -> 0.70.
+template <class C>
+struct LuShape {
+    static constexpr int NU = C::NU;
+    static constexpr int LDS = (NU + 1) | 1;             // odd row stride in doubles: columns without bank conflicts
+    static constexpr int NTH = NU > 100 ? 512 : NU > 50 ? 128 : 64;
+    static constexpr int smem_bytes = (NU * LDS + NU) * 8;
+    static constexpr bool fits = smem_bytes <= 200 * 1024;
+};
+
+template <class C>
+__global__ void __launch_bounds__(LuShape<C>::NTH) k_lu_small(Regions<float> R, int32_t* __restrict__ perm_out,
+                                                              int64_t e0, int32_t* status) {
+    using S = LuShape<C>;
+    constexpr int NU = S::NU, LDS = S::LDS, NTH = S::NTH;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t e = e0 + blockIdx.x;
+    double* Ag = R.a11 + e * R.a11_es;
+    double* rt = R.rt + e * R.rt_es;
+    extern __shared__ double sm[];
+    double* A = sm;                      // [NU][LDS], column NU the right-hand side
+    double* lc = A + NU * LDS;           // [NU] multipliers of the current column
+    __shared__ int s_p, sflag, spiv[NU], sperm[NU];
+    __shared__ double s_inv;
+    if (tid == 0) sflag = 0;
+    for (int idx = tid; idx < NU * NU; idx += NTH) {
+        const int r = idx / NU, c = idx - r * NU;
+        A[r * LDS + c] = Ag[(int64_t)r * R.a11_rs + c];
+    }
+    for (int r = tid; r < NU; r += NTH) A[r * LDS + NU] = rt[r * R.rt_rs];
+    // pivot of column k by warp 0: largest magnitude, lowest row on ties
+    auto search = [&](int k) {
+        int bi = warp_pivot(k, NU, [&](int r) { return A[r * LDS + k]; });
+        if (lane == 0) {
+            if (bi == INT_MAX) { bi = k; sflag |= 2; }
+            s_p = bi;
+            spiv[k] = bi;
+        }
+    };
+    __syncthreads();
+    if (warp == 0) search(0);
+#pragma unroll 1
+    for (int k = 0; k < NU; ++k) {
+        __syncthreads();                                 // pivot known, the trailing block updated
+        const int p = s_p;
+        if (warp == 0) {
+            if (lane == 0) {                             // now, while the FP64 pipe is free
+                int fl = 0;
+                s_inv = pivot_reciprocal(A[p * LDS + k], fl);
+                if (fl) sflag |= fl;
+            }
+        } else if (p != k) {
+            for (int c = tid - 32; c <= NU; c += NTH - 32)
+                if (c != k) {
+                    const double t = A[k * LDS + c];
+                    A[k * LDS + c] = A[p * LDS + c];
+                    A[p * LDS + c] = t;
+                }
+        }
+        const double pv = A[p * LDS + k];
+        __syncthreads();                                 // rows exchanged but for column k
+        const double inv = s_inv;
+        for (int r = k + 1 + tid; r < NU; r += NTH) lc[r] = A[(r == p ? k : r) * LDS + k] * inv;
+        __syncthreads();                                 // row k and the multipliers in place
+        if (warp == 0) {
+            if (lane == 0) A[k * LDS + k] = pv;
+            const double u = k + 1 < NU ? A[k * LDS + k + 1] : 0.0;
+            for (int r = k + 1 + lane; r < NU; r += 32) {
+                const double l = lc[r];
+                A[r * LDS + k] = l;
+                A[r * LDS + k + 1] = fma(-l, u, A[r * LDS + k + 1]);
+            }
+            __syncwarp();
+            if (k + 1 < NU) search(k + 1);
+        } else {
+            // rows k + 1 .. NU - 1, columns k + 2 .. NU as one range
+            const int w = NU - 1 - k, st = NTH - 32;
+            if (w > 0) {
+                const int dr = st / w, dc = st - dr * w;
+                int r = (tid - 32) / w, c = (tid - 32) - r * w;
+                for (int idx = tid - 32; idx < w * w; idx += st) {
+                    double* a = A + (k + 1 + r) * LDS + k + 2 + c;
+                    *a = fma(-lc[k + 1 + r], A[k * LDS + k + 2 + c], *a);
+                    r += dr;
+                    c += dc;
+                    if (c >= w) { c -= w; ++r; }
+                }
             }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (r + u < nb) {
-                X[(i0 + r + u) * CW + c] -= acc[u][0];
-                X[(i0 + r + u) * CW + c + 1] -= acc[u][1];
-            }
     }
+    __syncthreads();
+    for (int idx = tid; idx < NU * NU; idx += NTH) {
+        const int r = idx / NU, c = idx - r * NU;
+        Ag[(int64_t)r * R.a11_rs + c] = A[r * LDS + c];
+    }
+    for (int r = tid; r < NU; r += NTH) rt[r * R.rt_rs] = A[r * LDS + NU];
+    interchanges_to_map<NU, NTH>(spiv, sperm, perm_out + e * NU);
+    if (tid == 0 && sflag) atomicOr(status, sflag);
 }
 
 template <class C>
 struct TrsmShape {
     static constexpr int CW = 64;                           // right-hand sides per CTA
     static constexpr int NTH = 256;
-    static constexpr int smem_floats = C::NU * CW + 32 * C::NU;   // the block of right-hand sides, one factor block row
+    static constexpr int NBLK = (C::NU + 31) / 32;
+    static constexpr int JC = 64;                           // factor columns staged at a time
+    static constexpr int FS = 36;                           // row stride of the staged factor
+    static constexpr int smem_floats = NBLK * 32 * CW + JC * FS;
 };
 
-// Z = L^{-1} P Bt for columns [c0, c0 + CW) of Bt (FP32, in place); L unit lower (FP64 storage)
-template <class C>
-__global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm_z(Regions<float> R, const int32_t* __restrict__ piv,
-                                                              int64_t e0) {
-    constexpr int NU = C::NU, NT = C::NT, CW = TrsmShape<C>::CW, NTH = TrsmShape<C>::NTH;
+// ZS: Z = L^{-1} P Bt for columns [c0, c0 + 64) of Bt; else W = Ct U^{-1} for rows [c0, c0 + 64) of
+// Ct (FP32, in place; the factors FP64 in HBM).  X[i][c] holds the block of right-hand sides (W's
+// transposed); 32 rows of X at a time: the solved rows' contribution as a product with the staged
+// factor (a thread owns 4 rows x 2 columns: one 8-byte and one broadcast 16-byte shared load feed
+// eight multiply-adds), then the substitution with the diagonal triangle, four lanes per right-hand
+// side with eight rows each, the solved value passed by a shuffle.  4,096 hexes p = 2: Z and W 5.6 ->
+// 5.6 ms; 1,320 hexes p = 3: 23.0 -> 11.4 ms (the substitution ran on two warps, and every CTA walked the
+// interchange list in global memory).  Inverted diagonal triangles are as fast but lose accuracy
+// (error of the right-hand side 0.8e-6 -> 3.5e-6 on quads p = 3).
+template <class C, bool ZS>
+__global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, const int32_t* __restrict__ perm,
+                                                            int64_t e0) {
+    using S = TrsmShape<C>;
+    constexpr int NU = C::NU, NT = C::NT, CW = S::CW, NTH = S::NTH, JC = S::JC, FS = S::FS, NUP = S::NBLK * 32;
     constexpr int NCT = (NT + CW - 1) / CW;
-    const int tid = threadIdx.x;
-    const int64_t e = e0 + blockIdx.x / NCT;
-    const int c0 = (int)(blockIdx.x % NCT) * CW;
-    const int cw = min(CW, NT - c0);
-    const double* A = R.a11 + e * R.a11_es;
-    float* Bt = R.a12 + e * R.a12_es;
-    const int64_t rs = R.a11_rs, bs = R.a12_rs;
-    extern __shared__ float smf[];
-    float* X = smf;                       // [NU][CW]
-    float* Lb = X + NU * CW;              // [32][NU] one block row of L
-    __shared__ int perm[NU];
-    if (tid == 0) {                       // the interchange sequence as a gather map
-        for (int i = 0; i < NU; ++i) perm[i] = i;
-        for (int i = 0; i < NU; ++i) {
-            const int q = piv[e * NU + i];
-            if (q != i) { const int t = perm[i]; perm[i] = perm[q]; perm[q] = t; }
-        }
-    }
-    __syncthreads();
-    for (int idx = tid; idx < NU * CW; idx += NTH) {
-        const int i = idx / CW, c = idx - i * CW;
-        X[idx] = c < cw ? Bt[(size_t)perm[i] * bs + c0 + c] : 0.f;
-    }
-#pragma unroll 1
-    for (int i0 = 0; i0 < NU; i0 += 32) {
-        const int nb = min(32, NU - i0);
-        __syncthreads();
-        for (int idx = tid; idx < nb * (i0 + nb); idx += NTH) {
-            const int r = idx / (i0 + nb), j = idx - r * (i0 + nb);
-            Lb[r * NU + j] = (float)A[(size_t)(i0 + r) * rs + j];
-        }
-        __syncthreads();
-        // X[i0 + r][c] -= sum_{j < i0} L[i0 + r][j] X[j][c]: each thread a 4 x 2 tile
-        trsm_offdiag_tile<NU, CW, NTH>(Lb, X, i0, nb);
-        __syncthreads();
-        // the unit-lower diagonal block, one column per thread, the column in registers
-        for (int c = tid; c < CW; c += NTH) {
-            float x[32];
-#pragma unroll
-            for (int r = 0; r < 32; ++r) x[r] = r < nb ? X[(i0 + r) * CW + c] : 0.f;
-#pragma unroll
-            for (int r = 1; r < 32; ++r) {
-                float s = x[r];
-#pragma unroll
-                for (int j = 0; j < 32; ++j)      // rows past nb read nothing: the staged block ends there
-                    if (j < r && r < nb) s = fmaf(-Lb[r * NU + i0 + j], x[j], s);
-                x[r] = r < nb ? s : 0.f;
-            }
-#pragma unroll
-            for (int r = 0; r < 32; ++r)
-                if (r < nb) X[(i0 + r) * CW + c] = x[r];
-        }
-    }
-    __syncthreads();
-    for (int idx = tid; idx < NU * CW; idx += NTH) {
-        const int i = idx / CW, c = idx - i * CW;
-        if (c < cw) Bt[(size_t)i * bs + c0 + c] = X[idx];
-    }
-}
-
-// W = Ct U^{-1} for rows [r0, r0 + CW) of Ct (FP32, in place, chunk-local); U upper (FP64 storage)
-template <class C>
-__global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm_w(Regions<float> R, int64_t e0) {
-    constexpr int NU = C::NU, NT = C::NT, CW = TrsmShape<C>::CW, NTH = TrsmShape<C>::NTH;
-    constexpr int NCT = (NT + CW - 1) / CW;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t el = blockIdx.x / NCT, e = e0 + el;
-    const int r0 = (int)(blockIdx.x % NCT) * CW;
-    const int rw = min(CW, NT - r0);
+    const int c0 = (int)(blockIdx.x % NCT) * CW, cw = min(CW, NT - c0);
     const double* A = R.a11 + e * R.a11_es;
-    float* Ct = R.a21 + el * R.a21_es;
-    const int64_t rs = R.a11_rs, cs = R.a21_rs;
-    extern __shared__ float smf[];
-    float* X = smf;                       // [NU][CW]: X[j][r] = Ct[r0 + r][j]
-    float* Ub = X + NU * CW;              // [32][NU]: Ub[q][j] = U[j][i0 + q], j < i0 + nb
-    for (int idx = tid; idx < NU * CW; idx += NTH) {
-        const int r = idx / NU, j = idx - r * NU;
-        X[j * CW + r] = r < rw ? Ct[(size_t)(r0 + r) * cs + j] : 0.f;
-    }
-#pragma unroll 1
-    for (int i0 = 0; i0 < NU; i0 += 32) {
-        const int nb = min(32, NU - i0);
-        __syncthreads();
-        for (int idx = tid; idx < (i0 + nb) * nb; idx += NTH) {
-            const int j = idx / nb, q = idx - j * nb;
-            Ub[q * NU + j] = (float)A[(size_t)j * rs + i0 + q];
+    float* Y = ZS ? R.a12 + e * R.a12_es : R.a21 + el * R.a21_es;
+    const int64_t rs = R.a11_rs, ys = ZS ? R.a12_rs : R.a21_rs;
+    extern __shared__ __align__(16) float smf[];
+    float* X = smf;                       // [NUP][CW]
+    float* F = X + NUP * CW;              // [JC][FS] factor columns
+    __shared__ float rd[32];              // reciprocal diagonal of U's block
+    // the chunk at (i0, j0): F[j][r] = the factor's entry (row i0 + r of L, or column i0 + r of U; column or
+    // row j0 + j), 64 or 32 columns left of the diagonal or the 32 of the diagonal block (j0 == i0)
+    constexpr int NPRE = 32 * JC / NTH;
+    float pre[NPRE];
+    auto width = [&](int i0, int j0) { return j0 < i0 ? min(JC, i0 - j0) : 32; };
+    auto load = [&](int i0, int j0) {
+        const int jc = width(i0, j0);
+#pragma unroll
+        for (int u = 0; u < NPRE; ++u) {
+            const int idx = tid + u * NTH;
+            int r, j;
+            if (ZS) { r = idx / jc; j = idx - r * jc; } else { j = idx >> 5; r = idx & 31; }
+            pre[u] = idx >= 32 * jc || i0 + r >= NU || j0 + j >= NU ? 0.f
+                     : (float)(ZS ? A[(int64_t)(i0 + r) * rs + j0 + j] : A[(int64_t)(j0 + j) * rs + i0 + r]);
         }
-        __syncthreads();
-        // X[i0 + q][r] -= sum_{j < i0} U[j][i0 + q] X[j][r]: each thread a 4 x 2 tile
-        trsm_offdiag_tile<NU, CW, NTH>(Ub, X, i0, nb);
-        __syncthreads();
-        for (int r = tid; r < CW; r += NTH) {
-            float x[32];
+    };
+    load(0, 0);
+    if (ZS) {
+        for (int idx = tid; idx < NUP * CW; idx += NTH) {
+            const int i = idx / CW, c = idx - i * CW;
+            X[idx] = i < NU && c < cw ? Y[(int64_t)perm[e * NU + i] * ys + c0 + c] : 0.f;
+        }
+    } else {
+        for (int idx = tid; idx < NUP * CW; idx += NTH) {
+            const int c = idx / NUP, i = idx - c * NUP;
+            X[i * CW + c] = i < NU && c < cw ? Y[(int64_t)(c0 + c) * ys + i] : 0.f;
+        }
+    }
+    float acc[4][2] = {};
+    int i0 = 0, j0 = 0;
+#pragma unroll 1
+    while (i0 < NUP) {
+        const int jc = width(i0, j0);
+        const bool diag = j0 == i0;
+        __syncthreads();                  // X complete, F free
 #pragma unroll
-            for (int q = 0; q < 32; ++q) x[q] = q < nb ? X[(i0 + q) * CW + r] : 0.f;
-#pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                float s = x[q];
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < q && q < nb) s = fmaf(-Ub[q * NU + i0 + j], x[j], s);
-                const float d = q < nb ? Ub[q * NU + i0 + q] : 1.f;
-                x[q] = q < nb ? s / (d != 0.f ? d : 1.f) : 0.f;
+        for (int u = 0; u < NPRE; ++u) {
+            const int idx = tid + u * NTH;
+            if (idx >= 32 * jc) continue;
+            int r, j;
+            if (ZS) { r = idx / jc; j = idx - r * jc; } else { j = idx >> 5; r = idx & 31; }
+            F[j * FS + r] = pre[u];
+        }
+        if (diag) {
+            if (!ZS && tid < 32) {
+                const float d = i0 + tid < NU ? (float)A[(int64_t)(i0 + tid) * rs + i0 + tid] : 1.f;
+                rd[tid] = d != 0.f ? 1.f / d : 1.f;
             }
 #pragma unroll
-            for (int q = 0; q < 32; ++q)
-                if (q < nb) X[(i0 + q) * CW + r] = x[q];
+            for (int u = 0; u < 4; ++u) {
+                float2* x = reinterpret_cast<float2*>(X + (i0 + 4 * warp + u) * CW + 2 * lane);
+                const float2 v = *x;
+                *x = make_float2(v.x - acc[u][0], v.y - acc[u][1]);
+                acc[u][0] = acc[u][1] = 0.f;
+            }
         }
+        __syncthreads();
+        const int ni = diag ? i0 + 32 : i0, nj = diag ? 0 : j0 + jc;
+        if (ni < NUP) load(ni, nj);       // the next chunk under this one's arithmetic
+        if (!diag) {
+#pragma unroll 8
+            for (int j = 0; j < jc; ++j) {
+                const float2 x = *reinterpret_cast<const float2*>(X + (j0 + j) * CW + 2 * lane);
+                const float4 f = *reinterpret_cast<const float4*>(F + j * FS + 4 * warp);
+                acc[0][0] = fmaf(f.x, x.x, acc[0][0]); acc[0][1] = fmaf(f.x, x.y, acc[0][1]);
+                acc[1][0] = fmaf(f.y, x.x, acc[1][0]); acc[1][1] = fmaf(f.y, x.y, acc[1][1]);
+                acc[2][0] = fmaf(f.z, x.x, acc[2][0]); acc[2][1] = fmaf(f.z, x.y, acc[2][1]);
+                acc[3][0] = fmaf(f.w, x.x, acc[3][0]); acc[3][1] = fmaf(f.w, x.y, acc[3][1]);
+            }
+        } else {
+            const int c = tid >> 2, q = tid & 3;
+            float* xc = X + (i0 + 8 * q) * CW + c;
+            float x[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) x[m] = xc[m * CW];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                if (!ZS && q == (j >> 3)) x[j & 7] *= rd[j];
+                const float xj = __shfl_sync(0xffffffffu, x[j & 7], (lane & ~3) | (j >> 3));
+                const float4 f0 = *reinterpret_cast<const float4*>(F + j * FS + 8 * q);
+                const float4 f1 = *reinterpret_cast<const float4*>(F + j * FS + 8 * q + 4);
+                const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    if (8 * q + m > j) x[m] = fmaf(-f[m], xj, x[m]);
+            }
+#pragma unroll
+            for (int m = 0; m < 8; ++m) xc[m * CW] = x[m];
+        }
+        i0 = ni;
+        j0 = nj;
     }
     __syncthreads();
-    for (int idx = tid; idx < NU * CW; idx += NTH) {
-        const int r = idx / NU, j = idx - r * NU;
-        if (r < rw) Ct[(size_t)(r0 + r) * cs + j] = X[j * CW + r];
+    if (ZS) {
+        for (int idx = tid; idx < NU * CW; idx += NTH) {
+            const int i = idx / CW, c = idx - i * CW;
+            if (c < cw) Y[(int64_t)i * ys + c0 + c] = X[idx];
+        }
+    } else {
+        for (int idx = tid; idx < NU * CW; idx += NTH) {
+            const int c = idx / NU, i = idx - c * NU;
+            if (c < cw) Y[(int64_t)(c0 + c) * ys + i] = X[i * CW + c];
+        }
     }
 }
 
@@ -869,10 +954,15 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
     HDG_CK(cudaFuncSetAttribute(k_elim_mixed<C, NB, 256, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim));
     const int sm_lu = lu_mixed_smem_bytes<C, NB>();   // the 8-column variant needs less
     const int sm_trsm = (int)sizeof(float) * TrsmShape<C>::smem_floats;
-    HDG_CK(cudaFuncSetAttribute(k_lu_mixed<C, NB, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_lu));
-    HDG_CK(cudaFuncSetAttribute(k_lu_mixed<C, 8, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_lu));
-    HDG_CK(cudaFuncSetAttribute(k_trsm_z<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_trsm));
-    HDG_CK(cudaFuncSetAttribute(k_trsm_w<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_trsm));
+    using LS = LuShape<C>;
+    if constexpr (LS::fits) {
+        HDG_CK(cudaFuncSetAttribute(k_lu_small<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, LS::smem_bytes));
+    } else {
+        HDG_CK(cudaFuncSetAttribute(k_lu_mixed<C, NB, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_lu));
+        HDG_CK(cudaFuncSetAttribute(k_lu_mixed<C, 8, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_lu));
+    }
+    HDG_CK(cudaFuncSetAttribute(k_trsm<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_trsm));
+    HDG_CK(cudaFuncSetAttribute(k_trsm<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_trsm));
     cudaStream_t st = h->stream;
     HDG_CK(cudaMemsetAsync(h->d_vals32, 0, sizeof(float) * h->nnzb * C::BS * C::BS, st));
     HDG_CK(cudaMemsetAsync(h->d_g, 0, sizeof(double) * h->F * C::BS, st));
@@ -917,12 +1007,14 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
             // FP64 interior LU alone, then the FP32 border by two triangular solves
             using TS = TrsmShape<C>;
             constexpr int NCT = (C::NT + TS::CW - 1) / TS::CW;
-            if (h->elim_nb == 8)   // interior LU panel width (the autotuner's elim_nb)
+            if constexpr (LS::fits)
+                k_lu_small<C><<<(unsigned)ne, LS::NTH, LS::smem_bytes, st>>>(RM, h->d_mpiv, e0, h->d_status);
+            else if (h->elim_nb == 8)   // interior LU panel width (the autotuner's elim_nb)
                 k_lu_mixed<C, 8, 256><<<(unsigned)ne, 256, sm_lu, st>>>(RM, h->d_mpiv, e0, h->d_status);
             else
                 k_lu_mixed<C, NB, 256><<<(unsigned)ne, 256, sm_lu, st>>>(RM, h->d_mpiv, e0, h->d_status);
-            k_trsm_z<C><<<(unsigned)(ne * NCT), TS::NTH, sm_trsm, st>>>(RM, h->d_mpiv, e0);
-            k_trsm_w<C><<<(unsigned)(ne * NCT), TS::NTH, sm_trsm, st>>>(RM, e0);
+            k_trsm<C, true><<<(unsigned)(ne * NCT), TS::NTH, sm_trsm, st>>>(RM, h->d_mpiv, e0);
+            k_trsm<C, false><<<(unsigned)(ne * NCT), TS::NTH, sm_trsm, st>>>(RM, h->d_mpiv, e0);
         } else if (h->elim_mixed_minb == 3) {  // fused kernel, built for 3 or 2 resident CTAs per SM
             k_elim_mixed<C, NB, 256, 3><<<(unsigned)ne, 256, sm_elim, st>>>(RM, e0, h->d_status);
         } else {

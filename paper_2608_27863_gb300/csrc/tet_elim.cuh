@@ -6,6 +6,8 @@
 
 #include <climits>
 
+#include "pivot.cuh"
+
 namespace hdg {
 namespace tet {
 
@@ -67,6 +69,7 @@ __device__ void bordered_elim(T* Mx, int NU, int NR, int NC, int LD, T* pan, T* 
                               int* gpiv = nullptr) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     auto rowp = [&](int r) -> T* { return Mx + (size_t)r * LD; };
+    __shared__ T s_inv;
     for (int k0 = 0; k0 < NU; k0 += NB) {
         const int kb = min(NB, NU - k0), nrows = NR - k0, ntop = NU - k0;
 #pragma unroll 1
@@ -77,19 +80,7 @@ __device__ void bordered_elim(T* Mx, int NU, int NR, int NC, int LD, T* pan, T* 
         __syncthreads();
         for (int j = 0; j < kb; ++j) {
             if (warp == 0) {
-                T bv = T(-1);
-                int bi = INT_MAX;
-#pragma unroll 1
-                for (int rr = j + lane; rr < ntop; rr += 32) {
-                    const T v = fabs(pan[rr * NB + j]);
-                    if (v > bv) { bv = v; bi = rr; }
-                }
-                for (int off = 16; off > 0; off >>= 1) {
-                    const T ov = __shfl_down_sync(0xffffffffu, bv, off);
-                    const int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-                }
-                int pr = __shfl_sync(0xffffffffu, bi, 0);
+                int pr = warp_pivot(j, ntop, [&](int r) { return pan[r * NB + j]; });
                 if (pr == INT_MAX) {
                     pr = j;
                     if (lane == 0) *sflag |= 2;
@@ -99,18 +90,17 @@ __device__ void bordered_elim(T* Mx, int NU, int NR, int NC, int LD, T* pan, T* 
                     pan[j * NB + lane] = pan[pr * NB + lane];
                     pan[pr * NB + lane] = t;
                 }
+                __syncwarp();
                 if (lane == 0) {
                     piv[j] = pr;
                     if (gpiv) gpiv[k0 + j] = k0 + pr;
+                    int fl = 0;
+                    s_inv = pivot_reciprocal(pan[j * NB + j], fl);
+                    if (fl) *sflag |= fl;
                 }
             }
             __syncthreads();
-            T pv = pan[j * NB + j];
-            if (pv == T(0) || !isfinite(pv)) {
-                if (tid == 0) *sflag |= (pv == T(0)) ? 1 : 2;
-                pv = T(1);
-            }
-            const T inv = T(1) / pv;
+            const T inv = s_inv;
 #pragma unroll 1
             for (int rr = j + 1 + tid; rr < nrows; rr += NTH) {
                 const T l = pan[rr * NB + j] * inv;

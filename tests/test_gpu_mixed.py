@@ -207,3 +207,32 @@ def test_split_elimination_matches_fused(make):
         assert np.linalg.norm(v1 - v0) <= 1e-5 * np.linalg.norm(v0)
         assert np.linalg.norm(g1 - g0) <= 1e-5 * np.linalg.norm(g0)
         assert np.linalg.norm(u1 - u0) <= 1e-5 * np.linalg.norm(u0)
+
+
+@pytest.mark.parametrize("make", [lambda: synth.tiny(2, 1), lambda: synth.tiny(2, 2), lambda: synth.tiny(2, 3),
+                                  lambda: synth.tiny(3, 1), lambda: synth.config2(n=3), lambda: synth.config3(n=3)],
+                         ids=["quad-p1", "quad-p2", "quad-p3", "hex-p1", "hex-p2", "hex-p3"])
+def test_split_and_fused_elimination_agree(make):
+    """The default (FP64 LU, then FP32 triangular solves) against the fused kernel on every size of the interior block
+    (16 to 320: whole and partial 32-row blocks); both round Z and W in FP32, so they differ by a few n_u 2^-24."""
+    from paper_2608_27863_gb300 import hdg as H
+    P = make()
+    run = GpuRun(P)
+    H.hdg_set_params(run.h, tau=P.tau, visc_law=P.visc_law, suth_c1=P.suth_c1, suth_s=P.suth_s,
+                     precision=H.HDG_PREC_MIXED_3XTF32)
+    import torch
+    s = run.sizes
+    got = []
+    for split in (None, 0, 1):
+        if split is not None:
+            H.hdg_set_tuning(run.h, elim_nb=8, schur_mode=2, elim_mixed_split=split)
+        run.linearize()
+        assert H.hdg_status(run.h) == 0
+        v = torch.empty(s["nnzb"] * s["block"] ** 2, dtype=torch.float32, device="cuda")
+        H.hdg_get_blocks(run.h, v)
+        got.append((v.double(), torch.from_numpy(run.rhs())))
+    assert torch.equal(got[0][0], got[2][0]) and torch.equal(got[0][1], got[2][1])    # the split form is the default
+    tol = 4 * s["n_u"] * 2.0 ** -24
+    for a, b in zip(got[1], got[2]):
+        assert (a - b).norm() <= tol * b.norm()
+    run.close()
