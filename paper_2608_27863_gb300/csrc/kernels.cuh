@@ -129,15 +129,32 @@ template <class S> __device__ __forceinline__ const PhysT<S>& jac_phys(const Poi
 template <> __device__ __forceinline__ const PhysT<double>& jac_phys<double>(const PointArgs& A) { return A.ph; }
 template <> __device__ __forceinline__ const PhysT<float>& jac_phys<float>(const PointArgs& A) { return A.phf; }
 
+// Points are taken PB at a time.  First every (point, component) pair interpolates its values into shared
+// memory, then every (point, column b) pair evaluates the Jacobian column and one more role per point the
+// residual fluxes, so that a point's serial chain is one column's instead of all of them: small
+// meshes are bound by that chain (64 quads p = 2: 122 -> 44 us), large ones by the FP64 pipe (693 hexes
+// p = 1 1.12 -> 0.72 ms; 512 hexes p = 2 1.01 -> 0.89 ms; mixed form, 4,096 hexes p = 2 2.38 -> 2.20 ms).  The viscous flux is linear in q with a short
+// closed form per unit gradient, where evaluating it for all D M unit gradients was most of the arithmetic.
+template <class C>
+struct PointShape {
+    static constexpr int NTH = (C::M + 1) * 32;
+    static constexpr int PB = C::D == 3 ? 64 : 32;
+    static constexpr int PVS = (C::M * (2 + C::D) + 2) | 1;        // u, lifted q, uhat, nu, tau of one point (FP64)
+    static constexpr int PJS = (C::M * (2 + C::D) + 1) | 1;        // u, q, uhat, nu in the Jacobian's type
+};
+
 template <class C>
 constexpr int point_smem_doubles() {
-    return C::NU + 2 * C::NQV + C::NP + 2 * C::NT + C::D * C::M * C::NQ + 2 * C::NF * C::M * C::NFQ;
+    return C::NU + 2 * C::NQV + C::NP + 2 * C::NT + C::D * C::M * C::NQ + 2 * C::NF * C::M * C::NFQ +
+           PointShape<C>::PB * (PointShape<C>::PVS + PointShape<C>::PJS);
 }
 
-template <class C, int NTH, class TJ>
-__global__ void __launch_bounds__(NTH) k_point(PointArgs A) {
+template <class C, class TJ>
+__global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
+    constexpr int NTH = PointShape<C>::NTH, PB = PointShape<C>::PB, PVS = PointShape<C>::PVS, PJS = PointShape<C>::PJS;
     constexpr int D = C::D, M = C::M, NP = C::NP, NQ = C::NQ, NF = C::NF, NFP = C::NFP, NFQ = C::NFQ;
-    constexpr int NU = C::NU, NQV = C::NQV, NT = C::NT, NCOEF = C::NCOEF;
+    constexpr int NU = C::NU, NQV = C::NQV, NT = C::NT, NCOEF = C::NCOEF, NPT = NQ + NF * NFQ;
+    constexpr int OG = M, OH = M + M * D, ON = 2 * M + M * D, OT = ON + 1;   // offsets in a point's values: gradient, uhat, nu, tau
     constexpr int GEO = Geo<D>::N;
     const int tid = threadIdx.x;
     const int64_t el = blockIdx.x, e = A.e0 + el;
@@ -151,7 +168,16 @@ __global__ void __launch_bounds__(NTH) k_point(PointArgs A) {
     double* sFH = sFres + D * M * NQ;    // [nf][m][Nfq]
     double* sRh = sFH + NF * M * NFQ;    // [nf][m][Nfp]
     double* sFB = sRh + NT;              // [nf][m][Nfq] boundary form bhat (boundary faces)
+    double* sPV = sFB + NF * M * NFQ;    // [PB][PVS] values at the points of the batch (gradient: lifted)
+    TJ* sPJ = reinterpret_cast<TJ*>(sPV + PB * PVS);   // [PB][PJS] the same for the Jacobian (gradient: Q)
+    __shared__ double fnrm[NF], fnh[NF][D], s_hinv;     // face normals: length, direction; 1 / h
     __shared__ double geo[GEO];
+    // directions a flux can be taken along: the rows of Jinv (volume points), the face normals NW, and the
+    // lifting directions NW / detJ; their inner products with the directions of the q variation
+    constexpr int ND = D + NF;
+    __shared__ TJ sA[ND][D];             // rows of Jinv, then NW
+    __shared__ TJ sB[ND][D];             // rows of Jinv, then NW / detJ
+    __shared__ TJ sAB[ND][ND];           // sA . sB
     const DeviceTables& T = A.tab;
 
     for (int i = tid; i < NU; i += NTH) sU[i] = A.U[e * NU + i];
@@ -199,177 +225,207 @@ __global__ void __launch_bounds__(NTH) k_point(PointArgs A) {
     const PhysT<double>& ph = A.ph;
     const PhysT<TJ>& pj = jac_phys<TJ>(A);
     TJ* vc = reinterpret_cast<TJ*>(A.vcoef) + el * (size_t)(M * M * D * NCOEF * NQ);
-    TJ Jj[D * D], NWj[NF * D];
-    for (int i = 0; i < D * D; ++i) Jj[i] = (TJ)Jinv[i];
-    for (int i = 0; i < NF * D; ++i) NWj[i] = (TJ)(NW[i] / detJ);
-    // volume points
-    for (int g = tid; g < NQ; g += NTH) {
-        double u[M], q[M][D], ql[M][D], nuv = 0.0;
-        for (int a = 0; a < M; ++a) { u[a] = 0.0; for (int l = 0; l < D; ++l) { q[a][l] = 0.0; ql[a][l] = 0.0; } }
-        for (int j = 0; j < NP; ++j) {
-            double w = T.phi[g * NP + j];
-            nuv += w * sNu[j];
-            for (int a = 0; a < M; ++a) {
-                u[a] += w * sU[a * NP + j];
-                for (int l = 0; l < D; ++l) {
-                    q[a][l] += w * sQ[(l * M + a) * NP + j];
-                    ql[a][l] += w * sQL[(l * M + a) * NP + j];
-                }
-            }
-        }
-        const double wJ = -A.dt * T.wq[g] * detJ;
-        {
-            double Fc[M][D], Fv[M][D];
-            conv_flux<D, double, double>(u, ph, Fc);
-            visc_flux<D, double, double>(u, ql, nuv, ph, Fv);
-            for (int r = 0; r < D; ++r)
-                for (int a = 0; a < M; ++a) {
-                    double s = 0.0;
-                    for (int k = 0; k < D; ++k) s += Jinv[r * D + k] * (Fc[a][k] - Fv[a][k]);
-                    sFres[(r * M + a) * NQ + g] = wJ * s;
-                }
-        }
-        // Jacobian coefficients in TJ
-        TJ uj[M], qj[M][D];
-        for (int a = 0; a < M; ++a) { uj[a] = (TJ)u[a]; for (int l = 0; l < D; ++l) qj[a][l] = (TJ)q[a][l]; }
-        const TJ nuj = (TJ)nuv, wJj = (TJ)wJ;
-        for (int b = 0; b < M; ++b) {
-            DirT<TJ> ud[M];
-            for (int a = 0; a < M; ++a) ud[a] = {uj[a], a == b ? TJ(1) : TJ(0)};
-            DirT<TJ> Fc[M][D], Fv[M][D];
-            conv_flux<D, DirT<TJ>, TJ>(ud, pj, Fc);
-            visc_flux<D, DirT<TJ>, TJ>(ud, qj, nuj, pj, Fv);
-            for (int a = 0; a < M; ++a)
-                for (int r = 0; r < D; ++r) {
-                    TJ s = 0;
-                    for (int k = 0; k < D; ++k) s += Jj[r * D + k] * (Fc[a][k].t - Fv[a][k].t);
-                    vc[((((size_t)a * M + b) * D + r) * NCOEF + 0) * NQ + g] = wJj * s;
-                }
-        }
-        for (int b = 0; b < M; ++b) {
-            TJ cq[D][M][D];
-            for (int l = 0; l < D; ++l) {
-                TJ qe[M][D];
-                for (int a = 0; a < M; ++a) for (int k = 0; k < D; ++k) qe[a][k] = (a == b && k == l) ? TJ(1) : TJ(0);
-                TJ Fv[M][D];
-                visc_flux<D, TJ, TJ>(uj, qe, nuj, pj, Fv);
-                for (int r = 0; r < D; ++r)
-                    for (int a = 0; a < M; ++a) {
-                        TJ s = 0;
-                        for (int k = 0; k < D; ++k) s += Jj[r * D + k] * Fv[a][k];
-                        cq[r][a][l] = -wJj * s;
-                    }
-            }
-            for (int a = 0; a < M; ++a)
-                for (int r = 0; r < D; ++r) {
-                    TJ* o = vc + ((((size_t)a * M + b) * D + r) * NCOEF) * NQ + g;
-                    for (int r2 = 0; r2 < D; ++r2) {
-                        TJ s = 0;
-                        for (int l = 0; l < D; ++l) s += cq[r][a][l] * Jj[r2 * D + l];
-                        o[(1 + r2) * NQ] = s;
-                    }
-                    for (int f = 0; f < NF; ++f) {
-                        TJ s = 0;
-                        for (int l = 0; l < D; ++l) s += cq[r][a][l] * NWj[f * D + l];
-                        o[(1 + D + f) * NQ] = s;
-                    }
-                }
-        }
-    }
-    // face points
     TJ* fc = reinterpret_cast<TJ*>(A.fcoef) + el * (size_t)(NF * M * M * NCOEF * NFQ);
-    for (int fs = tid; fs < NF * NFQ; fs += NTH) {
-        const int f = fs / NFQ, s = fs - f * NFQ;
-        double u[M], uh[M], q[M][D], ql[M][D], nuv = 0.0;
-        for (int a = 0; a < M; ++a) { u[a] = 0.0; uh[a] = 0.0; for (int l = 0; l < D; ++l) { q[a][l] = 0.0; ql[a][l] = 0.0; } }
-        for (int lam = 0; lam < NFP; ++lam) {
-            double w = T.mu[s * NFP + lam];
-            int j = T.fnode[f * NFP + lam];
-            nuv += w * sNu[j];
-            for (int a = 0; a < M; ++a) {
-                u[a] += w * sU[a * NP + j];
-                uh[a] += w * sUH[(f * M + a) * NFP + lam];
-                for (int l = 0; l < D; ++l) {
-                    q[a][l] += w * sQ[(l * M + a) * NP + j];
-                    ql[a][l] += w * sQL[(l * M + a) * NP + j];
-                }
-            }
-        }
-        const double* nw = NW + f * D;
-        double nrm = 0.0;
-        for (int k = 0; k < D; ++k) nrm += nw[k] * nw[k];
-        nrm = sqrt(nrm);
-        const double ws = T.wf[s];
-        double nh[D];
-        for (int k = 0; k < D; ++k) nh[k] = nw[k] / nrm;
-        const double hinv = A.tau_mode ? 1.0 / pow(double(1 << D) * detJ, 1.0 / D) : 0.0;   // |K|^{-1/d}
-        const double tau_s = A.tau_mode ? stab_tau<D, double, double>(uh, nh, hinv, ph) : A.tau;
-        if (A.taup) A.taup[(el * NF + f) * NFQ + s] = tau_s;
-        {
-            double Fc[M][D], Fv[M][D];
-            conv_flux<D, double, double>(uh, ph, Fc);
-            visc_flux<D, double, double>(uh, ql, nuv, ph, Fv);
-            const int tag = A.ftag ? A.ftag[e * NF + f] : 0;
-            for (int a = 0; a < M; ++a) {
-                double fn = 0.0;
-                for (int k = 0; k < D; ++k) fn += (Fc[a][k] - Fv[a][k]) * nw[k];
-                const double fh = ws * (fn + nrm * tau_s * (u[a] - uh[a]));
-                sFH[(f * M + a) * NFQ + s] = fh;
-                const double ub_a = tag == 1 ? boundary_state<NF, M, NFP>(A.ub, A.ubf, A.e2f, A.perm, T.mu, e, f, s, a) : 0.0;
-                sFB[(f * M + a) * NFQ + s] = boundary_form<M>(tag, a, fh, ws * nrm, u, uh, ub_a, A.ew);
-            }
-        }
-        TJ uhj[M], qj[M][D], nwj[D];
-        for (int a = 0; a < M; ++a) { uhj[a] = (TJ)uh[a]; for (int l = 0; l < D; ++l) qj[a][l] = (TJ)q[a][l]; }
-        for (int k = 0; k < D; ++k) nwj[k] = (TJ)nw[k];
-        const TJ nuj = (TJ)nuv, wsj = (TJ)ws, taun = (TJ)(nrm * tau_s);
-        TJ nhj[D];
-        for (int k = 0; k < D; ++k) nhj[k] = (TJ)nh[k];
-        for (int b = 0; b < M; ++b) {
-            DirT<TJ> ud[M];
-            for (int a = 0; a < M; ++a) ud[a] = {uhj[a], a == b ? TJ(1) : TJ(0)};
-            DirT<TJ> Fc[M][D], Fv[M][D];
-            conv_flux<D, DirT<TJ>, TJ>(ud, pj, Fc);
-            visc_flux<D, DirT<TJ>, TJ>(ud, qj, nuj, pj, Fv);
-            // d tau / d uhat_b (state-dependent stabilization): (u_a - uhat_a) |nw| d tau / d uhat_b
-            const TJ dtau = A.tau_mode ? (TJ)nrm * stab_tau<D, DirT<TJ>, TJ>(ud, nhj, (TJ)hinv, pj).t : TJ(0);
-            for (int a = 0; a < M; ++a) {
-                TJ fn = 0;
-                for (int k = 0; k < D; ++k) fn += (Fc[a][k].t - Fv[a][k].t) * nwj[k];
-                if (a == b) fn -= taun;
-                fn += ((TJ)u[a] - uhj[a]) * dtau;
-                fc[((((size_t)f * M + a) * M + b) * NCOEF + 0) * NFQ + s] = wsj * fn;
-            }
-        }
-        for (int b = 0; b < M; ++b) {
-            TJ qh[M][D];
-            for (int l = 0; l < D; ++l) {
-                TJ qe[M][D];
-                for (int a = 0; a < M; ++a) for (int k = 0; k < D; ++k) qe[a][k] = (a == b && k == l) ? TJ(1) : TJ(0);
-                TJ Fv[M][D];
-                visc_flux<D, TJ, TJ>(uhj, qe, nuj, pj, Fv);
-                for (int a = 0; a < M; ++a) {
-                    TJ fn = 0;
-                    for (int k = 0; k < D; ++k) fn += Fv[a][k] * nwj[k];
-                    qh[a][l] = -wsj * fn;
-                }
-            }
-            for (int a = 0; a < M; ++a) {
-                TJ* o = fc + ((((size_t)f * M + a) * M + b) * NCOEF) * NFQ + s;
-                for (int r2 = 0; r2 < D; ++r2) {
-                    TJ t = 0;
-                    for (int l = 0; l < D; ++l) t += qh[a][l] * Jj[r2 * D + l];
-                    o[(1 + r2) * NFQ] = t;
-                }
-                for (int f2 = 0; f2 < NF; ++f2) {
-                    TJ t = 0;
-                    for (int l = 0; l < D; ++l) t += qh[a][l] * NWj[f2 * D + l];
-                    o[(1 + D + f2) * NFQ] = t;
-                }
-            }
-        }
+    for (int i = tid; i < ND * D; i += NTH) {
+        const int n = i / D, k = i - n * D;
+        const double v = n < D ? Jinv[n * D + k] : NW[(n - D) * D + k];
+        sA[n][k] = (TJ)v;
+        sB[n][k] = (TJ)(n < D ? v : v / detJ);
+    }
+    if (tid < NF) {
+        double v = 0.0;
+        for (int k = 0; k < D; ++k) v += NW[tid * D + k] * NW[tid * D + k];
+        v = sqrt(v);
+        fnrm[tid] = v;
+        for (int k = 0; k < D; ++k) fnh[tid][k] = NW[tid * D + k] / v;
+        if (tid == 0) s_hinv = A.tau_mode ? 1.0 / pow(double(1 << D) * detJ, 1.0 / D) : 0.0;   // |K|^{-1/d}
     }
     __syncthreads();
+    for (int i = tid; i < ND * ND; i += NTH) {
+        TJ v = 0;
+        for (int k = 0; k < D; ++k) v += sA[i / ND][k] * sB[i % ND][k];
+        sAB[i / ND][i % ND] = v;
+    }
+    for (int x0 = 0; x0 < NPT; x0 += PB) {
+        const int nx = min(PB, NPT - x0);
+        // values at the points: items (component or nu, point), points fastest
+        for (int it = tid; it < (M + 1) * PB; it += NTH) {
+            const int a = it / PB, xl = it - a * PB, x = x0 + xl;
+            if (xl >= nx) continue;
+            double* o = sPV + xl * PVS;
+            TJ* oj = sPJ + xl * PJS;
+            const bool vol = x < NQ;
+            const int f = vol ? 0 : (x - NQ) / NFQ, s = vol ? 0 : x - NQ - f * NFQ;
+            const double* w = vol ? T.phi + (size_t)x * NP : T.mu + (size_t)s * NFP;
+            const int n = vol ? NP : NFP;
+            if (a == M) {
+                double v = 0.0;
+                if (A.nu)
+                    for (int j = 0; j < n; ++j) v += w[j] * sNu[vol ? j : T.fnode[f * NFP + j]];
+                o[ON] = v;
+                o[OT] = A.tau;
+                oj[ON] = (TJ)v;
+                continue;
+            }
+            double u = 0.0, uh = 0.0, q[D], ql[D];
+            for (int l = 0; l < D; ++l) { q[l] = 0.0; ql[l] = 0.0; }
+            for (int j = 0; j < n; ++j) {
+                const double wj = w[j];
+                const int nd = vol ? j : T.fnode[f * NFP + j];
+                u += wj * sU[a * NP + nd];
+                if (!vol) uh += wj * sUH[(f * M + a) * NFP + j];
+#pragma unroll
+                for (int l = 0; l < D; ++l) {
+                    q[l] += wj * sQ[(l * M + a) * NP + nd];
+                    ql[l] += wj * sQL[(l * M + a) * NP + nd];
+                }
+            }
+            o[a] = u;
+            o[OH + a] = uh;
+            oj[a] = (TJ)u;
+            oj[OH + a] = (TJ)uh;
+#pragma unroll
+            for (int l = 0; l < D; ++l) { o[OG + a * D + l] = ql[l]; oj[OG + a * D + l] = (TJ)q[l]; }
+        }
+        __syncthreads();
+        if (A.tau_mode) {
+            for (int xl = tid; xl < nx; xl += NTH)
+                if (x0 + xl >= NQ) {
+                    const int f = (x0 + xl - NQ) / NFQ;
+                    double* o = sPV + xl * PVS;
+                    o[OT] = stab_tau<D, double, double>(o + OH, fnh[f], s_hinv, ph);
+                }
+            __syncthreads();
+        }
+        // items (role, point): role b < M the Jacobian column b, role M the residual fluxes
+        for (int it = tid; it < (M + 1) * PB; it += NTH) {
+            const int b = it / PB, xl = it - b * PB, x = x0 + xl;
+            if (xl >= nx) continue;
+            const double* pv = sPV + xl * PVS;
+            const bool vol = x < NQ;
+            const int f = vol ? 0 : (x - NQ) / NFQ, s = vol ? 0 : x - NQ - f * NFQ;
+            const double wgt = vol ? -A.dt * T.wq[x] * detJ : T.wf[s];
+            if (b == M) {
+                double Fc[M][D], Fv[M][D], ql[M][D];
+                const double* st = vol ? pv : pv + OH;     // the state the flux is evaluated at
+                for (int a = 0; a < M; ++a) for (int l = 0; l < D; ++l) ql[a][l] = pv[OG + a * D + l];
+                conv_flux<D, double, double>(st, ph, Fc);
+                visc_flux<D, double, double>(st, ql, pv[ON], ph, Fv);
+                if (vol) {
+                    for (int r = 0; r < D; ++r)
+                        for (int a = 0; a < M; ++a) {
+                            double v = 0.0;
+                            for (int k = 0; k < D; ++k) v += Jinv[r * D + k] * (Fc[a][k] - Fv[a][k]);
+                            sFres[(r * M + a) * NQ + x] = wgt * v;
+                        }
+                } else {
+                    const double nrm = fnrm[f], tau_s = pv[OT];
+                    const double* nw = NW + f * D;
+                    if (A.taup) A.taup[(el * NF + f) * NFQ + s] = tau_s;
+                    const int tag = A.ftag ? A.ftag[e * NF + f] : 0;
+                    for (int a = 0; a < M; ++a) {
+                        double fn = 0.0;
+                        for (int k = 0; k < D; ++k) fn += (Fc[a][k] - Fv[a][k]) * nw[k];
+                        const double fh = wgt * (fn + nrm * tau_s * (pv[a] - pv[OH + a]));
+                        sFH[(f * M + a) * NFQ + s] = fh;
+                        const double ub_a = tag == 1 ? boundary_state<NF, M, NFP>(A.ub, A.ubf, A.e2f, A.perm, T.mu, e, f, s, a) : 0.0;
+                        sFB[(f * M + a) * NFQ + s] = boundary_form<M>(tag, a, fh, wgt * nrm, pv, pv + OH, ub_a, A.ew);
+                    }
+                }
+                continue;
+            }
+            // Jacobian column b in TJ
+            const TJ* pvj = sPJ + xl * PJS;
+            const TJ* stj = vol ? pvj : pvj + OH;
+            const TJ nuj = pvj[ON], wj = (TJ)wgt;
+            const int c0 = vol ? 0 : D + f, nr = vol ? D : 1;              // flux directions sA[c0 .. c0 + nr)
+            TJ uj[M], qj[M][D];
+            for (int a = 0; a < M; ++a) { uj[a] = stj[a]; for (int l = 0; l < D; ++l) qj[a][l] = pvj[OG + a * D + l]; }
+            const int cs = vol ? NQ : NFQ;                                 // stride between coefficients
+            // element (a, r), coefficient 0 of column b
+            TJ* o0 = vol ? vc + (size_t)b * D * NCOEF * NQ + x : fc + ((size_t)f * M * M + b) * NCOEF * NFQ + s;
+            const size_t sa = vol ? (size_t)M * D * NCOEF * NQ : (size_t)M * NCOEF * NFQ, sr = (size_t)NCOEF * NQ;
+            {
+                DirT<TJ> ud[M], Fc[M][D], Fv[M][D];
+#pragma unroll
+                for (int a = 0; a < M; ++a) ud[a] = {uj[a], a == b ? TJ(1) : TJ(0)};
+                conv_flux<D, DirT<TJ>, TJ>(ud, pj, Fc);
+                visc_flux<D, DirT<TJ>, TJ>(ud, qj, nuj, pj, Fv);
+                // face points: d tau / d uhat_b (state-dependent stabilization)
+                TJ dtau = TJ(0), taun = TJ(0);
+                if (!vol) {
+                    taun = (TJ)(fnrm[f] * pv[OT]);
+                    if (A.tau_mode) {
+                        TJ nhj[D];
+                        for (int k = 0; k < D; ++k) nhj[k] = (TJ)fnh[f][k];
+                        dtau = (TJ)fnrm[f] * stab_tau<D, DirT<TJ>, TJ>(ud, nhj, (TJ)s_hinv, pj).t;
+                    }
+                }
+                for (int r = 0; r < nr; ++r) {
+                    TJ d[D];
+                    for (int k = 0; k < D; ++k) d[k] = sA[c0 + r][k];
+#pragma unroll
+                    for (int a = 0; a < M; ++a) {
+                        TJ v = 0;
+                        for (int k = 0; k < D; ++k) v += d[k] * (Fc[a][k].t - Fv[a][k].t);
+                        if (!vol) {
+                            if (a == b) v -= taun;
+                            v += (pvj[a] - uj[a]) * dtau;
+                        }
+                        o0[a * sa + r * sr] = wj * v;
+                    }
+                }
+            }
+            // q columns: a unit gradient q_{b,l} gives dv_ij = s_i delta_jl / rho and d(rho E)_j -> t, so along a
+            // direction d: stress rows mu/rho (s_i d_l + (d.s) delta_il - 2/3 d_i s_l), energy row
+            // mu/rho ((v.s + kappa (t - v.s)) d_l + (d.s) v_l - 2/3 (d.v) s_l); plus nu d_l on row b
+            const TJ irho = recip(uj[0]);
+            TJ vel[D], sv[D], kin = 0;
+#pragma unroll
+            for (int i = 0; i < D; ++i) { vel[i] = uj[1 + i] * irho; kin += vel[i] * vel[i]; }
+            const TJ E = uj[M - 1] * irho, mur = viscosity(E - kin * pj.half, pj) * irho;
+            TJ vs = 0;
+#pragma unroll
+            for (int i = 0; i < D; ++i) {
+                sv[i] = b == 0 ? -vel[i] : (b == 1 + i ? TJ(1) : TJ(0));
+                vs += vel[i] * sv[i];
+            }
+            const TJ t = b == 0 ? -E : (b == M - 1 ? TJ(1) : TJ(0));
+            // the common factor -w mu / rho goes into the operands: three operations per entry
+            const TJ fac = -wj * mur, ce = fac * (vs + pj.kap * (t - vs)), nuw = -wj * nuj;
+            TJ sf[D], ds[D], dv[D];                                        // d . s and d . v of the flux directions
+#pragma unroll
+            for (int i = 0; i < D; ++i) sf[i] = fac * sv[i];
+#pragma unroll
+            for (int r = 0; r < D; ++r) {
+                ds[r] = 0; dv[r] = 0;
+                if (r < nr)
+                    for (int k = 0; k < D; ++k) { ds[r] += sA[c0 + r][k] * sf[k]; dv[r] += sA[c0 + r][k] * vel[k]; }
+            }
+            for (int n = 0; n < ND; ++n) {                                 // directions the q variation is seen along
+                TJ bn[D], bs = 0, bv = 0;
+                for (int k = 0; k < D; ++k) { bn[k] = sB[n][k]; bs += bn[k] * sf[k]; bv += bn[k] * vel[k]; }
+                bs *= -pj.two_thirds;
+                TJ* on = o0 + (1 + n) * cs;
+#pragma unroll
+                for (int r = 0; r < D; ++r) {
+                    if (r >= nr) continue;
+                    const TJ g = sAB[c0 + r][n];
+                    on[r * sr] = b == 0 ? nuw * g : TJ(0);
+#pragma unroll
+                    for (int i = 0; i < D; ++i) {
+                        TJ v = sf[i] * g + ds[r] * bn[i] + sA[c0 + r][i] * bs;
+                        if (b == 1 + i) v += nuw * g;
+                        on[(1 + i) * sa + r * sr] = v;
+                    }
+                    TJ v = ce * g + ds[r] * bv + dv[r] * bs;
+                    if (b == M - 1) v += nuw * g;
+                    on[(M - 1) * sa + r * sr] = v;
+                }
+            }
+        }
+        __syncthreads();
+    }
     // right-hand-side column: Rh (trace rows) then Rt (interior rows)
     double* rbe = A.rb + el * A.rb_es;
     for (int idx = tid; idx < NT; idx += NTH) {
@@ -1276,13 +1332,12 @@ int run_linearize(hdg_ctx* h, const LinArgs& la) {
     using BS_ = BlkShape<C, BC::TY, BC::TX, BC::KC>;
     auto kblk = k_blocks<C, BC::TY, BC::TX, BC::KC, double, double>;
     auto kface = k_blocks<C, BC::TY, BC::TX, BC::KC, double, double, false>;
-    constexpr int PT = 128;
     const size_t sm_sf = sizeof(double) * SfShape<C>::smem_words;
     const size_t sm_point = sizeof(double) * point_smem_doubles<C>();
     const size_t sm_blk = sizeof(double) * BS_::smem;
     const size_t sm_elim16 = sizeof(double) * elim_smem_doubles<C, 16>();
     const size_t sm_elim8 = sizeof(double) * elim_smem_doubles<C, 8>();
-    HDG_CK(cudaFuncSetAttribute(k_point<C, PT, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
+    HDG_CK(cudaFuncSetAttribute(k_point<C, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
     HDG_CK(cudaFuncSetAttribute(kblk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
     HDG_CK(cudaFuncSetAttribute(kface, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
     HDG_CK(cudaFuncSetAttribute(k_blocks_sf<C, double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sf));
@@ -1321,7 +1376,7 @@ int run_linearize(hdg_ctx* h, const LinArgs& la) {
         const int64_t ne = std::min<int64_t>(h->chunk, h->E - e0);
         pa.e0 = e0; ba.e0 = e0;
         prof_begin(h, HDG_K_POINT);
-        k_point<C, PT, double><<<(unsigned)ne, PT, sm_point, st>>>(pa);
+        k_point<C, double><<<(unsigned)ne, PointShape<C>::NTH, sm_point, st>>>(pa);
         prof_end(h);
         prof_begin(h, HDG_K_BLOCKS);
         if (h->blocks64_mode == 1) {         // sum-factorised volume terms, then the face terms

@@ -935,7 +935,7 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
     using C = Cfg<D, P>;
     using BC = BlkCfg<C>;
     using BS_ = BlkShape<C, BC::TY, BC::TX, BC::KC>;
-    constexpr int PT = 128, NB = 16;
+    constexpr int NB = 16;
     int rc;
     if ((rc = ensure_system_storage(h, HDG_PREC_MIXED))) return rc;
     auto kblk = k_blocks<C, BC::TY, BC::TX, BC::KC, float, float>;
@@ -943,7 +943,7 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
     const size_t sm_point = sizeof(double) * point_smem_doubles<C>();
     const size_t sm_blk = sizeof(float) * BS_::smem_f32;
     const size_t sm_elim = elim_mixed_smem_bytes<C, NB>();
-    HDG_CK(cudaFuncSetAttribute(k_point<C, PT, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
+    HDG_CK(cudaFuncSetAttribute(k_point<C, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
     HDG_CK(cudaFuncSetAttribute(kblk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
     HDG_CK(cudaFuncSetAttribute(kface, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
     if (C::D == 3)
@@ -986,7 +986,7 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
         const int64_t ne = std::min<int64_t>(h->chunk, h->E - e0);
         pa.e0 = e0; ba.e0 = e0;
         prof_begin(h, HDG_K_POINT);
-        k_point<C, PT, float><<<(unsigned)ne, PT, sm_point, st>>>(pa);
+        k_point<C, float><<<(unsigned)ne, PointShape<C>::NTH, sm_point, st>>>(pa);
         prof_end(h);
         prof_begin(h, HDG_K_BLOCKS);
         if (h->blocks_mode == 1 && C::D == 3) {
