@@ -352,10 +352,8 @@ int hdg_sdirk3_tableau(double* A, double* b);
  * the same quantities to the same accuracy on the caller's own inputs
  * (reps linearize + condense calls each, after one warm-up, CUDA events on
  * the handle's stream) and keeps the fastest for later calls:
- *  - FP64 form: the volume contraction as a dense GEMM (blocks64_mode 0)
- *    or by sum factorisation over the tensor-product basis (1), the
- *    elimination kernel's panel width (16 or 8 columns) and the residency it
- *    is compiled for (2 or 1 CTAs per SM), and the Schur product
+ *  - FP64 form: the elimination kernel's panel width (16 or 8 columns) and
+ *    the residency it is compiled for (2 or 1 CTAs per SM), and the Schur product
  *    S = Dt - W Z inside the FP64 elimination (schur_mode 0) or on the BF16
  *    tensor cores by exact digit splitting of the FP64 factors (schur_mode 3:
  *    W and Z cut into 8..10 digits of 6..8 bits, products accumulated exactly
@@ -365,11 +363,11 @@ int hdg_sdirk3_tableau(double* A, double* b);
  *    (hexes, quads of degree 3);
  *  - mixed form: the elimination as one fused kernel (at 2 or 3 CTAs per
  *    SM) or split into an FP64 LU (panel width 16 or 8) and two FP32
- *    triangular solves,
- *    the volume contraction as FP32 SIMT (blocks_mode 0) or
- *    3xTF32 tensor cores (1, 3-D), and, when requested as HDG_PREC_MIXED,
+ *    triangular solves (the default), and, when requested as HDG_PREC_MIXED,
  *    the Schur product as FP32 SIMT (schur_mode 0) or 3xTF32 tensor cores
  *    (2) — all FP32-accurate; TF32 / 3xTF32 requested explicitly are kept;
+ *  - blocks64_mode (0, 1) and blocks_mode (0..2) are accepted and reported but
+ *    select nothing any more: every value runs the one contraction kernel;
  *  - tetrahedral handles: the elimination panel width (16 or 8 columns) of
  *    the persistent linearize + condense kernel (elim_nb; the other fields
  *    are zero; hdg_set_tuning reads elim_nb only).
@@ -433,7 +431,7 @@ int hdg_measure_peaks(double* tflops, double* ms);
  * HDG_EINVAL.  The per-chunk scratch (trace rows, point coefficients and the
  * per-point stabilization) comes from a 64 MiB file-scope device array of the
  * library instead of the handle's scratch, so elements are condensed in
- * chunks of at most 64 MiB / (scratch of one element) (45 hex p=2, 15 hex
+ * chunks of at most 64 MiB / (scratch of one element) (60 hex p=2, 19 hex
  * p=3 elements), whatever scratch budget the handle was created with.  The
  * call issues no cudaMalloc, cudaFree or other allocating routine.  The first
  * call on each device looks up the array's device address

@@ -115,7 +115,7 @@ int create_host(hdg_ctx* h, const hdg_mesh* mesh, int p, double gamma, double Re
     h->Nfp = ipow(p + 1, d - 1); h->Nfq = ipow(p + 2, d - 1);
     h->NU = h->m * h->Np; h->NQV = d * h->m * h->Np; h->NT = h->nf * h->m * h->Nfp;
     h->NR = h->NU + h->NT; h->NC = h->NR + 1; h->LD = (h->NC + 3) & ~3;
-    h->BS = h->m * h->Nfp; h->NCOEF = 1 + d + h->nf;
+    h->BS = h->m * h->Nfp; h->NCOEF = 1 + d;
     h->E = mesh->n_elem;
     h->phys = Phys{gamma, Re, Pr, Mach, 5.0, 0, 1.4042, 0.40417};
     try {
@@ -207,13 +207,9 @@ int create_device(hdg_ctx* h) {
     UP(h->tab.phi, t.phi); UP(h->tab.dphi, t.dphi); UP(h->tab.wq, t.wq);
     UP(h->tab.mu, t.mu); UP(h->tab.wf, t.wf); UP(h->tab.fnode, t.fnode); UP(h->tab.node_face, t.node_face);
     UP(h->tab.mhat, t.mhat); UP(h->tab.mf, t.mf); UP(h->tab.minv_c, t.minv_c); UP(h->tab.minv_e, t.minv_e);
-    UP(h->tab.psi, t.psi); UP(h->tab.theta, t.theta); UP(h->tab.psi_f, t.psi_f); UP(h->tab.theta_f, t.theta_f);
-    UP(h->tab.b1, t.b1); UP(h->tab.d1, t.d1);
+    UP(h->tab.b1, t.b1);
     auto f32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
-    UP(h->tab.fphi, f32(t.phi)); UP(h->tab.fdphi, f32(t.dphi)); UP(h->tab.fpsi, f32(t.psi));
-    UP(h->tab.ftheta, f32(t.theta)); UP(h->tab.fpsi_f, f32(t.psi_f)); UP(h->tab.ftheta_f, f32(t.theta_f));
-    UP(h->tab.fmu, f32(t.mu)); UP(h->tab.fmf, f32(t.mf));
-    UP(h->tab.fb1, f32(t.b1)); UP(h->tab.fd1, f32(t.d1));
+    UP(h->tab.fdphi, f32(t.dphi)); UP(h->tab.fmu, f32(t.mu));
     const int d = h->d, G = 1 + d * d + h->nf * d;
     std::vector<double> geo((size_t)h->E * G);
     for (int64_t e = 0; e < h->E; ++e) {
@@ -387,10 +383,8 @@ int hdg_autotune(hdg_handle h, const double* U, const double* Q, const double* U
                         cand[n][4] = h->elim_mixed_minb; cand[n][5] = bm64; cand[n][6] = h->elim_mixed_split; ++n;
                     }
     } else {
-        // FP32 SIMT and 3xTF32 tensor-core products are both FP32-accurate: the volume
-        // contraction always, the Schur product unless TF32 / 3xTF32 was requested explicitly
-        // contraction: tensor cores (3-D) or FP32 sum factorisation; the dense FP32 SIMT
-        // contraction only when the Schur precision is fixed (the candidate list holds 8)
+        // FP32 SIMT and 3xTF32 tensor-core Schur products are both FP32-accurate, unless TF32 /
+        // 3xTF32 was requested explicitly; the values of blocks_mode run the same kernel
         const bool free_schur = h->prec_req == HDG_PREC_MIXED;
         for (int sm : {0, 2}) {
             if (!free_schur && sm != 0) continue;

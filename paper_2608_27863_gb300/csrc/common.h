@@ -30,7 +30,7 @@ struct Cfg {
     static constexpr int NC = NU + NT + 1;       // columns (+ right-hand side)
     static constexpr int LD = (NC + 3) & ~3;     // padded row stride
     static constexpr int BS = M * NFP;           // BSR block size
-    static constexpr int NCOEF = 1 + D + NF;     // coefficients per (a, b, r, point)
+    static constexpr int NCOEF = 1 + D;          // coefficients per (a, b, r, point): u, q along the reference directions
 };
 
 // Reference-element tables of one configuration (host, FP64).
@@ -43,9 +43,7 @@ struct RefTables {
     std::vector<int32_t> node_face;                 // [Np][d]: f*Nfp + l, or -1
     std::vector<double> mhat, mf;                   // [Np][Np], [Nfp][Nfp]
     std::vector<double> minv_c, minv_e;             // [d][Np][Np], [nf][Np][Nfp]
-    std::vector<double> psi, theta;                 // [d][Nq][Np], [nf][Nq][Nfp]
-    std::vector<double> psi_f, theta_f;             // [nf][d][Nfq][Np], [nf][nf][Nfq][Nfp]
-    std::vector<double> b1, d1;                     // [p+2][p+1] 1-D basis values / derivatives at Gauss points
+    std::vector<double> b1;                         // [p+2][p+1] 1-D basis values at Gauss points
 };
 void build_ref_tables(int d, int p, RefTables& t);
 
@@ -77,11 +75,8 @@ struct DeviceTables {
     int32_t* fnode; int32_t* node_face;
     double* mhat; double* mf;
     double* minv_c; double* minv_e;
-    double* psi; double* theta; double* psi_f; double* theta_f;
-    double* b1; double* d1;          // 1-D tables of the tensor-product basis (sum factorisation)
-    float* fb1; float* fd1;
-    // float copies for the mixed form's FP32 contraction
-    float* fphi; float* fdphi; float* fpsi; float* ftheta; float* fpsi_f; float* ftheta_f; float* fmu; float* fmf;
+    double* b1;                      // 1-D basis values (sum factorisation)
+    float* fdphi; float* fmu;        // float copies for the mixed form's FP32 contraction
 };
 
 namespace tet { struct Ctx; }
@@ -197,9 +192,8 @@ struct hdg_ctx {
     // mixed form (allocated on the first mixed linearization)
     int sys_prec = HDG_PREC_FP64;          // precision of the assembled system
     int schur_mode = 0;                    // mixed Schur product: 0 FP32 SIMT, 1 TF32, 2 3xTF32 tensor cores
-    int blocks_mode = 1;                   // mixed volume contraction: 0 FP32 SIMT, 1 3xTF32 tensor cores (3-D),
-                                           // 2 FP32 sum factorisation
-    int blocks64_mode = 1;                 // FP64 volume contraction: 0 dense GEMM, 1 sum factorisation
+    int blocks_mode = 1;                   // accepted by the tuning calls (0..2); one contraction kernel serves all
+    int blocks64_mode = 1;                 // the same (0, 1)
     int schur64_mode = 0;                  // FP64 Schur product: 0 inside the FP64 elimination, 1 on the BF16
                                            // tensor cores by exact digit splitting (k_schur_ozaki); the
                                            // default is set with the device storage

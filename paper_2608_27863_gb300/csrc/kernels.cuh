@@ -172,12 +172,11 @@ __global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
     TJ* sPJ = reinterpret_cast<TJ*>(sPV + PB * PVS);   // [PB][PJS] the same for the Jacobian (gradient: Q)
     __shared__ double fnrm[NF], fnh[NF][D], s_hinv;     // face normals: length, direction; 1 / h
     __shared__ double geo[GEO];
-    // directions a flux can be taken along: the rows of Jinv (volume points), the face normals NW, and the
-    // lifting directions NW / detJ; their inner products with the directions of the q variation
+    // directions a flux is taken along, the rows of Jinv (volume points) and the face normals NW, and their
+    // inner products with the reference directions of the q variation
     constexpr int ND = D + NF;
     __shared__ TJ sA[ND][D];             // rows of Jinv, then NW
-    __shared__ TJ sB[ND][D];             // rows of Jinv, then NW / detJ
-    __shared__ TJ sAB[ND][ND];           // sA . sB
+    __shared__ TJ sAB[ND][D];            // sA . rows of Jinv
     const DeviceTables& T = A.tab;
 
     for (int i = tid; i < NU; i += NTH) sU[i] = A.U[e * NU + i];
@@ -228,9 +227,7 @@ __global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
     TJ* fc = reinterpret_cast<TJ*>(A.fcoef) + el * (size_t)(NF * M * M * NCOEF * NFQ);
     for (int i = tid; i < ND * D; i += NTH) {
         const int n = i / D, k = i - n * D;
-        const double v = n < D ? Jinv[n * D + k] : NW[(n - D) * D + k];
-        sA[n][k] = (TJ)v;
-        sB[n][k] = (TJ)(n < D ? v : v / detJ);
+        sA[n][k] = (TJ)(n < D ? Jinv[n * D + k] : NW[(n - D) * D + k]);
     }
     if (tid < NF) {
         double v = 0.0;
@@ -241,10 +238,10 @@ __global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
         if (tid == 0) s_hinv = A.tau_mode ? 1.0 / pow(double(1 << D) * detJ, 1.0 / D) : 0.0;   // |K|^{-1/d}
     }
     __syncthreads();
-    for (int i = tid; i < ND * ND; i += NTH) {
+    for (int i = tid; i < ND * D; i += NTH) {
         TJ v = 0;
-        for (int k = 0; k < D; ++k) v += sA[i / ND][k] * sB[i % ND][k];
-        sAB[i / ND][i % ND] = v;
+        for (int k = 0; k < D; ++k) v += sA[i / D][k] * sA[i % D][k];
+        sAB[i / D][i % D] = v;
     }
     for (int x0 = 0; x0 < NPT; x0 += PB) {
         const int nx = min(PB, NPT - x0);
@@ -402,9 +399,9 @@ __global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
                 if (r < nr)
                     for (int k = 0; k < D; ++k) { ds[r] += sA[c0 + r][k] * sf[k]; dv[r] += sA[c0 + r][k] * vel[k]; }
             }
-            for (int n = 0; n < ND; ++n) {                                 // directions the q variation is seen along
+            for (int n = 0; n < D; ++n) {                                  // reference directions of the q variation
                 TJ bn[D], bs = 0, bv = 0;
-                for (int k = 0; k < D; ++k) { bn[k] = sB[n][k]; bs += bn[k] * sf[k]; bv += bn[k] * vel[k]; }
+                for (int k = 0; k < D; ++k) { bn[k] = sA[n][k]; bs += bn[k] * sf[k]; bv += bn[k] * vel[k]; }
                 bs *= -pj.two_thirds;
                 TJ* on = o0 + (1 + n) * cs;
 #pragma unroll
@@ -458,405 +455,11 @@ __global__ void __launch_bounds__(PointShape<C>::NTH) k_point(PointArgs A) {
     }
 }
 
-// ----------------------------------------------------------------------------
-// A2: contraction of the coefficients with the basis tables into the blocks
-// ----------------------------------------------------------------------------
-template <class TL>
-struct BlkArgs {
-    const void* vcoef; const void* fcoef;   // Jacobian coefficients in the accumulation type
-    const int32_t* ftag;                    // [E][nf] or NULL
-    const double* geo;
-    DeviceTables tab;
-    Regions<TL> R;
-    double dt, a_ii, tau;
-    double ew;                              // wall internal energy of tag-3 faces
-    const double* taup;                     // [chunk][nf][Nfq] per-point tau (state-dependent), or NULL
-    int64_t e0;
-};
+}  // namespace hdg
 
-template <class C, int TY, int TX, int KC>
-struct BlkShape {
-    static constexpr int NCB = C::NP + C::NF * C::NFP;
-    static constexpr int NTH = TY * TX;
-    // register tiles when the output tile divides evenly; otherwise a flat
-    // thread -> output map (two shared loads per DFMA are free next to the FP64 pipe)
-    static constexpr bool FLAT = (C::NP % TY) != 0 || (NCB % TX) != 0;
-    static constexpr int TM = FLAT ? 1 : C::NP / TY, TN = FLAT ? 1 : NCB / TX;
-    static constexpr int SLOTS = (C::NP * NCB + NTH - 1) / NTH;
-    static constexpr int NPP = C::NP, NCBP = NCB;
-    static constexpr int main_smem = KC * (NPP + NCBP + C::NCOEF);
-    static constexpr int face_smem = C::NCOEF * C::NFQ + C::NFQ * NCB;
-    static constexpr int smem = main_smem > face_smem ? main_smem : face_smem;
-    // FP32 form: the face terms of the interior block are summed over the faces in a
-    // [Np][Np] shared tile and added to the FP64 block once
-    static constexpr int face_acc_smem = face_smem + C::NP * C::NP;
-    static constexpr int smem_f32 = main_smem > face_acc_smem ? main_smem : face_acc_smem;
-};
+#include "contract.cuh"
 
-// VOL = false skips the volume contraction (done on tensor cores by
-// k_blocks_tc in the mixed form) and adds only the face terms.
-template <class C, int TY, int TX, int KC, class TA, class TL, bool VOL = true>
-__global__ void __launch_bounds__(TY * TX) k_blocks(BlkArgs<TL> A) {
-    constexpr int D = C::D, M = C::M, NP = C::NP, NQ = C::NQ, NF = C::NF, NFP = C::NFP, NFQ = C::NFQ;
-    constexpr int NCOEF = C::NCOEF;
-    using S = BlkShape<C, TY, TX, KC>;
-    constexpr int NCB = S::NCB, TM = S::TM, TN = S::TN, NPP = S::NPP, NCBP = S::NCBP;
-    constexpr int K = D * NQ, NTH = TY * TX;
-    constexpr int GEO = Geo<D>::N;
-    const int tid = threadIdx.x, ty = tid / TX, tx = tid - ty * TX;
-    const int64_t bid = blockIdx.x;
-    const int b = (int)(bid % M), a = (int)((bid / M) % M);
-    const int64_t el = bid / (M * M), e = A.e0 + el;
-    const DeviceTables& T = A.tab;
-    extern __shared__ double sm_raw[];
-    TA* sm = reinterpret_cast<TA*>(sm_raw);
-    TA* As = sm;
-    TA* Bs = As + KC * NPP;
-    TA* Cs = Bs + KC * NCBP;
-    const TA* cf = reinterpret_cast<const TA*>(A.vcoef) + (((size_t)el * M + a) * M + b) * (size_t)(D * NCOEF * NQ);
-    // reference tables in the accumulation type
-    constexpr bool F32 = sizeof(TA) == 4;
-    const TA* tphi = F32 ? (const TA*)T.fphi : (const TA*)T.phi;
-    const TA* tdphi = F32 ? (const TA*)T.fdphi : (const TA*)T.dphi;
-    const TA* tpsi = F32 ? (const TA*)T.fpsi : (const TA*)T.psi;
-    const TA* ttheta = F32 ? (const TA*)T.ftheta : (const TA*)T.theta;
-    const TA* tpsif = F32 ? (const TA*)T.fpsi_f : (const TA*)T.psi_f;
-    const TA* tthetaf = F32 ? (const TA*)T.ftheta_f : (const TA*)T.theta_f;
-    const TA* tmu = F32 ? (const TA*)T.fmu : (const TA*)T.mu;
-    const TA* tmf = F32 ? (const TA*)T.fmf : (const TA*)T.mf;
-
-    constexpr bool FLAT = S::FLAT;
-    constexpr int SL = FLAT ? S::SLOTS : TM * TN;
-    TA acc[SL];
-    int ri[SL], ci[SL];
-#pragma unroll
-    for (int s = 0; s < SL; ++s) {
-        acc[s] = 0.0;
-        if (FLAT) {
-            int idx = tid + NTH * s;
-            ri[s] = idx < NP * NCB ? idx / NCB : -1;
-            ci[s] = idx < NP * NCB ? idx - (idx / NCB) * NCB : 0;
-        } else {
-            ri[s] = ty + TY * (s / TN);
-            ci[s] = tx + TX * (s % TN);
-        }
-    }
-
-    for (int k0 = 0; VOL && k0 < K; k0 += KC) {
-        const int kc = min(KC, K - k0);
-        for (int idx = tid; idx < kc * NCOEF; idx += NTH) {
-            int kk = idx / NCOEF, c = idx - kk * NCOEF, k = k0 + kk, r = k / NQ, g = k - r * NQ;
-            Cs[idx] = cf[(r * NCOEF + c) * NQ + g];
-        }
-        for (int idx = tid; idx < kc * NPP; idx += NTH) As[idx] = tdphi[(size_t)k0 * NP + idx];
-        __syncthreads();
-        for (int idx = tid; idx < kc * NCBP; idx += NTH) {
-            int kk = idx / NCBP, c = idx - kk * NCBP;
-            int k = k0 + kk, r = k / NQ, g = k - r * NQ;
-            const TA* cc = Cs + kk * NCOEF;
-            TA v;
-            if (c < NP) {
-                v = cc[0] * tphi[g * NP + c];
-                for (int r2 = 0; r2 < D; ++r2) v -= cc[1 + r2] * tpsi[((size_t)r2 * NQ + g) * NP + c];
-            } else {
-                int c2 = c - NP, f = c2 / NFP, l = c2 - f * NFP;
-                v = cc[1 + D + f] * ttheta[((size_t)f * NQ + g) * NFP + l];
-            }
-            Bs[idx] = v;
-        }
-        __syncthreads();
-        if (FLAT) {
-            for (int kk = 0; kk < kc; ++kk) {
-#pragma unroll
-                for (int s = 0; s < SL; ++s)
-                    if (ri[s] >= 0) acc[s] = fma(As[kk * NPP + ri[s]], Bs[kk * NCBP + ci[s]], acc[s]);
-            }
-        } else {
-            for (int kk = 0; kk < kc; ++kk) {
-                TA av[TM], bv[TN];
-#pragma unroll
-                for (int ii = 0; ii < TM; ++ii) av[ii] = As[kk * NPP + ty + TY * ii];
-#pragma unroll
-                for (int jj = 0; jj < TN; ++jj) bv[jj] = Bs[kk * NCBP + tx + TX * jj];
-#pragma unroll
-                for (int ii = 0; ii < TM; ++ii)
-#pragma unroll
-                    for (int jj = 0; jj < TN; ++jj) acc[ii * TN + jj] = fma(av[ii], bv[jj], acc[ii * TN + jj]);
-            }
-        }
-        __syncthreads();
-    }
-
-    const double* G = A.geo + e * GEO;
-    const double detJ = G[0];
-    double* A11 = A.R.a11 + e * A.R.a11_es;
-    TL* A12 = A.R.a12 + e * A.R.a12_es;
-#pragma unroll
-    for (int s = 0; s < SL; ++s) {
-        const int i = ri[s], c = ci[s];
-        if (!VOL || i < 0 || i >= NP || c >= NCB) continue;
-        const int64_t row = a * NP + i;
-        if (c < NP) {
-            double v = (double)acc[s];
-            if (a == b) v += detJ / A.a_ii * T.mhat[i * NP + c];
-            A11[row * A.R.a11_rs + b * NP + c] = v;
-        } else {
-            int c2 = c - NP, f = c2 / NFP, l = c2 - f * NFP;
-            A12[row * A.R.a12_rs + (f * M + b) * NFP + l] = (TL)acc[s];
-        }
-    }
-    __syncthreads();
-
-    // face terms: rows of Ct / Dt, and dt x the same rows added to At / Bt at the face nodes
-    TL* A21 = A.R.a21 + el * A.R.a21_es;
-    TL* A22 = A.R.a22 + el * A.R.a22_es;
-    TA* Fc = sm;                           // [NCOEF][Nfq]
-    TA* Tt = Fc + NCOEF * NFQ;             // [Nfq][NCB]
-    constexpr bool FACC = sizeof(TA) == 4;  // FP32 form: sum the At face terms in shared memory
-    TA* Acc = Tt + NFQ * NCB;              // [Np][Np] (FP32 form only)
-    if (FACC) {
-        for (int idx = tid; idx < NP * NP; idx += NTH) Acc[idx] = (TA)0;
-        __syncthreads();
-    }
-    const double* NW = G + 1 + D * D;
-    const double* Jg = G + 1;
-    (void)Jg;
-    __shared__ TA mft[NFP * NFP];          // state-dependent tau: face mass weighted by tau(s)
-    for (int f = 0; f < NF; ++f) {
-        const TA* fsrc = reinterpret_cast<const TA*>(A.fcoef) + ((((size_t)el * NF + f) * M + a) * M + b) * (size_t)(NCOEF * NFQ);
-        for (int idx = tid; idx < NCOEF * NFQ; idx += NTH) Fc[idx] = fsrc[idx];
-        if (A.taup)
-            for (int idx = tid; idx < NFP * NFP; idx += NTH) {
-                const int lam = idx / NFP, l = idx - lam * NFP;
-                double w = 0.0;
-                for (int q = 0; q < NFQ; ++q)
-                    w += T.wf[q] * A.taup[(el * NF + f) * NFQ + q] * T.mu[q * NFP + lam] * T.mu[q * NFP + l];
-                mft[idx] = (TA)w;
-            }
-        __syncthreads();
-        for (int idx = tid; idx < NFQ * NCB; idx += NTH) {
-            int s = idx / NCB, c = idx - s * NCB;
-            TA v = 0;
-            if (c < NP) {
-                for (int r2 = 0; r2 < D; ++r2)
-                    v -= Fc[(1 + r2) * NFQ + s] * tpsif[(((size_t)f * D + r2) * NFQ + s) * NP + c];
-            } else {
-                int c2 = c - NP, f2 = c2 / NFP, l2 = c2 - f2 * NFP;
-                v = Fc[(1 + D + f2) * NFQ + s] * tthetaf[(((size_t)f * NF + f2) * NFQ + s) * NFP + l2];
-                if (f2 == f) v += Fc[s] * tmu[s * NFP + l2];
-            }
-            Tt[idx] = v;
-        }
-        __syncthreads();
-        double nrm = 0.0;
-        for (int k = 0; k < D; ++k) nrm += NW[f * D + k] * NW[f * D + k];
-        nrm = sqrt(nrm);
-        const TA taun = (TA)(A.tau * nrm), dtt = (TA)A.dt;
-        const int tag = A.ftag ? A.ftag[e * NF + f] : 0;
-        // trace rows of a boundary face: copies of the numerical-flux rows, or algebraic in
-        // (uhat, u) with d bhat_a / d uhat_b = cb * face mass and d bhat_a / d u_b = cu * face mass
-        const bool flux_row = boundary_row_is_flux<M>(tag, a);
-        const TA nrmt = (TA)nrm;
-        TA cb = (a == b) ? (TA)1 : (TA)0, cu = (TA)0;
-        if (tag == 3 && a == M - 1 && b == 0) cb = (TA)(-A.ew);
-        if (tag == 2 && a == b) cu = (TA)(-1);
-        for (int idx = tid; idx < NFP * NCB; idx += NTH) {
-            int lam = idx / NCB, c = idx - lam * NCB;
-            TA v = 0;
-            for (int s = 0; s < NFQ; ++s) v += tmu[s * NFP + lam] * Tt[s * NCB + c];
-            const int64_t trow = (f * M + a) * NFP + lam;
-            const int64_t irow = a * NP + T.fnode[f * NFP + lam];
-            if (c < NP) {
-                TA vu = 0, vut = 0;                // face mass coupling of node c, if it lies on face f
-                for (int k = 0; k < D; ++k) {
-                    int nfc = T.node_face[c * D + k];
-                    if (nfc >= 0 && nfc / NFP == f) {
-                        vu = tmf[lam * NFP + (nfc - f * NFP)];
-                        if (A.taup) vut = mft[lam * NFP + (nfc - f * NFP)];
-                    }
-                }
-                if (a == b) v += A.taup ? nrmt * vut : taun * vu;
-                const int col = b * NP + c;
-                A21[trow * A.R.a21_rs + col] = flux_row ? (TL)v : (TL)(cu * nrmt * vu);
-                if (FACC)   // one thread per (node, column) within a face; faces run one after another
-                    Acc[T.fnode[f * NFP + lam] * NP + c] += dtt * v;
-                else
-                    A11[irow * A.R.a11_rs + col] += A.dt * (double)v;
-            } else {
-                int c2 = c - NP, f2 = c2 / NFP, l2 = c2 - f2 * NFP;
-                const int col = (f2 * M + b) * NFP + l2;
-                const TA vb = (f2 == f) ? cb * nrmt * tmf[lam * NFP + l2] : (TA)0;
-                A22[trow * A.R.a22_rs + col] = flux_row ? (TL)v : (TL)vb;
-                A12[irow * A.R.a12_rs + col] = (TL)(A12[irow * A.R.a12_rs + col] + dtt * v);
-            }
-        }
-        __syncthreads();
-    }
-    if (FACC)
-        for (int idx = tid; idx < NP * NP; idx += NTH) {
-            const int i = idx / NP, c = idx - i * NP;
-            const TA v = Acc[idx];
-            if (v != (TA)0) A11[(a * NP + i) * A.R.a11_rs + b * NP + c] += (double)v;
-        }
-}
-
-// ----------------------------------------------------------------------------
-// A2 (FP64 form) by sum factorisation.  The volume contraction
-//   Out[i][c] = sum_k sum_g dphi_k[g][i] G_k[g][c]
-// (i a test function, c a block column, g a quadrature point, k a direction)
-// has a tensor-product operator dphi_k = T_{k,0} (x) T_{k,1} (x) T_{k,2} with
-// T_{k,r} the 1-D derivative table on axis r = k and the 1-D basis table
-// elsewhere ((p+2) x (p+1) each).  It is applied one axis at a time to every
-// column of G_k: (p+2)^2 (p+1) + (p+2)(p+1)^2 + (p+1)^3 multiply-adds per
-// column and direction in 3-D instead of (p+1)^3 (p+2)^3.  G_k is generated
-// from the point coefficients exactly as in k_blocks.  One CTA per (element,
-// component pair), columns in chunks of CW; the face terms follow in
-// k_blocks<..., VOL = false>.
-// ----------------------------------------------------------------------------
-template <class C, class TA = double>
-struct SfShape {
-    static constexpr int N1 = C::P + 1, Q1 = C::P + 2;
-    static constexpr int NCB = C::NP + C::NF * C::NFP;
-    // columns per chunk: 16 in FP64 (the FP64 pipe bounds the kernel), 32 in FP32, where the
-    // per-chunk barriers and coefficient reloads, not the FMAs, set the time
-    static constexpr int CW = sizeof(TA) == 4 ? 32 : 16;
-    static constexpr int NX = (C::D == 3) ? Q1 * Q1 * N1 : Q1 * N1;      // after the first axis
-    static constexpr int NY = (C::D == 3) ? Q1 * N1 * N1 : 0;            // after the second (3-D)
-    static constexpr int NTH = 128;
-    static constexpr int SLOTS = (C::NP * CW + NTH - 1) / NTH;
-    static constexpr int smem_words = C::NCOEF * C::NQ + CW * (C::NQ + NX + NY);   // in the accumulation type
-};
-
-template <class C, class TA, class TL>
-__global__ void __launch_bounds__(SfShape<C, TA>::NTH) k_blocks_sf(BlkArgs<TL> A) {
-    using S = SfShape<C, TA>;
-    constexpr int D = C::D, M = C::M, NP = C::NP, NQ = C::NQ, NFP = C::NFP, NCOEF = C::NCOEF;
-    constexpr int N1 = S::N1, Q1 = S::Q1, NCB = S::NCB, CW = S::CW, NTH = S::NTH;
-    constexpr int GEO = Geo<D>::N;
-    const int tid = threadIdx.x;
-    const int64_t bid = blockIdx.x;
-    const int b = (int)(bid % M), a = (int)((bid / M) % M);
-    const int64_t el = bid / (M * M), e = A.e0 + el;
-    const DeviceTables& T = A.tab;
-    // tables in the accumulation type (FP64 form: double; mixed form: float)
-    constexpr bool F32 = sizeof(TA) == 4;
-    const TA* tphi = F32 ? (const TA*)T.fphi : (const TA*)T.phi;
-    const TA* tpsi = F32 ? (const TA*)T.fpsi : (const TA*)T.psi;
-    const TA* ttheta = F32 ? (const TA*)T.ftheta : (const TA*)T.theta;
-    const TA* tb1 = F32 ? (const TA*)T.fb1 : (const TA*)T.b1;
-    const TA* td1 = F32 ? (const TA*)T.fd1 : (const TA*)T.d1;
-    extern __shared__ double sm_raw[];
-    TA* cs = reinterpret_cast<TA*>(sm_raw);   // [NCOEF][Nq] coefficients of one direction
-    TA* Gs = cs + NCOEF * NQ;        // [Nq][CW]
-    TA* Xs = Gs + NQ * CW;           // [NX][CW]
-    TA* Ys = Xs + S::NX * CW;        // [NY][CW] (3-D)
-    const TA* cf = static_cast<const TA*>(A.vcoef) + (((size_t)el * M + a) * M + b) * (size_t)(D * NCOEF * NQ);
-    const double detJ = A.geo[e * GEO];
-    double* A11 = A.R.a11 + e * A.R.a11_es;
-    TL* A12 = A.R.a12 + e * A.R.a12_es;
-#pragma unroll 1
-    for (int c0 = 0; c0 < NCB; c0 += CW) {
-        const int cw = min(CW, NCB - c0);
-        TA acc[S::SLOTS];
-#pragma unroll
-        for (int s = 0; s < S::SLOTS; ++s) acc[s] = (TA)0;
-#pragma unroll 1
-        for (int k = 0; k < D; ++k) {
-            __syncthreads();                 // the previous direction is done with cs / Gs
-            for (int idx = tid; idx < NCOEF * NQ; idx += NTH) cs[idx] = cf[(size_t)k * NCOEF * NQ + idx];
-            __syncthreads();
-            for (int idx = tid; idx < NQ * CW; idx += NTH) {
-                const int g = idx / CW, cc = idx - g * CW, c = c0 + cc;
-                TA v = (TA)0;
-                if (cc < cw) {
-                    if (c < NP) {
-                        v = cs[g] * tphi[g * NP + c];
-                        for (int r2 = 0; r2 < D; ++r2) v -= cs[(1 + r2) * NQ + g] * tpsi[((size_t)r2 * NQ + g) * NP + c];
-                    } else {
-                        const int c2 = c - NP, f = c2 / NFP, l = c2 - f * NFP;
-                        v = cs[(1 + D + f) * NQ + g] * ttheta[((size_t)f * NQ + g) * NFP + l];
-                    }
-                }
-                Gs[idx] = v;
-            }
-            __syncthreads();
-            const TA* T0 = (k == 0) ? td1 : tb1;
-            const TA* T1 = (k == 1) ? td1 : tb1;
-            if (D == 3) {
-                const TA* T2 = (k == 2) ? td1 : tb1;
-                // X[j2][g1][g0] = sum_g2 T2[g2][j2] G[g0 + Q1 g1 + Q1^2 g2]
-                for (int idx = tid; idx < S::NX * CW; idx += NTH) {
-                    const int cc = idx % CW, rest = idx / CW, j2 = rest % N1, g01 = rest / N1;
-                    TA s = (TA)0;
-#pragma unroll
-                    for (int g2 = 0; g2 < Q1; ++g2) s = fma(T2[g2 * N1 + j2], Gs[(g01 + Q1 * Q1 * g2) * CW + cc], s);
-                    Xs[(j2 * Q1 * Q1 + g01) * CW + cc] = s;
-                }
-                __syncthreads();
-                // Y[j2][j1][g0] = sum_g1 T1[g1][j1] X[j2][g1][g0]
-                for (int idx = tid; idx < S::NY * CW; idx += NTH) {
-                    const int cc = idx % CW, rest = idx / CW, g0 = rest % Q1, j12 = rest / Q1;
-                    const int j1 = j12 % N1, j2 = j12 / N1;
-                    TA s = (TA)0;
-#pragma unroll
-                    for (int g1 = 0; g1 < Q1; ++g1) s = fma(T1[g1 * N1 + j1], Xs[(j2 * Q1 * Q1 + g1 * Q1 + g0) * CW + cc], s);
-                    Ys[(j12 * Q1 + g0) * CW + cc] = s;
-                }
-                __syncthreads();
-                // out[j0 + N1 j12] += sum_g0 T0[g0][j0] Y[j12][g0]
-#pragma unroll
-                for (int s = 0; s < S::SLOTS; ++s) {
-                    const int idx = tid + NTH * s;
-                    if (idx < NP * CW) {
-                        const int cc = idx % CW, j = idx / CW, j0 = j % N1, j12 = j / N1;
-                        TA t = (TA)0;
-#pragma unroll
-                        for (int g0 = 0; g0 < Q1; ++g0) t = fma(T0[g0 * N1 + j0], Ys[(j12 * Q1 + g0) * CW + cc], t);
-                        acc[s] += t;
-                    }
-                }
-            } else {
-                // X[j1][g0] = sum_g1 T1[g1][j1] G[g0 + Q1 g1]
-                for (int idx = tid; idx < S::NX * CW; idx += NTH) {
-                    const int cc = idx % CW, rest = idx / CW, g0 = rest % Q1, j1 = rest / Q1;
-                    TA s = (TA)0;
-#pragma unroll
-                    for (int g1 = 0; g1 < Q1; ++g1) s = fma(T1[g1 * N1 + j1], Gs[(g0 + Q1 * g1) * CW + cc], s);
-                    Xs[(j1 * Q1 + g0) * CW + cc] = s;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int s = 0; s < S::SLOTS; ++s) {
-                    const int idx = tid + NTH * s;
-                    if (idx < NP * CW) {
-                        const int cc = idx % CW, j = idx / CW, j0 = j % N1, j1 = j / N1;
-                        TA t = (TA)0;
-#pragma unroll
-                        for (int g0 = 0; g0 < Q1; ++g0) t = fma(T0[g0 * N1 + j0], Xs[(j1 * Q1 + g0) * CW + cc], t);
-                        acc[s] += t;
-                    }
-                }
-            }
-        }
-        // the chunk's columns of At (with the DIRK mass term) and Bt
-#pragma unroll
-        for (int s = 0; s < S::SLOTS; ++s) {
-            const int idx = tid + NTH * s;
-            if (idx >= NP * CW) continue;
-            const int cc = idx % CW, i = idx / CW, c = c0 + cc;
-            if (cc >= cw) continue;
-            const int64_t row = a * NP + i;
-            if (c < NP) {
-                double v = (double)acc[s];
-                if (a == b) v += detJ / A.a_ii * T.mhat[i * NP + c];
-                A11[row * A.R.a11_rs + b * NP + c] = v;
-            } else {
-                const int c2 = c - NP, f = c2 / NFP, l = c2 - f * NFP;
-                A12[row * A.R.a12_rs + (f * M + b) * NFP + l] = (TL)acc[s];
-            }
-        }
-    }
-}
+namespace hdg {
 
 // ----------------------------------------------------------------------------
 // A3 + A4: bordered Gaussian elimination (interior LU, solves and Schur complement)
@@ -1285,14 +888,6 @@ __global__ void __launch_bounds__(NTH) k_recover(RecArgs A) {
 // ----------------------------------------------------------------------------
 // launchers
 // ----------------------------------------------------------------------------
-template <class C> struct BlkCfg;
-template <> struct BlkCfg<Cfg<2, 1>> { static constexpr int TY = 4, TX = 8, KC = 16; };
-template <> struct BlkCfg<Cfg<2, 2>> { static constexpr int TY = 4, TX = 8, KC = 16; };
-template <> struct BlkCfg<Cfg<2, 3>> { static constexpr int TY = 8, TX = 8, KC = 16; };
-template <> struct BlkCfg<Cfg<3, 1>> { static constexpr int TY = 8, TX = 8, KC = 16; };
-template <> struct BlkCfg<Cfg<3, 2>> { static constexpr int TY = 8, TX = 16, KC = 16; };
-template <> struct BlkCfg<Cfg<3, 3>> { static constexpr int TY = 16, TX = 16, KC = 16; };
-
 #define HDG_CK(call)                                                                   \
     do {                                                                               \
         cudaError_t err_ = (call);                                                     \
@@ -1328,19 +923,12 @@ template <int D, int P>
 int run_linearize(hdg_ctx* h, const LinArgs& la) {
     if (int rc = ensure_system_storage(h, HDG_PREC_FP64)) return rc;
     using C = Cfg<D, P>;
-    using BC = BlkCfg<C>;
-    using BS_ = BlkShape<C, BC::TY, BC::TX, BC::KC>;
-    auto kblk = k_blocks<C, BC::TY, BC::TX, BC::KC, double, double>;
-    auto kface = k_blocks<C, BC::TY, BC::TX, BC::KC, double, double, false>;
-    const size_t sm_sf = sizeof(double) * SfShape<C>::smem_words;
+    using CS = ContractShape<C, double>;
     const size_t sm_point = sizeof(double) * point_smem_doubles<C>();
-    const size_t sm_blk = sizeof(double) * BS_::smem;
     const size_t sm_elim16 = sizeof(double) * elim_smem_doubles<C, 16>();
     const size_t sm_elim8 = sizeof(double) * elim_smem_doubles<C, 8>();
     HDG_CK(cudaFuncSetAttribute(k_point<C, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
-    HDG_CK(cudaFuncSetAttribute(kblk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
-    HDG_CK(cudaFuncSetAttribute(kface, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
-    HDG_CK(cudaFuncSetAttribute(k_blocks_sf<C, double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sf));
+    HDG_CK(cudaFuncSetAttribute(k_contract<C, double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS::smem_bytes));
     HDG_CK(cudaFuncSetAttribute(k_elim<C, 16, 256, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim16));
     HDG_CK(cudaFuncSetAttribute(k_elim<C, 16, 256, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim16));
     HDG_CK(cudaFuncSetAttribute(k_elim<C, 8, 256, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim8));
@@ -1371,7 +959,7 @@ int run_linearize(hdg_ctx* h, const LinArgs& la) {
     ba.vcoef = h->d_vcoef; ba.fcoef = h->d_fcoef; ba.geo = h->d_geo; ba.tab = h->tab; ba.ftag = h->d_ftag;
     ba.ew = h->e_wall;
     ba.taup = h->phys.tau_mode ? h->d_taup : nullptr;
-    ba.R = RG; ba.dt = la.dt; ba.a_ii = la.a_ii; ba.tau = h->phys.tau;
+    ba.R = RG; ba.dt = la.dt; ba.a_ii = la.a_ii; ba.tau = h->phys.tau; ba.has_nu = la.nu != nullptr;
     for (int64_t e0 = 0; e0 < h->E; e0 += h->chunk) {
         const int64_t ne = std::min<int64_t>(h->chunk, h->E - e0);
         pa.e0 = e0; ba.e0 = e0;
@@ -1379,12 +967,7 @@ int run_linearize(hdg_ctx* h, const LinArgs& la) {
         k_point<C, double><<<(unsigned)ne, PointShape<C>::NTH, sm_point, st>>>(pa);
         prof_end(h);
         prof_begin(h, HDG_K_BLOCKS);
-        if (h->blocks64_mode == 1) {         // sum-factorised volume terms, then the face terms
-            k_blocks_sf<C, double, double><<<(unsigned)(ne * C::M * C::M), SfShape<C>::NTH, sm_sf, st>>>(ba);
-            kface<<<(unsigned)(ne * C::M * C::M), BC::TY * BC::TX, sm_blk, st>>>(ba);
-        } else {
-            kblk<<<(unsigned)(ne * C::M * C::M), BC::TY * BC::TX, sm_blk, st>>>(ba);
-        }
+        k_contract<C, double, double><<<(unsigned)(ne * CS::NG), CS::NTH, CS::smem_bytes, st>>>(ba);
         prof_end(h);
         prof_begin(h, HDG_K_ELIM);
         // variant chosen by the autotuner: panel width 16 or 8, built for 1 or 2 resident CTAs per SM

@@ -913,10 +913,6 @@ template <class C, bool SPLIT3>
 __global__ void k_schur_tc(Regions<float> R, int64_t e0, int32_t* status);
 template <class C>
 struct SchurTC;
-template <class C>
-struct BlkTC;
-template <class C>
-__global__ void k_blocks_tc(BlkArgs<float> A, int32_t* status);
 
 inline Regions<float> mixed_regions(hdg_ctx* h) {
     const int64_t NU = h->NU, NT = h->NT;
@@ -933,23 +929,14 @@ inline Regions<float> mixed_regions(hdg_ctx* h) {
 template <int D, int P>
 int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
     using C = Cfg<D, P>;
-    using BC = BlkCfg<C>;
-    using BS_ = BlkShape<C, BC::TY, BC::TX, BC::KC>;
+    using CS = ContractShape<C, float>;
     constexpr int NB = 16;
     int rc;
     if ((rc = ensure_system_storage(h, HDG_PREC_MIXED))) return rc;
-    auto kblk = k_blocks<C, BC::TY, BC::TX, BC::KC, float, float>;
-    auto kface = k_blocks<C, BC::TY, BC::TX, BC::KC, float, float, false>;
     const size_t sm_point = sizeof(double) * point_smem_doubles<C>();
-    const size_t sm_blk = sizeof(float) * BS_::smem_f32;
     const size_t sm_elim = elim_mixed_smem_bytes<C, NB>();
     HDG_CK(cudaFuncSetAttribute(k_point<C, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_point));
-    HDG_CK(cudaFuncSetAttribute(kblk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
-    HDG_CK(cudaFuncSetAttribute(kface, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_blk));
-    if (C::D == 3)
-        HDG_CK(cudaFuncSetAttribute(k_blocks_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, BlkTC<C>::smem_bytes()));
-    const size_t sm_sf32 = sizeof(float) * SfShape<C, float>::smem_words;
-    HDG_CK(cudaFuncSetAttribute(k_blocks_sf<C, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sf32));
+    HDG_CK(cudaFuncSetAttribute(k_contract<C, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CS::smem_bytes));
     HDG_CK(cudaFuncSetAttribute(k_elim_mixed<C, NB, 256, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim));
     HDG_CK(cudaFuncSetAttribute(k_elim_mixed<C, NB, 256, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_elim));
     const int sm_lu = lu_mixed_smem_bytes<C, NB>();   // the 8-column variant needs less
@@ -981,7 +968,7 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
     ba.vcoef = h->d_vcoef; ba.fcoef = h->d_fcoef; ba.geo = h->d_geo; ba.tab = h->tab; ba.ftag = h->d_ftag;
     ba.ew = h->e_wall;
     ba.taup = h->phys.tau_mode ? h->d_taup : nullptr;
-    ba.R = RM; ba.dt = la.dt; ba.a_ii = la.a_ii; ba.tau = h->phys.tau;
+    ba.R = RM; ba.dt = la.dt; ba.a_ii = la.a_ii; ba.tau = h->phys.tau; ba.has_nu = la.nu != nullptr;
     for (int64_t e0 = 0; e0 < h->E; e0 += h->chunk) {
         const int64_t ne = std::min<int64_t>(h->chunk, h->E - e0);
         pa.e0 = e0; ba.e0 = e0;
@@ -989,18 +976,7 @@ int run_linearize_mixed(hdg_ctx* h, const LinArgs& la) {
         k_point<C, float><<<(unsigned)ne, PointShape<C>::NTH, sm_point, st>>>(pa);
         prof_end(h);
         prof_begin(h, HDG_K_BLOCKS);
-        if (h->blocks_mode == 1 && C::D == 3) {
-            // volume contraction on tensor cores (3xTF32), face terms added by the SIMT kernel
-            using BT = BlkTC<C>;
-            k_blocks_tc<C><<<(unsigned)(ne * BT::NMT), BT::THREADS, BT::smem_bytes(), st>>>(ba, h->d_status);
-            kface<<<(unsigned)(ne * C::M * C::M), BC::TY * BC::TX, sm_blk, st>>>(ba);
-        } else if (h->blocks_mode == 2) {
-            // volume contraction by FP32 sum factorisation, then the face terms
-            k_blocks_sf<C, float, float><<<(unsigned)(ne * C::M * C::M), SfShape<C, float>::NTH, sm_sf32, st>>>(ba);
-            kface<<<(unsigned)(ne * C::M * C::M), BC::TY * BC::TX, sm_blk, st>>>(ba);
-        } else {
-            kblk<<<(unsigned)(ne * C::M * C::M), BC::TY * BC::TX, sm_blk, st>>>(ba);
-        }
+        k_contract<C, float, float><<<(unsigned)(ne * CS::NG), CS::NTH, CS::smem_bytes, st>>>(ba);
         prof_end(h);
         prof_begin(h, HDG_K_ELIM);
         if (h->elim_mixed_split) {
@@ -1306,240 +1282,5 @@ __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float>
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(S::TCOLS));
 }
 
-template <class C>
-struct BlkTC {
-    static constexpr int NCB = C::NP + C::NF * C::NFP;
-    static constexpr int MR = C::M * C::M * NCB;
-    static constexpr int MT = 128, KC = 16;   // 16-wide chunks keep 4-5 CTAs (32-40 warps) per SM
-    static constexpr int NMT = (MR + MT - 1) / MT;
-    static constexpr int K = C::D * C::NQ;
-    static constexpr int CPD = (C::NQ + KC - 1) / KC;                     // chunks per direction
-    static constexpr int NCH = C::D * CPD;                                // chunks in all
-    static constexpr int NTN = (C::NP + 15) / 16 * 16;
-    static constexpr int TCOLS = NTN <= 32 ? 32 : NTN <= 64 ? 64 : 128;
-    static constexpr int THREADS = 256;
-    static_assert(THREADS == 2 * MT, "a thread forms one row for two K quads");
-    static constexpr int STAGE = 2 * (MT * KC + NTN * KC);                // floats of one stage (hi and lo)
-    static constexpr int MINB = NTN <= 32 ? 5 : 3;                        // resident CTAs (registers, stages)
-    static_assert(NTN <= 128, "N tile too wide");
-    __host__ __device__ static constexpr int smem_bytes() { return 2 * STAGE * 4 + 64; }
-};
-
-// Volume contraction of the mixed form on the tensor cores: Out[(a, b, c)][i] =
-// sum_k G_ab[k][c] dphi[k][i] per element, 3xTF32 with FP32 accumulation in TMEM.
-// 8 warps per (element, 128-row tile); the operand tiles are double-buffered so that
-// the threads generate chunk c + 1 (rows fastest: a quarter warp's 16-byte stores are
-// contiguous) while the tensor cores run chunk c.
-template <class C>
-__global__ void __launch_bounds__(BlkTC<C>::THREADS, BlkTC<C>::MINB) k_blocks_tc(BlkArgs<float> A, int32_t* status) {
-    using S = BlkTC<C>;
-    constexpr int D = C::D, M = C::M, NP = C::NP, NQ = C::NQ, NFP = C::NFP, NCOEF = C::NCOEF;
-    constexpr int NCB = S::NCB, MR = S::MR, MT = S::MT, KC = S::KC, NTN = S::NTN, TH = S::THREADS;
-    constexpr int GEO = Geo<D>::N;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t bid = blockIdx.x;
-    const int mt = (int)(bid % S::NMT);
-    const int64_t el = bid / S::NMT, e = A.e0 + el;
-    const int m0 = mt * MT;
-    const DeviceTables& T = A.tab;
-    const float* cfe = reinterpret_cast<const float*>(A.vcoef) + (size_t)el * M * M * D * NCOEF * NQ;
-    extern __shared__ __align__(1024) unsigned char smraw[];
-    float* stage0 = reinterpret_cast<float*>(smraw);
-    uint64_t* mbar = reinterpret_cast<uint64_t*>(smraw + S::smem_bytes() - 64);
-    uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
-
-    // Chunks run over one direction and 16 consecutive points each (every
-    // direction's points padded to whole chunks), so that a chunk needs no
-    // division per entry; thread tid forms row tid % 128 (decoded once) for the
-    // K quads tid / 128 and tid / 128 + 2, each quad's loads issued before they are used.
-    const int rl = tid & (MT - 1), r0 = m0 + rl;
-    const bool live = r0 < MR;
-    const int rab = live ? r0 / NCB : 0, rc = live ? r0 - rab * NCB : 0;
-    const bool vol = rc < NP;
-    const int rf = vol ? 0 : (rc - NP) / NFP, rlf = vol ? 0 : rc - NP - rf * NFP;
-    const float* rcf = cfe + (size_t)rab * D * NCOEF * NQ;
-
-    // operand tiles of chunk ci into stage buffer sb (Ah | Bh | Al | Bl)
-    auto generate = [&](int ci, float* sb) {
-        float* Ah = sb;
-        float* Bh = Ah + MT * KC;
-        float* Al = Bh + NTN * KC;
-        float* Bl = Al + MT * KC;
-        const int dir = ci / S::CPD, g0 = (ci - dir * S::CPD) * KC;
-        const float* cc = rcf + (size_t)dir * NCOEF * NQ;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {                  // one K quad at a time: its loads in flight together
-            const int q = (tid >> 7) + 2 * h;
-            float v[4];
-            if (vol) {
-                float c0[4], t0[4], cr[4][D], tr[4][D];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int g = min(g0 + 4 * q + u, NQ - 1);
-                    c0[u] = cc[g];
-                    t0[u] = T.fphi[g * NP + rc];
-#pragma unroll
-                    for (int r2 = 0; r2 < D; ++r2) {
-                        cr[u][r2] = cc[(1 + r2) * NQ + g];
-                        tr[u][r2] = T.fpsi[((size_t)r2 * NQ + g) * NP + rc];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float x = c0[u] * t0[u];
-#pragma unroll
-                    for (int r2 = 0; r2 < D; ++r2) x = fmaf(-cr[u][r2], tr[u][r2], x);
-                    v[u] = x;
-                }
-            } else {
-                float c1[4], t1[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int g = min(g0 + 4 * q + u, NQ - 1);
-                    c1[u] = cc[(1 + D + rf) * NQ + g];
-                    t1[u] = T.ftheta[((size_t)rf * NQ + g) * NFP + rlf];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = c1[u] * t1[u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (!live || g0 + 4 * q + u >= NQ) v[u] = 0.f;
-            const int off = ((rl >> 3) * (KC / 4) + q) * 32 + (rl & 7) * 4;
-            const float4 hi = make_float4(tf32_round(v[0]), tf32_round(v[1]), tf32_round(v[2]), tf32_round(v[3]));
-            *reinterpret_cast<float4*>(Ah + off) = hi;
-            *reinterpret_cast<float4*>(Al + off) = make_float4(tf32_round(v[0] - hi.x), tf32_round(v[1] - hi.y),
-                                                               tf32_round(v[2] - hi.z), tf32_round(v[3] - hi.w));
-        }
-        for (int it = tid; it < NTN * (KC / 4); it += TH) {
-            const int n = it % NTN, q = it / NTN;
-            float w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int g = g0 + q * 4 + u;
-                w[u] = (n < NP && g < NQ) ? T.fdphi[((size_t)dir * NQ + g) * NP + n] : 0.f;
-            }
-            const int off = ((n >> 3) * (KC / 4) + q) * 32 + (n & 7) * 4;
-            const float4 hi = make_float4(tf32_round(w[0]), tf32_round(w[1]), tf32_round(w[2]), tf32_round(w[3]));
-            *reinterpret_cast<float4*>(Bh + off) = hi;
-            *reinterpret_cast<float4*>(Bl + off) = make_float4(tf32_round(w[0] - hi.x), tf32_round(w[1] - hi.y),
-                                                               tf32_round(w[2] - hi.z), tf32_round(w[3] - hi.w));
-        }
-        asm volatile("fence.proxy.async.shared::cta;");
-    };
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tslot)),
-                     "r"(S::TCOLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar)), "r"(1));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_u32(mbar + 1)), "r"(1));
-        asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-    generate(0, stage0);
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem = *tslot;
-    const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NTN >> 3) << 17) | ((uint32_t)(MT >> 4) << 24);
-    // one barrier per stage buffer: the batch that reads buffer s commits to barrier s, and
-    // is waited for before buffer s is written again, so no barrier runs two phases ahead
-    uint32_t phase = 0u, pending = 0u;                          // bit s: barrier s
-    bool ok = true;
-    auto wait_stage = [&](int sb) {
-        if (!((pending >> sb) & 1u)) return;
-        const uint32_t bar = smem_u32(mbar + sb), par = (phase >> sb) & 1u;
-        if (!mbar_wait_bounded(bar, par, 1 << 24)) {
-            ok = false;
-            if (tid == 0) atomicOr(status, 4);
-            mbar_wait_bounded(bar, par, 1 << 24);
-        }
-        phase ^= 1u << sb;
-        pending &= ~(1u << sb);
-    };
-    for (int ci = 0; ci < S::NCH; ++ci) {
-        const int sbi = ci & 1;
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const float* Ah = stage0 + sbi * S::STAGE;
-            const float* Bh = Ah + MT * KC;
-            const float* Al = Bh + NTN * KC;
-            const float* Bl = Al + MT * KC;
-            for (int s = 0; s < KC / 8; ++s) {
-                const uint32_t off = s * 256;
-                const uint64_t ah = umma_desc(smem_u32(Ah) + off, 128, (KC / 4) * 128);
-                const uint64_t bh = umma_desc(smem_u32(Bh) + off, 128, (KC / 4) * 128);
-                const uint64_t al = umma_desc(smem_u32(Al) + off, 128, (KC / 4) * 128);
-                const uint64_t bl = umma_desc(smem_u32(Bl) + off, 128, (KC / 4) * 128);
-                uint32_t acc = (ci > 0 || s > 0) ? 1u : 0u;
-                asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                             "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
-                             :: "r"(tmem), "l"(ah), "l"(bh), "r"(idesc), "r"(acc));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;"
-                             :: "r"(tmem), "l"(ah), "l"(bl), "r"(idesc));
-                asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;"
-                             :: "r"(tmem), "l"(al), "l"(bh), "r"(idesc));
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(mbar + sbi)));
-        }
-        pending |= 1u << sbi;
-        if (ci + 1 < S::NCH) {
-            wait_stage(sbi ^ 1);                                 // the batch before this one read the other buffer
-            if (__syncthreads_or(ok ? 0 : 1)) {
-                ok = false;
-                break;
-            }
-            generate(ci + 1, stage0 + (sbi ^ 1) * S::STAGE);
-            __syncthreads();
-        }
-    }
-    wait_stage(0);                                               // every batch completes before the epilogue
-    wait_stage(1);
-    ok = !__syncthreads_or(ok ? 0 : 1);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok) {
-        // warp w reads lanes 32 (w % 4) .. + 31; warps 4..7 take the second half of the columns
-        const int lg = warp & 3, half = warp >> 2;
-        const int r = m0 + lg * 32 + lane;
-        const int ab = r / NCB, c = r - ab * NCB, a = ab / M, b = ab - a * M;
-        const double detJ = A.geo[e * GEO];
-        double* A11 = A.R.a11 + e * A.R.a11_es;
-        float* A12 = A.R.a12 + e * A.R.a12_es;
-        constexpr int HC = ((NTN / 2) + 15) / 16 * 16;
-#pragma unroll 1
-        for (int c0 = half * HC; c0 < min(NTN, (half + 1) * HC); c0 += 16) {
-            uint32_t v[16];
-            const uint32_t addr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                         : "r"(addr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (r < MR) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int i = c0 + j;
-                    if (i >= NP) continue;
-                    const float x = __uint_as_float(v[j]);
-                    const int64_t row = a * NP + i;
-                    if (c < NP) {
-                        double w = (double)x;
-                        if (a == b) w += detJ / A.a_ii * T.mhat[i * NP + c];
-                        A11[row * A.R.a11_rs + b * NP + c] = w;
-                    } else {
-                        const int c2 = c - NP, f = c2 / NFP, l = c2 - f * NFP;
-                        A12[row * A.R.a12_rs + (f * M + b) * NFP + l] = x;
-                    }
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(S::TCOLS));
-}
 
 }  // namespace hdg

@@ -145,7 +145,6 @@ void build_ref_tables(int d, int p, RefTables& t) {
     L.eval(-1.0, &Be[0], &De[0]);
     L.eval(1.0, &Be[n1], &De[n1]);
     t.b1 = B;
-    t.d1 = Dd;
 
     auto digit = [](int idx, int base, int r) { for (int k = 0; k < r; ++k) idx /= base; return idx % base; };
 
@@ -262,45 +261,6 @@ void build_ref_tables(int d, int p, RefTables& t) {
                 t.minv_e[((size_t)f * Np + i) * Nfp + l] = s;
             }
     }
-    // values at quadrature points
-    t.psi.assign((size_t)d * Nq * Np, 0.0);
-    for (int r = 0; r < d; ++r)
-        for (int g = 0; g < Nq; ++g)
-            for (int j = 0; j < Np; ++j) {
-                double s = 0.0;
-                for (int k = 0; k < Np; ++k)
-                    s += t.phi[(size_t)g * Np + k] * t.minv_c[((size_t)r * Np + k) * Np + j];
-                t.psi[((size_t)r * Nq + g) * Np + j] = s;
-            }
-    t.theta.assign((size_t)nf * Nq * Nfp, 0.0);
-    for (int f = 0; f < nf; ++f)
-        for (int g = 0; g < Nq; ++g)
-            for (int l = 0; l < Nfp; ++l) {
-                double s = 0.0;
-                for (int k = 0; k < Np; ++k)
-                    s += t.phi[(size_t)g * Np + k] * t.minv_e[((size_t)f * Np + k) * Nfp + l];
-                t.theta[((size_t)f * Nq + g) * Nfp + l] = s;
-            }
-    t.psi_f.assign((size_t)nf * d * Nfq * Np, 0.0);
-    for (int f = 0; f < nf; ++f)
-        for (int r = 0; r < d; ++r)
-            for (int q = 0; q < Nfq; ++q)
-                for (int j = 0; j < Np; ++j) {
-                    double s = 0.0;
-                    for (int k = 0; k < Np; ++k)
-                        s += phif[((size_t)f * Nfq + q) * Np + k] * t.minv_c[((size_t)r * Np + k) * Np + j];
-                    t.psi_f[(((size_t)f * d + r) * Nfq + q) * Np + j] = s;
-                }
-    t.theta_f.assign((size_t)nf * nf * Nfq * Nfp, 0.0);
-    for (int f = 0; f < nf; ++f)
-        for (int f2 = 0; f2 < nf; ++f2)
-            for (int q = 0; q < Nfq; ++q)
-                for (int l = 0; l < Nfp; ++l) {
-                    double s = 0.0;
-                    for (int k = 0; k < Np; ++k)
-                        s += phif[((size_t)f * Nfq + q) * Np + k] * t.minv_e[((size_t)f2 * Np + k) * Nfp + l];
-                    t.theta_f[(((size_t)f * nf + f2) * Nfq + q) * Nfp + l] = s;
-                }
 }
 
 }  // namespace hdg
