@@ -186,10 +186,10 @@ int ensure_system_storage(hdg_ctx* h, int precision) {
     if (h->d_m11) return HDG_OK;
     const size_t E = h->E, ch = h->chunk, NU = h->NU, NT = h->NT;
     if ((rc = dev_alloc(h, &h->d_m11, E * NU * NU))) return rc;
-    if ((rc = dev_alloc(h, &h->d_m12, E * NU * NT))) return rc;
+    if ((rc = dev_alloc(h, &h->d_m12, E * NU * mixed_stride(NT)))) return rc;
     if ((rc = dev_alloc(h, &h->d_mrt, E * NU))) return rc;
-    if ((rc = dev_alloc(h, &h->d_m21, ch * NT * NU))) return rc;
-    if ((rc = dev_alloc(h, &h->d_m22, ch * NT * NT))) return rc;
+    if ((rc = dev_alloc(h, &h->d_m21, ch * NT * mixed_stride(NU)))) return rc;
+    if ((rc = dev_alloc(h, &h->d_m22, ch * NT * mixed_stride(NT)))) return rc;
     if ((rc = dev_alloc(h, &h->d_mrb, ch * NT))) return rc;
     if ((rc = dev_alloc(h, &h->d_vals32, (size_t)h->nnzb * h->BS * h->BS))) return rc;
     if ((rc = dev_alloc(h, &h->d_x32, (size_t)h->F * h->BS))) return rc;

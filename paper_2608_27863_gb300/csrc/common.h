@@ -69,6 +69,9 @@ struct Phys {
     int tau_mode = 0;     // 0: constant tau; 1: state-dependent tau(uhat) = |v.n| + c + mu / h
 };
 
+// row stride of the mixed form's FP32 blocks: rows start on 16 bytes
+inline int64_t mixed_stride(int64_t n) { return (n + 3) / 4 * 4; }
+
 struct DeviceTables {
     double* phi;  double* dphi; double* wq;
     double* mu;   double* wf;
@@ -198,10 +201,10 @@ struct hdg_ctx {
                                            // tensor cores by exact digit splitting (k_schur_ozaki); the
                                            // default is set with the device storage
     double* d_m11 = nullptr;               // [E][NU][NU] interior block / its LU factors (FP64)
-    float* d_m12 = nullptr;                // [E][NU][NT] Bt, then Z = L^{-1} P Bt
+    float* d_m12 = nullptr;                // [E][NU][NT to 4] Bt, then Z = L^{-1} P Bt
     double* d_mrt = nullptr;               // [E][NU] Rt, then z
-    float* d_m21 = nullptr;                // [chunk][NT][NU] Ct, then W
-    float* d_m22 = nullptr;                // [chunk][NT][NT] Dt, then S^K
+    float* d_m21 = nullptr;                // [chunk][NT][NU to 4] Ct, then W
+    float* d_m22 = nullptr;                // [chunk][NT][NT to 4] Dt, then S^K
     double* d_mrb = nullptr;               // [chunk][NT] Rh, then -g^K
     int32_t* d_mpiv = nullptr;             // [E][NU] row permutation of the interior LU as a gather map (split
                                            // elimination)

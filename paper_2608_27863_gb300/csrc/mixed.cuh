@@ -918,9 +918,10 @@ inline Regions<float> mixed_regions(hdg_ctx* h) {
     const int64_t NU = h->NU, NT = h->NT;
     Regions<float> R;
     R.a11 = h->d_m11; R.a11_es = NU * NU; R.a11_rs = NU;
-    R.a12 = h->d_m12; R.a12_es = NU * NT; R.a12_rs = NT;
-    R.a21 = h->d_m21; R.a21_es = NT * NU; R.a21_rs = NU;
-    R.a22 = h->d_m22; R.a22_es = NT * NT; R.a22_rs = NT;
+    const int64_t su = mixed_stride(NU), st = mixed_stride(NT);
+    R.a12 = h->d_m12; R.a12_es = NU * st; R.a12_rs = st;
+    R.a21 = h->d_m21; R.a21_es = NT * su; R.a21_rs = su;
+    R.a22 = h->d_m22; R.a22_es = NT * st; R.a22_rs = st;
     R.rt = h->d_mrt;  R.rt_es = NU;       R.rt_rs = 1;
     R.rb = h->d_mrb;  R.rb_es = NT;       R.rb_rs = 1;
     return R;
@@ -1079,8 +1080,10 @@ namespace hdg {
 // columns are staged by the CTA's threads into shared memory in the canonical
 // K-major layout without swizzle (8-row x 16-byte core matrices; K-adjacent
 // cores 128 B apart, 8-row groups KC/4 x 128 B apart).  SPLIT3 selects 3xTF32:
-// x = hi + lo with hi = tf32(x), lo = tf32(x - hi), and W Z ~ Wh Zh + Wh Zl + Wl Zh.
-// One CTA (4 warps) per (element, 128-row tile, column tile).  Waits on the
+// x = hi + lo with hi = tf32(x), lo = tf32(x - hi), and W Z ~ Wh Zh + Wh Zl + Wl Zh; the
+// last two have an accumulator of their own, added at the end (the tensor cores' accumulation truncates,
+// and a third of the additions into the large sum truncates a third as often).
+// Waits on the
 // MMA completion barrier are bounded; on timeout the CTA latches status bit 4,
 // waits once more (bounded) and frees its tensor memory.
 // ----------------------------------------------------------------------------
@@ -1091,8 +1094,9 @@ struct SchurTC {
     static constexpr int NNT = (NT + 127) / 128;                          // column tiles (<= 128 TMEM columns each)
     static constexpr int NTN = (((NT + NNT - 1) / NNT) + 15) / 16 * 16;   // columns per tile (mult. of 16)
     static constexpr int NMT = (NT + MT - 1) / MT;                        // row tiles
-    static constexpr int TCOLS = NTN <= 32 ? 32 : NTN <= 64 ? 64 : NTN <= 128 ? 128 : 256;
-    static_assert(NTN <= 256, "column tile too wide");
+    static constexpr int TC1 = NTN <= 32 ? 32 : NTN <= 64 ? 64 : 128;     // columns of an accumulator
+    __host__ __device__ static constexpr int tcols(bool split3) { return split3 ? 2 * TC1 : TC1; }
+    static_assert(NTN <= 128, "column tile too wide");
     static constexpr int THREADS = 256;
     static constexpr int WRS = KC + 4;                                    // raw W row stride (floats)
     __host__ __device__ static constexpr int tile_floats(int rows) { return rows * KC; }
@@ -1100,19 +1104,46 @@ struct SchurTC {
     __host__ __device__ static constexpr int smem_bytes(bool split3) {
         return (split3 ? 2 : 1) * (tile_floats(MT) + tile_floats(NTN)) * 4 + raw_floats() * 4 + 64;
     }
+    // right-hand side: a column tile takes RPC of the 128 rows, PARTS threads a row with KP terms of a chunk each
+    static constexpr int RPC = (MT + NNT - 1) / NNT;
+    static constexpr int PARTS = THREADS / RPC >= 8 ? 8 : THREADS / RPC >= 4 ? 4 : 2;
+    static constexpr int KP = KC / PARTS;
+    static constexpr int OS = NTN + 1;                                    // row stride of the staged product
+    static_assert(RPC * PARTS <= THREADS && PARTS * KP == KC && KP % 4 == 0, "right-hand side layout");
+    static_assert(MT * OS <= tile_floats(MT) + tile_floats(NTN) + raw_floats(),
+                  "the product fits where the operands were");
+    static_assert(RPC * PARTS * 8 <= MT * WRS * 4, "partial sums of the right-hand side fit the raw tile");
 };
 
+// 16 accumulator columns of this warp's 32 lanes; complete after tcgen05.wait::ld
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+                 : "r"(addr));
+}
 
+// keeps the compiler from using the columns before the wait
+__device__ __forceinline__ void tmem_arrived(float (&v)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) asm volatile("" : "+f"(v[j]));
+}
 
-__device__ __forceinline__ void cp_async4(void* dst, const void* src, int src_bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" :: "r"(smem_u32(dst)), "l"(src), "r"(src_bytes));
+// 16 bytes, of which src_bytes are read and the rest is zero; both addresses on 16 bytes
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(smem_u32(dst)), "l"(src), "r"(src_bytes));
 }
 
 // One CTA (8 warps) per (element, 128-row tile, column tile).  The raw FP32 tiles of
 // the next K chunk (W rows, Z rows) are copied into shared memory asynchronously
-// (cp.async) while the tensor cores run the current chunk; the threads then split
+// (16-byte cp.async: the rows start on 16 bytes, see mixed_stride) while the tensor cores run the
+// current chunk; the threads then split
 // them into TF32 hi (/ lo) parts and store them in the core-matrix layout, rows
-// fastest so that the 16-byte stores of a quarter warp are contiguous.
+// fastest so that the 16-byte stores of a quarter warp are contiguous.  The right-hand side takes
+// its W from the raw tile too, the rows dealt out over the column tiles.  The product leaves tensor
+// memory through shared memory, so that Dt is read and written in whole lines.
+// 4,096 hexes p = 2: 4.97 -> 2.59 ms, 1,320 hexes p = 3: 7.81 -> 2.61 ms (4-byte copies, W read again
+// from global memory a row per thread for the right-hand side, Dt updated a row per thread).
 template <class C, bool SPLIT3>
 __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float> R, int64_t e0, int32_t* status) {
     using S = SchurTC<C>;
@@ -1137,34 +1168,28 @@ __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float>
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
 
     auto prefetch = [&](int k0) {
-        for (int it = tid; it < MT * KC; it += TH) {
-            const int r = it / KC, k = it - r * KC;
-            const bool in = m0 + r < NT && k0 + k < NU;
-            cp_async4(Wr + r * WRS + k, in ? (const void*)(W + (m0 + r) * sw + k0 + k) : (const void*)W, in ? 4 : 0);
+        for (int it = tid; it < MT * (KC / 4); it += TH) {
+            const int r = it / (KC / 4), k = (it - r * (KC / 4)) * 4;
+            const int nb = m0 + r < NT ? 4 * max(0, min(4, NU - k0 - k)) : 0;
+            cp_async16(Wr + r * WRS + k, nb ? (const void*)(W + (m0 + r) * sw + k0 + k) : (const void*)W, nb);
         }
-        for (int it = tid; it < KC * NTN; it += TH) {
-            const int k = it / NTN, n = it - k * NTN;
-            const bool in = k0 + k < NU && n0 + n < NT;
-            cp_async4(Zr + k * NTN + n, in ? (const void*)(Z + (k0 + k) * sz + n0 + n) : (const void*)Z, in ? 4 : 0);
+        for (int it = tid; it < KC * (NTN / 4); it += TH) {
+            const int k = it / (NTN / 4), n = (it - k * (NTN / 4)) * 4;
+            const int nb = k0 + k < NU ? 4 * max(0, min(4, NT - n0 - n)) : 0;
+            cp_async16(Zr + k * NTN + n, nb ? (const void*)(Z + (k0 + k) * sz + n0 + n) : (const void*)Z, nb);
         }
         asm volatile("cp.async.commit_group;");
     };
     prefetch(0);
 
-    // right-hand side of this row tile: Rh -= W z (FP64), done by the first column tile
-    if (nt == 0) {
-        const double* z = R.rt + e * R.rt_es;
-        double* rb = R.rb + el * R.rb_es;
-        const int r = m0 + tid;
-        if (tid < MT && r < NT) {
-            double s = rb[r * R.rb_rs];
-            for (int k = 0; k < NU; ++k) s -= (double)W[r * sw + k] * z[k * R.rt_rs];
-            rb[r * R.rb_rs] = s;
-        }
-    }
+    // right-hand side: Rh -= W z (FP64); this thread's row of the tile and part of every chunk
+    const double* z = R.rt + e * R.rt_es;
+    const int rpart = tid / S::RPC, rrow = nt * S::RPC + tid % S::RPC;
+    const bool rhs = rpart < S::PARTS && rrow < MT && m0 + rrow < NT;
+    double rsum = 0.0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(tslot)),
-                     "r"(S::TCOLS));
+                     "r"(S::tcols(SPLIT3)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
@@ -1193,6 +1218,17 @@ __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float>
         if (__syncthreads_or(ok ? 0 : 1)) {                     // raw tiles visible, operand tiles free
             ok = false;
             break;
+        }
+        if (rhs) {
+            const int kb = rpart * S::KP;
+#pragma unroll
+            for (int k = 0; k < S::KP; k += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(Wr + rrow * WRS + kb + k);
+                const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k0 + kb + k + u < NU) rsum = fma((double)w[u], z[(k0 + kb + k + u) * R.rt_rs], rsum);
+            }
         }
         // item = (row, 4-wide K group q) -> one 16-byte core-matrix row; rows fastest
         for (int it = tid; it < MT * (KC / 4); it += TH) {
@@ -1233,10 +1269,11 @@ __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float>
                 if (SPLIT3) {
                     const uint64_t al = umma_desc(smem_u32(Al) + off, 128, (KC / 4) * 128);
                     const uint64_t bl = umma_desc(smem_u32(Bl) + off, 128, (KC / 4) * 128);
+                    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
+                                 :: "r"(tmem + S::TC1), "l"(ah), "l"(bl), "r"(idesc), "r"(acc));
                     asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;"
-                                 :: "r"(tmem), "l"(ah), "l"(bl), "r"(idesc));
-                    asm volatile("tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, 1;"
-                                 :: "r"(tmem), "l"(al), "l"(bh), "r"(idesc));
+                                 :: "r"(tmem + S::TC1), "l"(al), "l"(bh), "r"(idesc));
                 }
             }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar));
@@ -1255,31 +1292,58 @@ __global__ void __launch_bounds__(SchurTC<C>::THREADS) k_schur_tc(Regions<float>
     ok = !__syncthreads_or(ok ? 0 : 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
-        // warp w reads lanes 32 (w % 4) .. + 31 and the column half w / 4 of the tile
+        // the parts of a row of the right-hand side, in order
+        double* rp = reinterpret_cast<double*>(Wr);
+        if (rhs) rp[rpart * S::RPC + tid % S::RPC] = rsum;
+        __syncthreads();
+        if (rhs && rpart == 0) {
+            double s = R.rb[el * R.rb_es + (m0 + rrow) * R.rb_rs];
+            for (int q = 0; q < S::PARTS; ++q) s -= rp[q * S::RPC + tid];
+            R.rb[el * R.rb_es + (m0 + rrow) * R.rb_rs] = s;
+        }
+        __syncthreads();
+        // the product into shared memory: warp w reads lanes 32 (w % 4) .. + 31 and the column half w / 4 of the tile
+        float* O = reinterpret_cast<float*>(smraw);
         const int lg = warp & 3, half = warp >> 2;
-        const int r = m0 + lg * 32 + lane;
+        const int r = lg * 32 + lane;
         constexpr int HC = ((NTN / 2) + 15) / 16 * 16;          // columns per half, in chunks of 16
 #pragma unroll 1
         for (int c0 = half * HC; c0 < min(NTN, (half + 1) * HC); c0 += 16) {
-            uint32_t v[16];
+            float v[16], x[16];
             const uint32_t addr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                         : "r"(addr));
+            tmem_ld16(addr, v);
+            if (SPLIT3) tmem_ld16(addr + S::TC1, x);
             asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (r < NT) {
+            tmem_arrived(v);
+            if (SPLIT3) tmem_arrived(x);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int c = n0 + c0 + j;
-                    if (c0 + j < NTN && c < NT) Dm[r * sd + c] -= __uint_as_float(v[j]);
+            for (int j = 0; j < 16; ++j) O[r * S::OS + c0 + j] = SPLIT3 ? v[j] + x[j] : v[j];
+        }
+        __syncthreads();
+        // Dt -= product, a warp a row, two rows' loads in flight
+        constexpr int NL = (NTN + 31) / 32;
+        const int nr = min(MT, NT - m0), nc = min(NTN, NT - n0);
+        for (int r0 = warp; r0 < nr; r0 += 2 * (TH / 32)) {
+            float d[2][NL];
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const int rr = r0 + u * (TH / 32), c = lane + 32 * j;
+                    d[u][j] = rr < nr && c < nc ? Dm[(m0 + rr) * sd + n0 + c] : 0.f;
                 }
-            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const int rr = r0 + u * (TH / 32), c = lane + 32 * j;
+                    if (rr < nr && c < nc) Dm[(m0 + rr) * sd + n0 + c] = d[u][j] - O[rr * S::OS + c];
+                }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(S::TCOLS));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(S::tcols(SPLIT3)));
 }
 
 
