@@ -506,7 +506,7 @@ struct TrsmShape {
     static constexpr int CW = 64;                           // right-hand sides per CTA
     static constexpr int NTH = 256;
     static constexpr int NBLK = (C::NU + 31) / 32;
-    static constexpr int JC = 64;                           // factor columns staged at a time
+    static constexpr int JC = 64;                           // factor columns staged at a time (64 or 32)
     static constexpr int FS = 36;                           // row stride of the staged factor
     static constexpr int smem_floats = NBLK * 32 * CW + JC * FS;
 };
@@ -514,10 +514,11 @@ struct TrsmShape {
 // ZS: Z = L^{-1} P Bt for columns [c0, c0 + 64) of Bt; else W = Ct U^{-1} for rows [c0, c0 + 64) of
 // Ct (FP32, in place; the factors FP64 in HBM).  X[i][c] holds the block of right-hand sides (W's
 // transposed); 32 rows of X at a time: the solved rows' contribution as a product with the staged
-// factor (a thread owns 4 rows x 2 columns: one 8-byte and one broadcast 16-byte shared load feed
-// eight multiply-adds), then the substitution with the diagonal triangle, four lanes per right-hand
+// factor (a thread owns 4 rows x 4 columns of one half of the factor's columns: two 16-byte shared
+// loads, one of them broadcast, feed sixteen multiply-adds; with 4 x 2 and no halves shared memory
+// bound it), then the substitution with the diagonal triangle, four lanes per right-hand
 // side with eight rows each, the solved value passed by a shuffle.  4,096 hexes p = 2: Z and W 5.6 ->
-// 5.6 ms; 1,320 hexes p = 3: 23.0 -> 11.4 ms (the substitution ran on two warps, and every CTA walked the
+// 5.4 ms; 1,320 hexes p = 3: 23.0 -> 9.8 ms (the substitution ran on two warps, and every CTA walked the
 // interchange list in global memory).  Inverted diagonal triangles are as fast but lose accuracy
 // (error of the right-hand side 0.8e-6 -> 3.5e-6 on quads p = 3).
 template <class C, bool ZS>
@@ -542,12 +543,12 @@ __global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, co
     float pre[NPRE];
     auto width = [&](int i0, int j0) { return j0 < i0 ? min(JC, i0 - j0) : 32; };
     auto load = [&](int i0, int j0) {
-        const int jc = width(i0, j0);
+        const int jc = width(i0, j0), sh = jc == 64 ? 6 : 5;
 #pragma unroll
         for (int u = 0; u < NPRE; ++u) {
             const int idx = tid + u * NTH;
             int r, j;
-            if (ZS) { r = idx / jc; j = idx - r * jc; } else { j = idx >> 5; r = idx & 31; }
+            if (ZS) { r = idx >> sh; j = idx & (jc - 1); } else { j = idx >> 5; r = idx & 31; }
             pre[u] = idx >= 32 * jc || i0 + r >= NU || j0 + j >= NU ? 0.f
                      : (float)(ZS ? A[(int64_t)(i0 + r) * rs + j0 + j] : A[(int64_t)(j0 + j) * rs + i0 + r]);
         }
@@ -564,11 +565,22 @@ __global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, co
             X[i * CW + c] = i < NU && c < cw ? Y[(int64_t)(c0 + c) * ys + i] : 0.f;
         }
     }
-    float acc[4][2] = {};
+    // rows prow.. + 3, columns pcol.. + 3; group 0 the first half of a chunk's factor columns, 1 the second
+    const int group = warp >> 2, prow = 8 * (warp & 3) + 4 * (lane >> 4), pcol = 4 * (lane & 15);
+    float acc[4][4] = {};
+    auto apply = [&](int i0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float4* x = reinterpret_cast<float4*>(X + (i0 + prow + u) * CW + pcol);
+            const float4 v = *x;
+            *x = make_float4(v.x - acc[u][0], v.y - acc[u][1], v.z - acc[u][2], v.w - acc[u][3]);
+            acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
+        }
+    };
     int i0 = 0, j0 = 0;
 #pragma unroll 1
     while (i0 < NUP) {
-        const int jc = width(i0, j0);
+        const int jc = width(i0, j0), sh = jc == 64 ? 6 : 5;
         const bool diag = j0 == i0;
         __syncthreads();                  // X complete, F free
 #pragma unroll
@@ -576,7 +588,7 @@ __global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, co
             const int idx = tid + u * NTH;
             if (idx >= 32 * jc) continue;
             int r, j;
-            if (ZS) { r = idx / jc; j = idx - r * jc; } else { j = idx >> 5; r = idx & 31; }
+            if (ZS) { r = idx >> sh; j = idx & (jc - 1); } else { j = idx >> 5; r = idx & 31; }
             F[j * FS + r] = pre[u];
         }
         if (diag) {
@@ -584,26 +596,27 @@ __global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, co
                 const float d = i0 + tid < NU ? (float)A[(int64_t)(i0 + tid) * rs + i0 + tid] : 1.f;
                 rd[tid] = d != 0.f ? 1.f / d : 1.f;
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                float2* x = reinterpret_cast<float2*>(X + (i0 + 4 * warp + u) * CW + 2 * lane);
-                const float2 v = *x;
-                *x = make_float2(v.x - acc[u][0], v.y - acc[u][1]);
-                acc[u][0] = acc[u][1] = 0.f;
+            if (i0 > 0) {                 // the first block has no solved rows before it
+                if (group == 0) apply(i0);
+                __syncthreads();
+                if (group == 1) apply(i0);
             }
         }
         __syncthreads();
         const int ni = diag ? i0 + 32 : i0, nj = diag ? 0 : j0 + jc;
         if (ni < NUP) load(ni, nj);       // the next chunk under this one's arithmetic
         if (!diag) {
+            const int jb = group * (jc >> 1);
 #pragma unroll 8
-            for (int j = 0; j < jc; ++j) {
-                const float2 x = *reinterpret_cast<const float2*>(X + (j0 + j) * CW + 2 * lane);
-                const float4 f = *reinterpret_cast<const float4*>(F + j * FS + 4 * warp);
-                acc[0][0] = fmaf(f.x, x.x, acc[0][0]); acc[0][1] = fmaf(f.x, x.y, acc[0][1]);
-                acc[1][0] = fmaf(f.y, x.x, acc[1][0]); acc[1][1] = fmaf(f.y, x.y, acc[1][1]);
-                acc[2][0] = fmaf(f.z, x.x, acc[2][0]); acc[2][1] = fmaf(f.z, x.y, acc[2][1]);
-                acc[3][0] = fmaf(f.w, x.x, acc[3][0]); acc[3][1] = fmaf(f.w, x.y, acc[3][1]);
+            for (int j = jb; j < jb + (jc >> 1); ++j) {
+                const float4 x = *reinterpret_cast<const float4*>(X + (j0 + j) * CW + pcol);
+                const float4 f = *reinterpret_cast<const float4*>(F + j * FS + prow);
+                const float fu[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    acc[u][0] = fmaf(fu[u], x.x, acc[u][0]); acc[u][1] = fmaf(fu[u], x.y, acc[u][1]);
+                    acc[u][2] = fmaf(fu[u], x.z, acc[u][2]); acc[u][3] = fmaf(fu[u], x.w, acc[u][3]);
+                }
             }
         } else {
             const int c = tid >> 2, q = tid & 3;
