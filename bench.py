@@ -37,13 +37,13 @@ sys.path.insert(0, ROOT)
 METRIC = "HDG linearize+condense elements/s & % of FP64/TC peak; mixed vs FP64 at tol"
 
 # DRAM bytes (read + write) per element of the dominant kernel, from one ncu
-# capture of the unchanged kernel on the 8^3 hex p=2 case (512 elements, above
+# capture of the kernel on the 8^3 hex p=2 case (512 elements, above
 # L2); every CTA works on its own element, so traffic scales with the element
 # count of a launch.
 # Keyed by (kernel, d, p, elimination panel width).
 DRAM_BYTES_PER_ELEMENT = {("elim", 3, 2, 16): 16.45e6, ("elim", 3, 2, 8): 30.84e6,
-                          # FP64 element blocks, sum-factorised: k_blocks_sf (0.377 GB) + the face-term
-                          # pass k_blocks (0.936 GB) on the 512-element 8^3 launch
+                          # FP64 element blocks before k_contract: two kernels, 0.377 + 0.936 GB on the
+                          # 512-element 8^3 launch
                           ("blocks_sf", 3, 2, 0): (0.3775e9 + 0.9359e9) / 512}
 # The persistent tetrahedral kernel k_tet_linearize<double>: 87.5 GB (read + write) in one
 # ncu-captured launch over the 3,600 elements of the 10 x 20 x 3 mesh, whose degree mix and
@@ -145,8 +145,8 @@ def hex_recover_bytes(d, p, E):
 
 def tet_flops(layout, elem_p):
     """Algorithmic FP64 flops per element of the tetrahedral linearize + condense kernel:
-    point values and lifting operators, contraction (element and trace rows, with the
-    per-point column variations), and the bordered elimination."""
+    point values and lifting operators, contraction (coupling matrices, and their products
+    with the lifting operators into element and trace rows), and the bordered elimination."""
     import numpy as np
     E = len(elem_p)
     fp = layout["face_p"][layout["e2f"]]                      # [E][4]
@@ -158,9 +158,16 @@ def tet_flops(layout, elem_p):
     Nc = Np + sfp
     NU, t = 5 * Np, 5 * sfp
     lift = 3 * Np * Np * Nq + 9 * Np * Np * Nq + 9 * Np * sfp * nfq.max(1) + Np ** 3 / 3 + 6 * Nc * Np * Np \
-        + 2 * 15 * Np * (Np + sfp) + 2 * 3 * (Nq + sfq) * Nc * Np
-    contr = 2 * 25 * Np * Nc * (3 * Nq + sfq) + 2 * 25 * (nfp * nfq).sum(1) * Nc \
-        + 25 * Nc * (3 * Nq * 8 + sfq * 10 + sfq * 10)
+        + 2 * 15 * Np * (Np + sfp)
+    n1, nt2 = elem_p + 1, (elem_p + 1) * (elem_p + 2) // 2    # 1-D functions; nodes of an element face
+    q = elem_p + 2
+    nP = nt2[:, None]
+    contr = 2 * (76 * Np * (3 * Nq + Nq * n1 + q * q * nt2 + q * Np)             # volume matrices
+                 + (nfp * nfq * (25 * (1 + nfp) + 56 * (1 + nP))).sum(1)          # face matrices
+                 + 17 * 3 * (nfp * nP).sum(1) * Nc                                # trace rows
+                 + 3 * Np * Np * Nc                                               # lifting operators, modal
+                 + 25 * Np ** 3 + 17 * 3 * Np * Np * Nc                           # element rows
+                 + 25 * Nc * (nP * np.where(fp == elem_p[:, None], 1, nfp)).sum(1))   # and dt times the flux rows
     elim = np.zeros(E)
     for e in range(E):
         k = np.arange(NU[e])
@@ -331,7 +338,7 @@ def run_tet(args, rank, world, local_rank):
              "kernels": {k: {"ms_per_step": v[0] / n_mixed, "launches_per_step": v[1] / n_mixed}
                          for k, v in prof_m.items() if v[1]},
              "dtype": "fp64 pointwise terms, lifting operators, elimination and residual; fp32 Jacobian "
-                      "coefficients, column variations and contraction",
+                      "coefficients, contraction and trace rows",
              "clocks": clocks_m}
     if mixed is not None and oracle_check is not None:
         mixed["block_err_vs_oracle"] = oracle_check["mixed"]["max_rel_err"]
@@ -444,9 +451,16 @@ def make_problem(name, cpu_sample=False):
 # algorithmic FLOP counts per element (the executed reduced-structure counts)
 # ----------------------------------------------------------------------------
 def ozaki_digits(K):
-    """Digit width and count of the tensor-core Schur product for inner size K."""
+    """Digit width and count that represent 54 bits of the operands for inner size K."""
     b = 8 if 5 * K * 255 ** 2 < 2 ** 24 else 7 if 5 * K * 127 ** 2 < 2 ** 24 else 6
     return b, -(-54 // b)
+
+
+def schur_digits(K):
+    """Digit width and count of the tensor-core Schur product: at least 60 bits, over
+    eight accumulator groups of at most 7 digit pairs each (5 at width 8)."""
+    b = 8 if 5 * K * 255 ** 2 < 2 ** 24 else 7 if 7 * K * 127 ** 2 < 2 ** 24 else 6
+    return b, -(-60 // b)
 
 
 def flop_counts(d, p, sum_factorised=False, tc_schur=False):
@@ -456,22 +470,27 @@ def flop_counts(d, p, sum_factorised=False, tc_schur=False):
     NR, NC = NU + NT, NU + NT + 1
     elim = sum(2 * (NR - k - 1) * (NC - k - 1) + (NR - k - 1) for k in range(NU))
     schur = 2 * NT * NT * NU                  # the trace-trace part of the trailing updates
-    b, s = ozaki_digits(NU)
+    _, s = schur_digits(NU)
     pairs = s * (s + 1) // 2                  # digit pairs kept (i + j <= s + 1)
     mt, nt = -(-NT // 128) * 128, -(-NT // 32) * 32
     schur_bf16 = pairs * 2 * mt * nt * (-(-NU // 16) * 16)   # executed BF16 MMA work, padded tiles
     if tc_schur:
         elim -= schur
     NCB = Np + nf * Nfp
-    K = d * Nq
-    if sum_factorised:       # one 1-D contraction per axis, per column and direction
-        axes = q1 * q1 * n1 * q1 + q1 * n1 * n1 * q1 + n1 ** 3 * q1 if d == 3 else q1 * n1 * q1 + n1 * n1 * q1
-        contraction = 2 * axes * NCB * d
-    else:
-        contraction = 2 * Np * NCB * K
-    blocks = m * m * (contraction                       # contraction
-                      + K * (2 * (1 + d) * Np + nf * Nfp)  # generated operand
-                      + nf * (2 * Nfq * NCB * (d + 1) + 2 * Nfp * NCB * Nfq))  # face terms
+    if sum_factorised:       # what k_contract runs
+        def sums(na, ax):    # multiply-adds of one set of point values against 1-D functions, axis by axis
+            e = [n1 + (2 if k == ax else 0) for k in range(na)] + [1] * (3 - na)
+            g = [q1] * na + [1] * (3 - na)
+            return g[0] * g[1] * g[2] * e[0] + g[1] * g[2] * e[0] * e[1] + g[2] * e[0] * e[1] * e[2]
+        vis = d * (d + 1) + m                 # component pairs with a viscous part
+        kinds = m * m + d * vis
+        vol = Np * (kinds * d * Nq + m * m * sums(d, -1) + vis * sum(sums(d, r) for r in range(d)))
+        face = nf * Nfp * ((kinds * Nfq) + m * m * sums(d - 1, -1)
+                           + vis * (sums(d - 1, -1) + Nfp * (n1 + 2) + sum(sums(d - 1, r) for r in range(d - 1))))
+        blocks = 2 * (vol + face + m * m * (nf * Nfp + Np) * NCB)   # last: dt times the flux rows of a node's faces
+    else:                    # the same blocks as products of tables with every column at every point
+        blocks = m * m * (2 * d * Np * NCB * Nq + d * Nq * (2 * (1 + d) * Np + nf * Nfp)
+                          + nf * (2 * Nfq * NCB * (d + 1) + 2 * Nfp * NCB * Nfq))
     out = {"elim": elim, "blocks": blocks, "total": elim + blocks + (schur if tc_schur else 0)}
     if tc_schur:
         out.update(schur=schur, schur_bf16=schur_bf16)
@@ -905,7 +924,7 @@ def run_ours(args, rank, world, local_rank):
         return out
     t64 = tuning.get("fp64") or {}
     oz = t64.get("schur_mode", 0) == 3          # FP64 Schur product on the tensor cores
-    fl = flop_counts(m.dim, P.p, sum_factorised=t64.get("blocks64_mode", 1) == 1, tc_schur=oz)
+    fl = flop_counts(m.dim, P.p, sum_factorised=True, tc_schur=oz)
     nb_used = t64.get("elim_nb", args.elim_nb or 16)
     kern = {}
     for k, (ms, n) in prof.items():
@@ -919,10 +938,9 @@ def run_ours(args, rank, world, local_rank):
         kern["schur"]["bf16_tflops_executed"] = fl["schur_bf16"] * E / (prof["schur"][0] / args.steps) / 1e9
         kern["schur"]["bf16_frac_of_probe"] = kern["schur"]["bf16_tflops_executed"] / peaks["bf16_tcgen05"]
     dom = max(("elim", "blocks"), key=lambda k: prof[k][0])
-    sf64 = t64.get("blocks64_mode", 1) == 1
-    dom_name = dom + ("_sf" if dom == "blocks" and sf64 else "")
+    dom_name = {"elim": "elim", "blocks": "contract"}[dom]
     traffic_key = (dom_name, m.dim, P.p, nb_used if dom == "elim" and not oz else 0)
-    dom_kernels = {"elim": "k_elim", "blocks_sf": "k_blocks_sf + k_blocks (face terms)", "blocks": "k_blocks"}
+    dom_kernels = {"elim": "k_elim", "contract": "k_contract"}
     avg_launch_ms = prof[dom][0] / max(prof[dom][1], 1)
     per_launch_elems = E / max(prof[dom][1] / args.steps, 1)
     achieved = fl[dom] * per_launch_elems / (avg_launch_ms * 1e-3) / 1e12

@@ -7,6 +7,8 @@
 // panel the interior rows hold [U | Z = L^{-1} P Bt | z = L^{-1} P Rt] and the
 // trace rows' multipliers W = Ct U^{-1}, so that the Schur complement is one
 // product S^K = Dt - W Z (K = n_u) and -g^K = Rh - W z, left to k_schur_*.
+// The default is the same in pieces: the FP64 LU of At alone (k_lu_small in
+// shared memory, k_lu_mixed above n_u = 135), then Z and W by k_trsm in FP32.
 #pragma once
 
 #include "kernels.cuh"

@@ -619,7 +619,7 @@ __device__ __forceinline__ void tc_tile_done() {
 
 // The trace rows' Schur product of the mixed form on the tensor cores:
 // S = Dt - W Z with W = Wt^T ([n_u][t], trace rows contiguous) and Z ([n_u][t]),
-// 3xTF32 as the contraction; tiles of 128 trace rows x 96 trace columns.
+// 3xTF32; tiles of 128 trace rows x 96 trace columns.
 __device__ void schur_tc(double* Mx, int NU, int t, int LD, const float* Wt, const float* Zf, float* st0,
                          TcState& ts, int* sflag) {
     const int tid = threadIdx.x;
@@ -872,8 +872,7 @@ __device__ void trace_schur_f32(double* Mx, int NU, int t, int LD, const int* gp
     schur_tc(Mx, NU, t, LD, Wt, Zf, smf, ts, sflag);
 }
 
-// TJ: type of the Jacobian coefficients, the column variations and the
-// contraction (double: FP64 form; float: mixed form).  Pointwise terms, lifting
+// TJ: type of the Jacobian coefficients and the contraction (double: FP64 form; float: mixed form).  Pointwise terms, lifting
 // operators, mass term, right-hand side and the elimination are FP64 in both.
 template <class TJ, int NBE>
 __device__ void process_element(const KArgs& A, const TetElem& d, double* W, double* sm, int* sflag, TcState* ts) {
@@ -1296,7 +1295,7 @@ __global__ void __launch_bounds__(NTH, 2) k_tet_linearize(KArgs A) {
     if (tid == 0) sflag = 0;
     TcState ts{0u, 0u, 0u};
     if constexpr (sizeof(TJ) == sizeof(float)) {
-        // tensor memory and the two stage barriers of the contraction, held for the whole launch
+        // tensor memory and the two stage barriers of the Schur product, held for the whole launch
         if ((tid >> 5) == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(smem_u32(&tslot)),
                          "r"(TTCOLS));
