@@ -44,12 +44,14 @@ METRIC = "HDG linearize+condense elements/s & % of FP64/TC peak; mixed vs FP64 a
 DRAM_BYTES_PER_ELEMENT = {("elim", 3, 2, 16): 16.45e6, ("elim", 3, 2, 8): 30.84e6,
                           # FP64 element blocks before k_contract: two kernels, 0.377 + 0.936 GB on the
                           # 512-element 8^3 launch
-                          ("blocks_sf", 3, 2, 0): (0.3775e9 + 0.9359e9) / 512}
-# The persistent tetrahedral kernel k_tet_linearize<double>: 87.5 GB (read + write) in one
+                          ("blocks_sf", 3, 2, 0): (0.3775e9 + 0.9359e9) / 512,
+                          # k_elim without the Schur product (panels of 8 columns), and k_contract
+                          ("elim", 3, 2, 0): 5.008e9 / 512, ("contract", 3, 2, 0): 0.8197e9 / 512}
+# The persistent tetrahedral kernel k_tet_linearize<double>: 55.8 GB (read + write) in one
 # ncu-captured launch over the 3,600 elements of the 10 x 20 x 3 mesh, whose degree mix and
 # curved fraction come from the same seeded generator as the 100,800-element mesh; the
 # traffic is the per-CTA workspace streamed per element, so it scales with the elements.
-TET_DRAM_BYTES_PER_ELEMENT = 87.5e9 / 3600
+TET_DRAM_BYTES_PER_ELEMENT = 55.77e9 / 3600
 L2_BYTES = 129 * 1024 * 1024
 
 # fn/kw: the synth generator; mixed_only: the FP64 arrays would not fit in HBM, so only
