@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(ContractShape<C, TA>::NTH) k_contract(BlkArgs<
             pair_at<D>(q0 + p2, a, b);
             for (int idx = tid; idx < NP * NCB; idx += NTH) {
                 const int ii = idx / NCB, c = idx - ii * NCB;
-                TA v = buf[((size_t)p2 * NCB + c) * BS + ii];
+                const TA v = buf[((size_t)p2 * NCB + c) * BS + ii];
                 const int64_t col = c < NP ? b * NP + c : (((c - NP) / NFP) * M + b) * NFP + (c - NP) % NFP;
                 TA fs = TA(0);
                 for (int k = 0; k < D; ++k) {
@@ -314,14 +314,13 @@ __global__ void __launch_bounds__(ContractShape<C, TA>::NTH) k_contract(BlkArgs<
                     const int64_t trow = ((nfc / NFP) * M + a) * NFP + nfc % NFP;
                     fs += (TA)(c < NP ? A21[trow * A.R.a21_rs + col] : A22[trow * A.R.a22_rs + col]);
                 }
-                v = fma((TA)A.dt, fs, v);
                 const int64_t row = a * NP + ii;
-                if (c < NP) {
-                    double w = (double)v;
+                if (c < NP) {                                // the interior block is FP64 in both forms: so are its sums
+                    double w = fma(A.dt, (double)fs, (double)v);
                     if (a == b) w += detJ / A.a_ii * T.mhat[ii * NP + c];
                     A11[row * A.R.a11_rs + col] = w;
                 } else {
-                    A12[row * A.R.a12_rs + col] = (TL)v;
+                    A12[row * A.R.a12_rs + col] = (TL)fma((TA)A.dt, fs, v);
                 }
             }
         }
