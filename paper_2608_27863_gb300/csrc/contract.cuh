@@ -230,11 +230,11 @@ __global__ void __launch_bounds__(ContractShape<C, TA>::NTH) k_contract(BlkArgs<
                 }
             }
             if (a == b) {                                    // tau u: the face mass, weighted by tau at the points if it varies
-                if (A.taup) {
+                if (A.taup) {                                // in FP64 in both forms: rounded once, as the constant tau's is
                     const double* tp = A.taup + (el * NF + f) * NFQ;
-                    tensor_sums<D - 1, N1, Q1, -1, TA>(tb, tx,
-                        [&](int s1, int s2, int) { const int s = s1 + Q1 * s2; return row(s1, s2) * (TA)(nrm * T.wf[s] * tp[s]); },
-                        [&](int l1, int l2, int, TA v) { out[ucol(l1, l2, jn) * BS] += v; });
+                    tensor_sums<D - 1, N1, Q1, -1, double>(T.b1, nullptr,
+                        [&](int s1, int s2, int) { const int s = s1 + Q1 * s2; return T.mu[s * NFP + lam] * (nrm * T.wf[s] * tp[s]); },
+                        [&](int l1, int l2, int, double v) { out[ucol(l1, l2, jn) * BS] += (TA)v; });
                 } else {
                     const TA taun = (TA)(A.tau * nrm);
                     for (int l = 0; l < NFP; ++l) out[ucol(l % N1, l / N1, jn) * BS] += taun * mf[lam * NFP + l];

@@ -64,3 +64,14 @@ def test_interior_block_adds_volume_and_face_parts_in_fp64(contract, d):
     f = contract(d, p, True, 0 * vol, face, tau, dt, 0.0)[0]
     assert np.abs(f).max() > 0 and np.abs(v).max() > 0
     assert (np.abs(both - (v + f)) <= 2.0 ** -51 * (np.abs(v) + np.abs(f))).all()
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_tau_weighted_face_mass_is_rounded_once(contract, d):
+    """State-dependent tau: without flux coefficients the trace rows hold |n| sum_s w tau mu mu, summed in FP64 and
+    rounded to FP32 once (2^-24); a sum in FP32 has (p + 2)^(d - 1) roundings."""
+    vol, face, tau = coefficients(d, 2, d)
+    ref = contract(d, 2, False, 0 * vol, 0 * face, tau, 0.37, 0.0)[2]
+    got = contract(d, 2, True, 0 * vol, 0 * face, tau, 0.37, 0.0)[2]
+    assert np.abs(ref).max() > 0
+    assert (np.abs(got - ref) <= (2.0 ** -24 + 1e-14) * np.abs(ref)).all()
