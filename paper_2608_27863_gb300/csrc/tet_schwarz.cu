@@ -177,7 +177,8 @@ template <> struct Vec16<float> { using V = float4; };
 template <> struct Vec16<double> { using V = double2; };
 
 // sum over k in [k0, k1) of row[k] y[k] by the four threads of a row (q = 0..3), k0 a multiple of 32;
-// the loads of up to eight groups of 16 bytes per thread go out together
+// the loads of up to eight groups of 16 bytes per thread go out together, and the groups' sums are
+// added as a tree: as few roundings in a row as with a warp per row
 template <class T>
 __device__ __forceinline__ T asm_row_dot(const T* row, const T* y, int k0, int k1, int q) {
     using V = typename Vec16<T>::V;
@@ -185,18 +186,21 @@ __device__ __forceinline__ T asm_row_dot(const T* row, const T* y, int k0, int k
     T s = T(0);
     for (int k = k0 + q * VW; k < k1; k += 4 * VW * U) {
         V v[U];
+        T p[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (k + 4 * VW * u < k1) v[u] = __ldcs(reinterpret_cast<const V*>(row + k + 4 * VW * u));
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const T* x = reinterpret_cast<const T*>(&v[u]);
+            p[u] = T(0);
 #pragma unroll
             for (int w = 0; w < VW; ++w) {
                 const int kk = k + 4 * VW * u + w;
-                if (kk < k1) s = fma(x[w], y[kk], s);
+                if (kk < k1) p[u] = fma(x[w], y[kk], p[u]);
             }
         }
+        s += ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
     }
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);

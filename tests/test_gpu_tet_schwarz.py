@@ -117,3 +117,72 @@ def test_tet_newton_schwarz_reaches_oracle_state(H):
         assert np.linalg.norm(UH.cpu().numpy() - oUH) < 1e-9 * np.linalg.norm(oUH)
     finally:
         H.hdg_destroy(h)
+
+
+def patch_solve_fp32(S, b):
+    """S_r^{-1} b_r of every patch in FP32 (S [E][t][t], b [E][t][n]): LU with partial pivoting, then substitutions
+    whose row sums are 32 interleaved chains joined by a tree, the shortest chains a warp's lanes give."""
+    f = np.float32
+    fma = lambda a, x, c: (a.astype(float) * x + c).astype(f)          # one rounding
+    A, y = S.astype(f), b.astype(f)
+    E, t, _ = A.shape
+    e = np.arange(E)
+    for k in range(t):
+        p = k + np.abs(A[:, k:, k]).argmax(1)
+        A[e, p], A[:, k] = A[:, k].copy(), A[e, p]
+        y[e, p], y[:, k] = y[:, k].copy(), y[e, p]
+        A[:, k + 1:, k] *= (f(1) / A[:, k, k])[:, None]
+        A[:, k + 1:, k + 1:] = fma(-A[:, k + 1:, k, None], A[:, k, None, k + 1:], A[:, k + 1:, k + 1:])
+
+    def dot(row, x):                                                    # [E][c], [E][c][n]
+        acc = np.zeros((E, 32, x.shape[2]), f)
+        for c in range(0, row.shape[1], 32):
+            w = min(32, row.shape[1] - c)
+            acc[:, :w] = fma(row[:, c:c + w, None], x[:, c:c + w], acc[:, :w])
+        for o in (16, 8, 4, 2, 1):
+            acc = acc[:, :o] + acc[:, o:2 * o]
+        return acc[:, 0]
+
+    for i in range(t):
+        y[:, i] -= dot(A[:, i, :i], y[:, :i])
+    for i in range(t - 1, -1, -1):
+        y[:, i] = (y[:, i] - dot(A[:, i, i + 1:], y[:, i + 1:])) / A[:, i, i, None]
+    return y
+
+
+def test_tet_schwarz_fp32_error_on_badly_conditioned_patches(H):
+    """FP32 patch solves of a long time step on an anisotropic wall layer (condition 4e4, t = 300) against 64 bits: over
+    the faces' geometric mean no further off than an FP32 substitution with the shortest chains of roundings.  A sum
+    of random roundings grows by the root of its chains' length, so row sums in four chains miss by 1.16 times as much."""
+    import synth.tetmesh as tm
+    from tests.test_gpu_tet import setup
+    c = [np.linspace(0, 1, 4), np.cumsum([0.0, 1e-3, 1.2e-3]), np.linspace(0, 0.6, 4)]
+    mesh = tm.kuhn_box((3, 2, 3), c, (True, False, True), tags={(1, 0): 4, (1, 1): 1}, degrees=4,
+                       bump=tm.wall_bump(0.05), curved_layers=2, seed=6)
+    prob, pb, h, dev = setup(H, mesh)
+    try:
+        H.hdg_set_params(h, tau=prob.tau, precision=H.HDG_PREC_MIXED)
+        H.hdg_linearize_condense(h, dev["U"], dev["Q"], dev["UH"], dev["Ustar"], None, 100 * prob.dt, prob.a_ii)
+        H.hdg_schwarz_setup(h)
+        assert H.hdg_status(h) == H.HDG_OK
+        s = H.hdg_tet_query(h)
+        vals = torch.zeros(s["n_vals"], dtype=torch.float32, device="cuda")
+        H.hdg_get_blocks(h, vals)
+        S, L = dense_operator(H, h, vals.double().cpu().numpy())
+        idx = np.array([np.concatenate([np.arange(L["hoff"][F], L["hoff"][F + 1]) for F in fs]) for fs in L["e2f"]])
+        Sr = S[idx[:, :, None], idx[:, None, :]]
+        X = np.random.default_rng(0).normal(size=(s["n_trace"], 6))
+        got = np.empty_like(X)
+        for i in range(X.shape[1]):
+            x = torch.from_numpy(np.ascontiguousarray(X[:, i])).cuda()
+            y = torch.empty_like(x)
+            H.hdg_schwarz_apply(h, x, y)
+            got[:, i] = y.cpu().numpy()
+        ref, sub = np.zeros_like(X), np.zeros_like(X)
+        np.add.at(ref, idx, np.linalg.solve(Sr, X[idx]))
+        np.add.at(sub, idx, patch_solve_fp32(Sr, X[idx]).astype(float))
+        err, bar = (np.add.reduceat((v - ref) ** 2, L["hoff"][:-1], axis=0) for v in (got, sub))   # [face][vector], squared
+        ratio = np.exp(0.5 * np.mean(np.log(err / bar)))
+        assert ratio < 1.05, ratio
+    finally:
+        H.hdg_destroy(h)
