@@ -379,3 +379,28 @@ def test_tet_contraction_one_degree_all_boundary_kinds(H, p):
         assert errs.max() < TOL, errs.max()
     finally:
         H.hdg_destroy(h)
+
+
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_tet_mixed_schur_product_truncation(H, p):
+    """Blocks of the mixed form against the FP64 form on an anisotropic wall layer, where the Schur product is larger than
+    its difference with D.  Every 8 terms added to a tensor-core accumulator truncate it, 2^-24 of it on average and always
+    towards zero: n_u / 8 times when it takes the leading products alone, three times as often when it takes the cross
+    products too.  |W Z| and the FP32 roundings of W and Z make 2.1 of the first sum here, 3.4 and more of the second."""
+    c = [np.linspace(0, 1, 4), np.cumsum([0.0, 1e-3, 1.2e-3]), np.linspace(0, 0.6, 4)]
+    mesh = tm.kuhn_box((3, 2, 3), c, (True, False, True), tags={(1, 0): 4, (1, 1): 1}, degrees=p,
+                       bump=tm.wall_bump(0.05), curved_layers=2, seed=6)
+    prob, pb, h, dev = setup(H, mesh)
+    try:
+        vals = []
+        for prec, dtype in ((H.HDG_PREC_FP64, torch.float64), (H.HDG_PREC_MIXED, torch.float32)):
+            H.hdg_set_params(h, tau=prob.tau, precision=prec)
+            H.hdg_linearize_condense(h, dev["U"], dev["Q"], dev["UH"], dev["Ustar"], None, prob.dt, prob.a_ii)
+            assert H.hdg_status(h) == H.HDG_OK
+            v = torch.zeros(H.hdg_tet_query(h)["n_vals"], dtype=dtype, device="cuda")
+            H.hdg_get_blocks(h, v)
+            vals.append(v.double())
+        n_u = 5 * (p + 1) * (p + 2) * (p + 3) // 6
+        assert (vals[1] - vals[0]).norm() <= 2.7 * n_u / 8 * 2.0 ** -24 * vals[0].norm()
+    finally:
+        H.hdg_destroy(h)
