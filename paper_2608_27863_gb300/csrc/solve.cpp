@@ -160,10 +160,12 @@ int ensure_krylov_workspace(hdg_ctx* h, int m) {
     int rc;
     if ((rc = alloc(h, (void**)&h->d_V, sizeof(double) * (size_t)(m + 1) * N))) return rc;
     if ((rc = alloc(h, (void**)&h->d_w, sizeof(double) * N))) return rc;
-    if (!h->d_red) {
-        if ((rc = alloc(h, (void**)&h->d_red, sizeof(double) * kRedBlocks))) return rc;
-        if ((rc = alloc(h, (void**)&h->d_ticket, sizeof(unsigned)))) return rc;
-        CKS(cudaMemsetAsync(h->d_ticket, 0, sizeof(unsigned), h->stream));
+    if (!h->d_red && (rc = alloc(h, (void**)&h->d_red, sizeof(double) * kRedBlocks))) return rc;
+    if (!h->d_ticket) {
+        unsigned* ticket = nullptr;
+        if ((rc = alloc(h, (void**)&ticket, sizeof(unsigned)))) return rc;
+        CKS(cudaMemsetAsync(ticket, 0, sizeof(unsigned), h->stream));
+        h->d_ticket = ticket;                               // the handle's only once it is cleared
     }
     if ((rc = alloc(h, (void**)&h->d_mred, sizeof(double) * kOrthBlocks * (m + 1)))) return rc;
     if ((rc = alloc(h, (void**)&h->d_h, sizeof(double) * 2 * (m + 2)))) return rc;
