@@ -167,6 +167,7 @@ int ensure_krylov_workspace(hdg_ctx* h, int m) {
         CKS(cudaMemsetAsync(ticket, 0, sizeof(unsigned), h->stream));
         h->d_ticket = ticket;                               // the handle's only once it is cleared
     }
+    CKS(orthogonalise_init());
     if ((rc = alloc(h, (void**)&h->d_mred, sizeof(double) * kOrthBlocks * (m + 1)))) return rc;
     if ((rc = alloc(h, (void**)&h->d_h, sizeof(double) * 2 * (m + 2)))) return rc;
     h->gm_cap = m;

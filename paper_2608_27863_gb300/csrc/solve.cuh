@@ -383,6 +383,9 @@ __global__ void k_axpy_dev(const double* coef, double sign, const double* x, dou
 // rotated right-hand side gv (R == NULL: no step)
 struct Givens { const double* col; double* R; double* cs; double* sn; double* gv; int m; };
 constexpr int kOrthBlocks = 152;  // one per SM
+// Allows the Gram-Schmidt kernels the shared memory of the longest basis.  The limit belongs to the function, not to a
+// handle, so that it is one value for all of them; before the first orthogonalise on a device.
+cudaError_t orthogonalise_init();
 // Classical Gram-Schmidt with one reorthogonalisation (CGS2) of w against V_0 .. V_{k-1} (length n each):
 // hcol[0..k-1] the projection coefficients, hcol[k] = ||w|| afterwards, w orthogonalised in place (not scaled).
 // htmp [k], part [k][kOrthBlocks], ticket one zeroed word.

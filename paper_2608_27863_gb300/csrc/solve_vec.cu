@@ -218,6 +218,12 @@ __global__ void __launch_bounds__(NTHR) k_orth(const double* __restrict__ V, int
     }
 }
 
+cudaError_t orthogonalise_init() {
+    constexpr int sm = (int)sizeof(double) * kMaxBasis * 16;
+    const cudaError_t e = cudaFuncSetAttribute(k_orth<0, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_orth<1, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+}
+
 void orthogonalise(cudaStream_t st, const double* V, int64_t n, int k, double* w, double* hcol, double* htmp,
                    double* part, unsigned* ticket, const Givens& G) {
     // one block per SM; narrow blocks while they alone do not reach every SM
@@ -231,10 +237,6 @@ void orthogonalise(cudaStream_t st, const double* V, int64_t n, int k, double* w
     } else {
         const unsigned nb = (unsigned)std::min<int64_t>(kOrthBlocks, (n + 511) / 512);
         const size_t sm = sizeof(double) * k * 16;
-        if (sm > 40 * 1024) {                           // k > 320 of at most 501
-            cudaFuncSetAttribute(k_orth<0, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            cudaFuncSetAttribute(k_orth<1, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        }
         k_orth<0, 512><<<nb, 512, sm, st>>>(V, n, k, w, n, nullptr, part, ticket, hcol, nullptr, none);
         k_orth<1, 512><<<nb, 512, sm, st>>>(V, n, k, w, n, hcol, part, ticket, htmp, hcol, none);
         k_orth<2, 512><<<nb, 512, 0, st>>>(V, n, k, w, n, htmp, part, ticket, hcol + k, nullptr, G);
