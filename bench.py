@@ -783,9 +783,7 @@ def run_ours(args, rank, world, local_rank):
         # the project's autotuner picks among equivalent kernel variants on these inputs (untimed)
         if args.no_autotune or args.elim_nb or args.tuning:
             if args.elim_nb or args.tuning:      # a fixed variant (profiling runs)
-                kw = dict(elim_nb=args.elim_nb or 16, elim_minb=2,
-                          schur_mode=0 if fp64 else {"fp32": 0, "tf32": 1, "3xtf32": 2}[args.mixed_prec],
-                          blocks_mode=1 if m.dim == 3 else 0, elim_mixed_minb=2, blocks64_mode=1)
+                kw = dict(elim_nb=args.elim_nb) if args.elim_nb else {}     # the rest stays as the handle has it
                 # "--tuning k=v,..." sets both legs; "fp64.k=v" / "mixed.k=v" one leg
                 for item in (args.tuning or "").split(","):
                     if item:
@@ -794,7 +792,7 @@ def run_ours(args, rank, world, local_rank):
                         if not leg or leg == ("fp64" if fp64 else "mixed"):
                             kw[key] = int(v)
                 H.hdg_set_tuning(h, **kw)
-                return dict(kw, fixed=True)
+                return dict(H.hdg_get_tuning(h), fixed=True)
             return None
         rep = H.hdg_autotune(h, U, Q, UH, Us, nu, P.dt, P.a_ii, reps=1)
         return {k: rep[k] for k in ("elim_nb", "elim_minb", "schur_mode", "blocks_mode", "elim_mixed_minb",

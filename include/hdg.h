@@ -385,6 +385,9 @@ typedef struct {
 int hdg_autotune(hdg_handle h, const double* U, const double* Q, const double* UH, const double* Ustar,
                  const double* nu, double dt, double a_ii, int reps, hdg_tune* out);
 int hdg_set_tuning(hdg_handle h, const hdg_tune* t);
+/* The variant the handle uses at its precision: the defaults, the autotuner's choice or the last
+ * hdg_set_tuning.  Fills the first seven fields (tetrahedral handles: elim_nb) and clears the rest. */
+int hdg_get_tuning(hdg_handle h, hdg_tune* t);
 
 /* Per-kernel timing with CUDA events recorded on the handle's stream around
  * every kernel launch (not from the paper: instrumentation for rooflines).

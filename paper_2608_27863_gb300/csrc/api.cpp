@@ -457,6 +457,23 @@ int hdg_autotune(hdg_handle h, const double* U, const double* Q, const double* U
     return HDG_OK;
 }
 
+int hdg_get_tuning(hdg_handle h, hdg_tune* t) {
+    if (!h || !t) return fail(h, HDG_EINVAL, "NULL argument");
+    std::memset(t, 0, sizeof(*t));
+    if (h->tet) {
+        t->elim_nb = h->tet->nb;
+        return HDG_OK;
+    }
+    t->elim_nb = h->elim_nb;
+    t->elim_minb = h->elim_minb;
+    t->schur_mode = h->precision == HDG_PREC_FP64 ? (h->schur64_mode ? 3 : 0) : h->schur_mode;
+    t->blocks_mode = h->blocks_mode;
+    t->elim_mixed_minb = h->elim_mixed_minb;
+    t->blocks64_mode = h->blocks64_mode;
+    t->elim_mixed_split = h->elim_mixed_split;
+    return HDG_OK;
+}
+
 int hdg_set_tuning(hdg_handle h, const hdg_tune* t) {
     if (h && h->tet) {
         if (!t || (t->elim_nb != 16 && t->elim_nb != 8)) return fail(h, HDG_EINVAL, "elim_nb must be 16 or 8");

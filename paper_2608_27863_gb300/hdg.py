@@ -39,8 +39,8 @@ EXPORTS = [
     "hdg_blockjacobi_setup", "hdg_blockjacobi_apply", "hdg_gmres", "hdg_newton", "hdg_set_bc_state",
     "hdg_newton_fixed", "hdg_dirk_step", "hdg_lift_gradient", "hdg_set_preconditioner", "hdg_schwarz_setup",
     "hdg_schwarz_apply", "hdg_rb_setup", "hdg_rb_push", "hdg_rb_guess", "hdg_av_field", "hdg_tgv_diagnostics",
-    "hdg_autotune", "hdg_set_tuning", "hdg_set_bc_field", "hdg_reserve", "hdg_create_tet", "hdg_create_tet_host",
-    "hdg_tet_query", "hdg_tet_layout", "hdg_tet_ref_tables", "hdg_tri_ref_tables", "hdg_partition",
+    "hdg_autotune", "hdg_set_tuning", "hdg_get_tuning", "hdg_set_bc_field", "hdg_reserve", "hdg_create_tet",
+    "hdg_create_tet_host", "hdg_tet_query", "hdg_tet_layout", "hdg_tet_ref_tables", "hdg_tri_ref_tables", "hdg_partition",
     "hdg_part_layout", "hdg_sdirk3_tableau", "hdg_measure_peaks", "hdg_set_element_block_output",
 ]
 KERNEL_CLASSES = ["point", "blocks", "elim", "assemble", "matvec", "recover", "schur"]
@@ -129,6 +129,7 @@ def lib():
         "hdg_rb_setup": [vp, i32],
         "hdg_autotune": [vp, vp, vp, vp, vp, vp, dbl, dbl, i32, vp],
         "hdg_set_tuning": [vp, vp],
+        "hdg_get_tuning": [vp, vp],
         "hdg_set_bc_field": [vp, vp],
         "hdg_reserve": [vp, i32],
         "hdg_av_field": [vp, vp, vp, dbl, dbl, dbl, vp],
@@ -447,11 +448,25 @@ def hdg_autotune(h, U, Q, UH, Ustar, nu, dt, a_ii, reps=2):
             "candidates": [(tuple(t.cand[i]), t.ms[i]) for i in range(t.n_cand)]}
 
 
-def hdg_set_tuning(h, elim_nb=16, elim_minb=2, schur_mode=0, blocks_mode=1, elim_mixed_minb=2, blocks64_mode=1,
-                   elim_mixed_split=0):
+_TUNING = ("elim_nb", "elim_minb", "schur_mode", "blocks_mode", "elim_mixed_minb", "blocks64_mode", "elim_mixed_split")
+
+
+def hdg_get_tuning(h):
+    """The kernel variant the handle uses at its precision, as a dict of hdg_set_tuning's arguments."""
     t = hdg_tune()
-    t.elim_nb, t.elim_minb, t.schur_mode, t.blocks_mode = elim_nb, elim_minb, schur_mode, blocks_mode
-    t.elim_mixed_minb, t.blocks64_mode, t.elim_mixed_split = elim_mixed_minb, blocks64_mode, elim_mixed_split
+    _check(h, lib().hdg_get_tuning(h, ctypes.byref(t)))
+    return {n: getattr(t, n) for n in _TUNING}
+
+
+def hdg_set_tuning(h, elim_nb=None, elim_minb=None, schur_mode=None, blocks_mode=None, elim_mixed_minb=None,
+                   blocks64_mode=None, elim_mixed_split=None):
+    """Choose kernel variants; what is not given stays as the handle has it."""
+    t = hdg_tune()
+    _check(h, lib().hdg_get_tuning(h, ctypes.byref(t)))
+    given = (elim_nb, elim_minb, schur_mode, blocks_mode, elim_mixed_minb, blocks64_mode, elim_mixed_split)
+    for name, value in zip(_TUNING, given):
+        if value is not None:
+            setattr(t, name, value)
     _check(h, lib().hdg_set_tuning(h, ctypes.byref(t)))
 
 

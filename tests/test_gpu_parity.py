@@ -226,6 +226,26 @@ def test_autotuned_variants_keep_parity():
         compare_handle.close()
 
 
+@pytest.mark.parametrize("precision", ["HDG_PREC_FP64", "HDG_PREC_MIXED"])
+def test_tuning_call_without_a_choice_changes_nothing(precision):
+    """hdg_set_tuning leaves a fresh handle's variant where it is: the same bits before and after."""
+    import torch
+    from paper_2608_27863_gb300 import hdg as H
+    P = synth.config2(n=3)
+    run = GpuRun(P)
+    H.hdg_set_params(run.h, tau=P.tau, precision=getattr(H, precision))
+    out = []
+    for _ in range(2):
+        run.linearize()
+        v = torch.empty(run.sizes["nnzb"] * run.sizes["block"] ** 2, device="cuda",
+                        dtype=torch.float64 if precision == "HDG_PREC_FP64" else torch.float32)
+        H.hdg_get_blocks(run.h, v)
+        out.append((v.cpu().numpy(), run.rhs()))
+        H.hdg_set_tuning(run.h)
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
+    run.close()
+
+
 def tagged(P, side_tags, twall=1.0):
     bt = P.mesh.bnd_tag.copy()
     for (r, s), t in side_tags.items():

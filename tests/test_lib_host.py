@@ -176,3 +176,21 @@ def test_sdirk3_tableau_from_the_library(H):
     assert np.array_equal(b, A[-1])
     c = A.sum(1)
     assert abs(b @ c ** 2 - 1 / 3) < 1e-14 and abs(b @ A @ c - 1 / 6) < 1e-14
+
+
+def test_set_tuning_keeps_what_is_not_given(H):
+    mesh = synth.box_mesh(3, (3, 3, 3), (0,) * 3, (1.0,) * 3, (True,) * 3)
+    h = H.hdg_create_host(3, mesh.vert_xyz, mesh.elem_vert, mesh.periodic_map, None, 2, 1.4, 100.0, 0.72, 0.3)
+    fresh = H.hdg_get_tuning(h)
+    H.hdg_set_tuning(h)
+    assert H.hdg_get_tuning(h) == fresh
+    for precision, schur in ((H.HDG_PREC_FP64, 3), (H.HDG_PREC_MIXED, 2)):
+        H.hdg_set_params(h, precision=precision)
+        H.hdg_set_tuning(h, elim_minb=1, schur_mode=schur)
+        before = H.hdg_get_tuning(h)
+        H.hdg_set_tuning(h, elim_nb=8)
+        assert H.hdg_get_tuning(h) == dict(before, elim_nb=8, elim_minb=1, schur_mode=schur)
+    H.hdg_set_params(h, precision=H.HDG_PREC_MIXED_TF32)         # a Schur precision fixed by the caller stays
+    H.hdg_set_tuning(h, elim_nb=16)
+    assert H.hdg_get_tuning(h)["schur_mode"] == 1
+    H.hdg_destroy(h)
