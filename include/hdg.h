@@ -362,12 +362,14 @@ int hdg_sdirk3_tableau(double* A, double* b);
  *    tuning call a handle uses panel width 8, and schur_mode 3 for n_u >= 40
  *    (hexes, quads of degree 3);
  *  - mixed form: the elimination as one fused kernel (at 2 or 3 CTAs per
- *    SM) or split into an FP64 LU (panel width 16 or 8) and two FP32
- *    triangular solves (the default), and, when requested as HDG_PREC_MIXED,
+ *    SM) or split into an FP64 LU (in shared memory; for hexes of degree 3 in
+ *    panels of 16 or 8 columns) and two FP32 triangular solves (the default),
+ *    and, when requested as HDG_PREC_MIXED,
  *    the Schur product as FP32 SIMT (schur_mode 0) or 3xTF32 tensor cores
  *    (2) — all FP32-accurate; TF32 / 3xTF32 requested explicitly are kept;
  *  - blocks64_mode (0, 1) and blocks_mode (0..2) are accepted and reported but
- *    select nothing any more: every value runs the one contraction kernel;
+ *    select nothing any more: every value runs the one contraction kernel, and
+ *    the autotuner leaves them as they are;
  *  - tetrahedral handles: the elimination panel width (16 or 8 columns) of
  *    the persistent linearize + condense kernel (elim_nb; the other fields
  *    are zero; hdg_set_tuning reads elim_nb only).

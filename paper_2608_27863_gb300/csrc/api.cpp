@@ -368,39 +368,34 @@ int hdg_autotune(hdg_handle h, const double* U, const double* Q, const double* U
     if (!h) return HDG_EINVAL;
     if (!h->device) return fail(h, HDG_EINVAL, "handle has no device storage");
     if (reps < 1 || reps > 100) return fail(h, HDG_EINVAL, "reps must be in 1..100");
-    // candidates: variants that compute the same quantities to the same accuracy
+    // candidates: variants that compute the same quantities to the same accuracy by different kernels; blocks_mode and
+    // blocks64_mode select nothing, so that every candidate carries the handle's
     int cand[16][7];
     int n = 0;
+    auto add = [&](int nb, int minb, int sm, int mminb, int split) {
+        const int c[7] = {nb, minb, sm, h->blocks_mode, mminb, h->blocks64_mode, split};
+        std::copy(c, c + 7, cand[n++]);
+    };
     if (h->precision == HDG_PREC_FP64) {
         // Schur product in the FP64 elimination (schur_mode 0) or on the tensor cores by exact
         // digit splitting (3); both FP64-accurate
-        const int nbs[2] = {16, 8}, minbs[2] = {2, 1};
         for (int sm : {0, 3})
-            for (int bm64 : {1, 0})
-                for (int a = 0; a < 2; ++a)
-                    for (int b = 0; b < 2; ++b) {
-                        cand[n][0] = nbs[a]; cand[n][1] = minbs[b]; cand[n][2] = sm; cand[n][3] = h->blocks_mode;
-                        cand[n][4] = h->elim_mixed_minb; cand[n][5] = bm64; cand[n][6] = h->elim_mixed_split; ++n;
-                    }
+            for (int nb : {16, 8})
+                for (int minb : {2, 1}) add(nb, minb, sm, h->elim_mixed_minb, h->elim_mixed_split);
     } else {
         // FP32 SIMT and 3xTF32 tensor-core Schur products are both FP32-accurate, unless TF32 /
-        // 3xTF32 was requested explicitly; the values of blocks_mode run the same kernel
+        // 3xTF32 was requested explicitly
         const bool free_schur = h->prec_req == HDG_PREC_MIXED;
         for (int sm : {0, 2}) {
             if (!free_schur && sm != 0) continue;
-            for (int bm : {1, 2, 0}) {
-                if (bm == 1 && h->d != 3) continue;
-                if (bm == 0 && free_schur) continue;
-                // elimination: split with the interior LU at panel width 16 or 8 (ev 16, 8), or
-                // fused at 2 or 3 CTAs per SM (ev 2, 3)
-                for (int ev : {16, 8, 2, 3}) {
-                    const bool split = ev >= 8;
-                    cand[n][0] = split ? ev : h->elim_nb; cand[n][1] = h->elim_minb;
-                    cand[n][2] = free_schur ? sm : h->schur_mode;
-                    cand[n][3] = bm; cand[n][4] = split ? h->elim_mixed_minb : ev; cand[n][5] = h->blocks64_mode;
-                    cand[n][6] = split ? 1 : 0; ++n;
-                }
+            const int mode = free_schur ? sm : h->schur_mode;
+            // split elimination: the LU in shared memory has one variant, the one in panels two
+            if (hdg::lu_in_shared_memory(h->NU)) {
+                add(h->elim_nb, h->elim_minb, mode, h->elim_mixed_minb, 1);
+            } else {
+                for (int nb : {16, 8}) add(nb, h->elim_minb, mode, h->elim_mixed_minb, 1);
             }
+            for (int mminb : {2, 3}) add(h->elim_nb, h->elim_minb, mode, mminb, 0);   // fused, at 2 or 3 CTAs per SM
         }
     }
     cudaEvent_t ev[2];

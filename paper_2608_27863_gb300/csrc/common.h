@@ -69,6 +69,11 @@ struct Phys {
     int tau_mode = 0;     // 0: constant tau; 1: state-dependent tau(uhat) = |v.n| + c + mu / h
 };
 
+// the mixed form's interior LU runs in shared memory: [n_u][n_u + 1 to odd] and a column of multipliers in at most 200 KB
+constexpr int lu_row_stride(int n_u) { return (n_u + 1) | 1; }
+constexpr int lu_smem_bytes(int n_u) { return (n_u * lu_row_stride(n_u) + n_u) * 8; }
+constexpr bool lu_in_shared_memory(int n_u) { return lu_smem_bytes(n_u) <= 200 * 1024; }
+
 // row stride of the mixed form's FP32 blocks: rows start on 16 bytes
 inline int64_t mixed_stride(int64_t n) { return (n + 3) / 4 * 4; }
 

@@ -407,10 +407,10 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
 template <class C>
 struct LuShape {
     static constexpr int NU = C::NU;
-    static constexpr int LDS = (NU + 1) | 1;             // odd row stride in doubles: columns without bank conflicts
+    static constexpr int LDS = lu_row_stride(NU);        // odd, in doubles: columns without bank conflicts
     static constexpr int NTH = NU > 100 ? 512 : NU > 50 ? 128 : 64;
-    static constexpr int smem_bytes = (NU * LDS + NU) * 8;
-    static constexpr bool fits = smem_bytes <= 200 * 1024;
+    static constexpr int smem_bytes = lu_smem_bytes(NU);
+    static constexpr bool fits = lu_in_shared_memory(NU);
 };
 
 template <class C>

@@ -1,5 +1,5 @@
 """The contraction kernel on one element with coefficients given here, its FP32
-instance against sums that the mixed form holds in FP64."""
+instance against the FP64 one and against sums that the mixed form holds in FP64."""
 import ctypes
 import os
 import subprocess
@@ -75,3 +75,14 @@ def test_tau_weighted_face_mass_is_rounded_once(contract, d):
     got = contract(d, 2, True, 0 * vol, 0 * face, tau, 0.37, 0.0)[2]
     assert np.abs(ref).max() > 0
     assert (np.abs(got - ref) <= (2.0 ** -24 + 1e-14) * np.abs(ref)).all()
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_fp32_blocks_follow_fp64_before_elimination(contract, d):
+    """All four blocks of the FP32 instance against the FP64 one.  An entry passes through about 20 sums, one axis at a
+    time and then dt times the face rows, of terms of random sign: 20^(1/2) 2^-24 = 2.7e-7 of its size, four times
+    which is the bar (half precision would miss it by 2^13)."""
+    args = coefficients(d, 2, 10 + d) + (0.37, 2.5)
+    ref, got = contract(d, 2, False, *args), contract(d, 2, True, *args)
+    for a, b in zip(ref, got):
+        assert np.linalg.norm(b - a) <= 1.1e-6 * np.linalg.norm(a)

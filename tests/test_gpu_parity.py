@@ -205,10 +205,10 @@ def test_autotuned_variants_keep_parity():
     run = GpuRun(P)
     rep = H.hdg_autotune(run.h, run.U, run.Q, run.UH, run.Ustar, run.nu, P.dt, P.a_ii, reps=1)
     cands = rep["candidates"]
-    assert len(cands) == 16 and all(ms > 0 for _, ms in cands)
-    chosen = (rep["elim_nb"], rep["elim_minb"], rep["schur_mode"], rep["blocks64_mode"])
-    assert min(ms for _, ms in cands) == [ms for c, ms in cands if (c[0], c[1], c[2], c[5]) == chosen][0]
-    assert {c[5] for c, _ in cands} == {0, 1}      # dense and sum-factorised contraction
+    assert len(cands) == 8 and all(ms > 0 for _, ms in cands)
+    assert len({c[:3] for c, _ in cands}) == 8      # each a kernel of its own: panel width, residency, Schur product
+    chosen = (rep["elim_nb"], rep["elim_minb"], rep["schur_mode"])
+    assert min(ms for _, ms in cands) == [ms for c, ms in cands if c[:3] == chosen][0]
     assert {c[2] for c, _ in cands} == {0, 3}      # Schur product on the FP64 pipe / the tensor cores
     run.close()
     for cand, _ms in cands:
