@@ -91,8 +91,9 @@ __device__ void givens_column(double* col, const double* c, const double* s, int
 // follows for the sums: an orthogonalisation with its norm and Givens step is three launches
 // instead of nine, which is what sets the time of small systems (one SDIRK3 step on 64 quads,
 // 1,536 unknowns, 480 GMRES iterations in a graph: 42.3 -> 26.1 ms, with the back substitution by a
-// warp instead of a thread).  Large systems are bound by the FP64 pipe, 2 k n multiply-adds of
-// 629e9 per second (2.7e5 unknowns, k ~ 78: 34 us a pass; MODE 0 62, MODE 1 90, MODE 2 38 us).
+// warp instead of a thread).  Large systems are bound by the FP64 pipe, 629e9 multiply-adds per second:
+// k n of them in MODE 0 and 2, 2 k n in MODE 1 (2.7e5 unknowns, k ~ 78: 34 and 67 us; measured MODE 0
+// 62, MODE 1 90, MODE 2 38 us).
 // Tried for MODE 0: 256 threads with four rows in flight 69 us (MODE 1 116: too few loads in
 // flight for its first part), no barrier between the groups 102 us (the warps drift over all k
 // streams).  part: [k][gridDim.x]; ticket: zero between launches.
@@ -226,10 +227,13 @@ cudaError_t orthogonalise_init() {
 
 void orthogonalise(cudaStream_t st, const double* V, int64_t n, int k, double* w, double* hcol, double* htmp,
                    double* part, unsigned* ticket, const Givens& G) {
-    // one block per SM; narrow blocks while they alone do not reach every SM
+    // One block per SM.  Narrow blocks, which leave no SM idle, up to two rows a thread; wide ones keep more loads in
+    // flight from there on.  A GMRES iteration with bases up to 100, narrow / wide, in us: 2,400 unknowns 89 / 128,
+    // 18,816 105 / 136, 24,576 122 / 140, 38,400 130 / 145, 48,600 149 / 153, 60,000 167 / 161, 101,400 230 / 198;
+    // with bases up to 300 the sides meet between 38,400 (254 / 297) and 48,600 (315 / 306).
     const Givens none{};
-    if (n <= (int64_t)kOrthBlocks * 128) {
-        const unsigned nb = (unsigned)((n + 127) / 128);
+    if (n <= 2 * (int64_t)kOrthBlocks * 128) {
+        const unsigned nb = (unsigned)std::min<int64_t>(kOrthBlocks, (n + 127) / 128);
         const size_t sm = sizeof(double) * k * 4;
         k_orth<0, 128><<<nb, 128, sm, st>>>(V, n, k, w, n, nullptr, part, ticket, hcol, nullptr, none);
         k_orth<1, 128><<<nb, 128, sm, st>>>(V, n, k, w, n, hcol, part, ticket, htmp, hcol, none);
