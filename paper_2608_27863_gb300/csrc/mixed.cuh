@@ -401,14 +401,19 @@ __global__ void __launch_bounds__(NTH, 2) k_lu_mixed(Regions<float> R, int32_t* 
 // that fit (n_u <= 135: every element type but the degree-3 hexes), right-looking one column at
 // a time.  FP64 multiply-adds take 16 cycles of an SM per warp here, so the shared-memory traffic of
 // rank-1 updates is free and no panel is needed; what is left to hide is the pivot chain, and warp 0
-// updates the next column first and searches its pivot while the other warps update the rest.  The trailing block is walked as one flat range, so that no lane idles at
-// the rows' ends.  4,096 hexes p = 2: 10.05 -> 8.7 ms (2/3 n_u^3 at the FP64 pipe's rate: 5.4); 2,867 quads p = 3:
-// 1.65 -> 0.70.
+// updates the next column first and searches its pivot while the other warps update the rest.  The
+// trailing block is walked as one flat range, so that no lane idles at the rows' ends.  4,096 hexes
+// p = 2: 10.05 -> 8.7 ms (2/3 n_u^3 at the FP64 pipe's rate: 5.4); 2,867 quads p = 3: 1.65 -> 0.62.
+// Threads: a wider CTA shortens an element's chain of columns, a narrower one wastes fewer barrier
+// waits when CTAs are many.  LU and triangular solves with 64 / 128 / 256 / 512 threads, in us, on 64
+// elements and on many: n_u = 16 36 33 33 35 and 128 135 144 195 (2,916 quads); 36 92 73 67 68 and 424
+// 406 413 500; 40 109 82 75 75 and 218 198 201 232 (729 hexes); 64 258 141 115 111 and 1337 1045 968
+// 1045; 135 1901 790 506 459 and 7839 3392 2219 2021 (512 hexes).
 template <class C>
 struct LuShape {
     static constexpr int NU = C::NU;
     static constexpr int LDS = lu_row_stride(NU);        // odd, in doubles: columns without bank conflicts
-    static constexpr int NTH = NU > 100 ? 512 : NU > 50 ? 128 : 64;
+    static constexpr int NTH = NU > 100 ? 512 : NU > 50 ? 256 : NU > 20 ? 128 : 64;
     static constexpr int smem_bytes = lu_smem_bytes(NU);
     static constexpr bool fits = lu_in_shared_memory(NU);
 };
