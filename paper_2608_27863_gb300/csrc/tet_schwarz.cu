@@ -177,31 +177,33 @@ template <> struct Vec16<float> { using V = float4; };
 template <> struct Vec16<double> { using V = double2; };
 
 // sum over k in [k0, k1) of row[k] y[k] by the four threads of a row (q = 0..3), k0 a multiple of 32;
-// the loads of up to eight groups of 16 bytes per thread go out together, and the groups' sums are
-// added as a tree: as few roundings in a row as with a warp per row
+// the loads of a thread's U groups of 16 bytes go out together.  As few roundings in a row as with a
+// warp per row: FP32 joins the groups' sums as a tree, FP64, whose additions cost as much as its
+// multiply-adds, keeps one chain per group
 template <class T>
 __device__ __forceinline__ T asm_row_dot(const T* row, const T* y, int k0, int k1, int q) {
     using V = typename Vec16<T>::V;
-    constexpr int VW = 16 / sizeof(T), U = 8;
-    T s = T(0);
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int VW = 16 / sizeof(T), U = F64 ? 4 : 8;
+    T s = T(0), p[U] = {};
     for (int k = k0 + q * VW; k < k1; k += 4 * VW * U) {
         V v[U];
-        T p[U];
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (k + 4 * VW * u < k1) v[u] = __ldcs(reinterpret_cast<const V*>(row + k + 4 * VW * u));
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const T* x = reinterpret_cast<const T*>(&v[u]);
-            p[u] = T(0);
+            if (!F64) p[u] = T(0);
 #pragma unroll
             for (int w = 0; w < VW; ++w) {
                 const int kk = k + 4 * VW * u + w;
                 if (kk < k1) p[u] = fma(x[w], y[kk], p[u]);
             }
         }
-        s += ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
+        if constexpr (!F64) s += ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
     }
+    if constexpr (F64) s = (p[0] + p[1]) + (p[2] + p[3]);
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     return s;
