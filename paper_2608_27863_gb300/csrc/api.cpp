@@ -244,7 +244,11 @@ int create_device(hdg_ctx* h) {
     // rows' words of a 16-wide one; 1-15 % faster on every element type), and the Schur product on the
     // tensor cores from n_u = 40 on.  Elimination + Schur product, in ms, FP64 pipe / tensor cores:
     // 2867 quads p = 1 0.33 / 0.53, p = 2 1.56 / 1.76, p = 3 (n_u = 64) 4.3 / 3.7; 693 hexes p = 1
-    // (n_u = 40) 1.29 / 0.85; 512 hexes p = 2 17.0 / 10.3; 210 hexes p = 3 69.4 / 37.0
+    // (n_u = 40) 1.29 / 0.85; 512 hexes p = 2 17.0 / 10.3; 210 hexes p = 3 69.4 / 37.0.  The sides do not
+    // cross with the element count.  A linearization of 1 / 64 / 2,916 quads or 1 / 64 / 216 hexes, in ms:
+    // quads p = 1 0.14 / 0.14 / 0.84 against 0.16 / 0.16 / 1.06, p = 2 0.21 / 0.21 / 2.54 against 0.22 / 0.23 /
+    // 2.73, p = 3 0.40 / 0.40 / 6.17 against 0.36 / 0.37 / 5.47; hexes p = 1 0.57 / 0.57 / 0.95 against 0.45 /
+    // 0.46 / 0.75, p = 2 5.2 / 5.6 / 10.3 against 2.7 / 3.4 / 6.7, p = 3 37 / 41 / 78 against 18 / 23 / 46
     h->elim_nb = 8;
     h->schur64_mode = h->NU >= 40 ? 1 : 0;
     if (const char* s = std::getenv("HDG_ELIM_MINB")) h->elim_minb = std::atoi(s) == 1 ? 1 : 2;
