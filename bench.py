@@ -42,9 +42,6 @@ METRIC = "HDG linearize+condense elements/s & % of FP64/TC peak; mixed vs FP64 a
 # count of a launch.
 # Keyed by (kernel, d, p, elimination panel width).
 DRAM_BYTES_PER_ELEMENT = {("elim", 3, 2, 16): 16.45e6, ("elim", 3, 2, 8): 30.84e6,
-                          # FP64 element blocks before k_contract: two kernels, 0.377 + 0.936 GB on the
-                          # 512-element 8^3 launch
-                          ("blocks_sf", 3, 2, 0): (0.3775e9 + 0.9359e9) / 512,
                           # k_elim without the Schur product (panels of 8 columns), and k_contract
                           ("elim", 3, 2, 0): 5.008e9 / 512, ("contract", 3, 2, 0): 0.8197e9 / 512}
 # The persistent tetrahedral kernel k_tet_linearize<double>: 55.8 GB (read + write) in one
@@ -452,12 +449,6 @@ def make_problem(name, cpu_sample=False):
 # ----------------------------------------------------------------------------
 # algorithmic FLOP counts per element (the executed reduced-structure counts)
 # ----------------------------------------------------------------------------
-def ozaki_digits(K):
-    """Digit width and count that represent 54 bits of the operands for inner size K."""
-    b = 8 if 5 * K * 255 ** 2 < 2 ** 24 else 7 if 5 * K * 127 ** 2 < 2 ** 24 else 6
-    return b, -(-54 // b)
-
-
 def schur_digits(K):
     """Digit width and count of the tensor-core Schur product: at least 60 bits, over
     eight accumulator groups of at most 7 digit pairs each (5 at width 8)."""
@@ -792,8 +783,7 @@ def run_ours(args, rank, world, local_rank):
                         if not leg or leg == ("fp64" if fp64 else "mixed"):
                             kw[key] = int(v)
                 H.hdg_set_tuning(h, **kw)
-                return dict(H.hdg_get_tuning(h), fixed=True)
-            return None
+            return dict(H.hdg_get_tuning(h), fixed=True)
         rep = H.hdg_autotune(h, U, Q, UH, Us, nu, P.dt, P.a_ii, reps=1)
         return {k: rep[k] for k in ("elim_nb", "elim_minb", "schur_mode", "blocks_mode", "elim_mixed_minb",
                                     "blocks64_mode", "elim_mixed_split")}
@@ -876,7 +866,7 @@ def run_ours(args, rank, world, local_rank):
         def hex_prec(prec):
             set_prec(prec)
             tn = tuning.get("fp64" if prec == H.HDG_PREC_FP64 else "mixed")
-            if tn:
+            if tn:                                  # this leg's choice
                 H.hdg_set_tuning(h, **{k: v for k, v in tn.items() if k != "fixed"})
 
         run1 = lambda: H.hdg_linearize_condense(h, U, Q, UH, Us, nu, P.dt, P.a_ii)
@@ -922,10 +912,10 @@ def run_ours(args, rank, world, local_rank):
             out["cpu_baseline"] = cpu
         H.hdg_destroy(h)
         return out
-    t64 = tuning.get("fp64") or {}
-    oz = t64.get("schur_mode", 0) == 3          # FP64 Schur product on the tensor cores
+    t64 = tuning["fp64"]
+    oz = t64["schur_mode"] == 3          # FP64 Schur product on the tensor cores
     fl = flop_counts(m.dim, P.p, sum_factorised=True, tc_schur=oz)
-    nb_used = t64.get("elim_nb", args.elim_nb or 16)
+    nb_used = t64["elim_nb"]
     kern = {}
     for k, (ms, n) in prof.items():
         if n:

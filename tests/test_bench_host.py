@@ -15,14 +15,14 @@ def test_flop_split_keeps_the_total():
         assert b["schur"] == 2 * NT * NT * NU
 
 
-def test_ozaki_digit_budget():
-    """5 K (2^b - 1)^2 < 2^24 (the groups k <= 6 accumulate exactly in FP32), b s >= 54,
-    and b the largest such width; hex p = 2 and p = 3 take (7, 8) and (6, 9)."""
-    for K in (16, 36, 40, 64, 135, 320):
-        b, s = bench.ozaki_digits(K)
-        assert 5 * K * (2 ** b - 1) ** 2 < 2 ** 24 and b * s >= 54 and b * (s - 1) < 54
-        assert b == 8 or 5 * K * (2 ** (b + 1) - 1) ** 2 >= 2 ** 24
-    assert bench.ozaki_digits(135) == (7, 8) and bench.ozaki_digits(320) == (6, 9)
+def test_digit_budget_of_the_schur_product():
+    """Digits of b bits, the widest for which the exact groups stay exact: (groups) K (2^b - 1)^2 < 2^24 with five of them
+    at b = 8 and seven below; 60 <= b s <= 64 bits in all."""
+    want = {16: (8, 8), 36: (8, 8), 40: (8, 8), 64: (7, 9), 135: (7, 9), 320: (6, 10)}
+    for K, (b, s) in want.items():
+        assert bench.schur_digits(K) == (b, s)
+        assert (5 if b == 8 else 7) * K * (2 ** b - 1) ** 2 < 2 ** 24 and 60 <= b * s <= 64
+        assert b == 8 or (5 if b == 7 else 7) * K * (2 ** (b + 1) - 1) ** 2 >= 2 ** 24
 
 
 def test_recover_bytes_models():
@@ -57,10 +57,11 @@ def test_oracle_check_elements_cover_every_degree():
 
 def test_hex_traffic_table_covers_the_autotuned_dominant_kernels():
     """The hex line's roofline traffic comes from ncu captures per (kernel, dim, p,
-    panel width): the FP64 element-block pair (sum-factorised volume + face terms)
-    and k_elim at both panel widths of hex p = 2; per-element bytes of the right
-    order (the 1.32 MB bordered matrix is read and written at least once)."""
+    panel width): the contraction and k_elim at both panel widths of hex p = 2, and
+    without the Schur product; per-element bytes of the right order (the 1.32 MB
+    bordered matrix is read and written at least once)."""
     t = bench.DRAM_BYTES_PER_ELEMENT
-    for key in (("elim", 3, 2, 16), ("elim", 3, 2, 8), ("blocks_sf", 3, 2, 0)):
+    for key in (("elim", 3, 2, 16), ("elim", 3, 2, 8), ("elim", 3, 2, 0), ("contract", 3, 2, 0)):
         assert key in t and 1e6 < t[key] < 1e8, key
     assert t[("elim", 3, 2, 8)] > t[("elim", 3, 2, 16)]      # narrower panels re-read the trailing matrix more
+    assert t[("elim", 3, 2, 0)] < t[("elim", 3, 2, 8)]       # the trace block is not touched
