@@ -17,10 +17,11 @@
 // Multiply-adds per hex p = 2 element: 2.3e6, where applying one side of the sum factorisation to every
 // column and the dense face products took 5.9e6.  One warp (two for p = 3) per CTA and 1..8 pairs; the
 // rows are collected in shared memory and leave in whole lines.  512 hexes p = 2, FP64: 7.27 -> 3.17 ms
-// (1.9 at the FP64 pipe's rate, which is 74 % active); 693 hexes p = 1 1.81 -> 0.63 ms; mixed form, 4,096 hexes p = 2: 10.1 ->
-// 5.1 ms (3xTF32 tensor-core tiles before, bound by forming their operands), 1,320 hexes p = 3: 10.9 ->
-// 8.0 ms.  The row factors come from the 3-D tables: with products of 1-D ones the FP32 form is 10 %
-// faster (4.7 and 7.2 ms) but its blocks at p = 3 lose a fifth of their accuracy.
+// (1.9 at the FP64 pipe's rate, which is 74 % active); 693 hexes p = 1 1.81 -> 0.63 ms; mixed form, 4,096
+// hexes p = 2: 10.1 -> 5.3 ms (3xTF32 tensor-core tiles before, bound by forming their operands), 1,320 hexes
+// p = 3: 10.9 -> 8.1 ms, of which the interior block's sums in FP64 take 0.1 to 0.2.  The row factors come
+// from the 3-D tables: with products of 1-D ones the FP32 form is 10 % faster but its blocks at p = 3 lose a
+// fifth of their accuracy.
 #pragma once
 
 namespace hdg {

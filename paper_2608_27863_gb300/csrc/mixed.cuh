@@ -254,8 +254,6 @@ __global__ void __launch_bounds__(NTH, MINB) k_elim_mixed(Regions<float> R, int6
     if (tid == 0 && sflag) atomicOr(status, sflag);
 }
 
-// S^K = Dt - W Z (in place over Dt) and Rh <- Rh - W z, FP32 SIMT with FP32
-// accumulation (W [t][n_u] = Ct region, Z [n_u][t] = Bt region after k_elim_mixed)
 // ----------------------------------------------------------------------------
 // A3 + A4 of the mixed form, split by precision.  k_lu_mixed factors the
 // interior block in FP64 alone, P At = L U with partial pivoting (blocked
@@ -662,6 +660,8 @@ __global__ void __launch_bounds__(TrsmShape<C>::NTH) k_trsm(Regions<float> R, co
     }
 }
 
+// S^K = Dt - W Z (in place over Dt) and Rh <- Rh - W z, FP32 SIMT with FP32
+// accumulation (W [t][n_u] = Ct region, Z [n_u][t] = Bt region)
 template <class C, int NTH>
 __global__ void __launch_bounds__(NTH) k_schur_simt(Regions<float> R, int64_t e0) {
     constexpr int NU = C::NU, NT = C::NT, KC = 32, TW = 64;
